@@ -151,3 +151,23 @@ def test_device_built_outage_cases(lu):
         assert st[bi] == sto
         if sto == 0:
             assert np.max(np.abs(v[bi] - Vo)) < 1e-6
+
+
+@pytest.mark.parametrize("B", [1, 17, 2600, 20011])
+def test_branch_flows_every_instance_block(B):
+    """Blocks of one, of two and of 16 instances, the last with a remainder:
+    every instance's flows against the pi model in NumPy, and zero where a
+    branch is out of service."""
+    g = gridgen.make_grid("mesh30_b64")
+    rng = np.random.default_rng(B)
+    V = rng.uniform(0.9, 1.1, (B, g.n)) * np.exp(1j * rng.uniform(-0.5, 0.5, (B, g.n)))
+    ins = rng.random((B, g.n_branch)) < 0.9
+    with _plan(g) as p:
+        sf, st = (a.cpu().numpy() for a in p.branch_flows(_dev(V), torch.from_numpy(ins).cuda()))
+        sa, sb = (a.cpu().numpy() for a in p.branch_flows(_dev(V)))
+    ys, bh = 1.0 / (g.r + 1j * g.x), 0.5j * g.b
+    vf, vt = V[:, g.f], V[:, g.t]
+    of, ot = vf * np.conj(ys * (vf - vt) + bh * vf), vt * np.conj(-ys * (vf - vt) + bh * vt)
+    # |V| <= 1.1, |ys| <= 20: a dozen roundings of values below 50
+    assert np.max(np.abs(sa - of)) < 1e-12 and np.max(np.abs(sb - ot)) < 1e-12
+    assert np.array_equal(sf, np.where(ins, sa, 0)) and np.array_equal(st, np.where(ins, sb, 0))
