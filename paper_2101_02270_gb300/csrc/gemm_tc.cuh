@@ -43,10 +43,11 @@ __device__ __forceinline__ uint64_t make_sdesc(uint32_t saddr, uint32_t lbo, uin
   return d;  // base offset 0, relative LBO, layout type 0 (no swizzle)
 }
 
-// Instruction descriptor, kind::f16: FP32 accumulator, BF16 A and B, both
-// K-major, N >> 3 at bit 17, M >> 4 at bit 24.
-__host__ __device__ constexpr uint32_t make_idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// Instruction descriptor, kind::f16: FP32 accumulator, BF16 A and B, each
+// K-major or (bits 15, 16) MN-major, N >> 3 at bit 17, M >> 4 at bit 24.
+__host__ __device__ constexpr uint32_t make_idesc_bf16(int M, int N, bool a_mn = false, bool b_mn = false) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
+         ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
@@ -117,8 +118,37 @@ __device__ __forceinline__ void load_tile_kmajor(uint8_t* s, const __nv_bfloat16
   }
 }
 
-// Epilogue functor interface: op(row, col, value) for one C element.
+// The same layout from a [64 x rows] tile stored with the rows contiguous (row
+// stride ld elements between consecutive k).
+template <int ROWS>
+__device__ __forceinline__ void load_tile_mnmajor(uint8_t* s, const __nv_bfloat16* __restrict__ g, int64_t ld,
+                                                  int tid) {
+  constexpr int chunks = ROWS * 8;
+#pragma unroll 4
+  for (int c = tid; c < chunks; c += kGemmThreads) {
+    const int r = c % ROWS, k8 = c / ROWS;
+    __align__(16) __nv_bfloat16 v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = g[(int64_t)(k8 * 8 + j) * ld + r];
+    *reinterpret_cast<uint4*>(s + (r >> 3) * 1024 + k8 * 128 + (r & 7) * 16) = *reinterpret_cast<const uint4*>(v);
+  }
+}
+
+// Epilogue functor interface: op(row, col, value) for one C element.  With
+// Epi::kSum it returns a summand: a warp adds its summands in FP32 per lane and
+// FP64 beyond, into *epi.sum.
 template <class Epi>
+__device__ __forceinline__ void epi_sum(const Epi& epi, float part) {
+  if constexpr (Epi::kSum) {
+    double d = (double)part;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(epi.sum, d);
+  }
+}
+
+// AT (BT): A is stored [K][M] (B is stored [K][N]) instead of K-contiguous.
+template <class Epi, bool AT, bool BT>
 __global__ void __launch_bounds__(kGemmThreads) k_gemm_tc(const __nv_bfloat16* __restrict__ A,
                                                           const __nv_bfloat16* __restrict__ B, int M, int N, int K,
                                                           Epi epi, int* __restrict__ err) {
@@ -144,8 +174,10 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_tc(const __nv_bfloat16* _
   bool timed_out = false;
   const int nk = K / kGemmBK;
   for (int kc = 0; kc < nk; ++kc) {
-    load_tile_kmajor<kGemmBM>(sA, A + (int64_t)m0 * K + kc * kGemmBK, K, tid);
-    load_tile_kmajor<kGemmBN>(sB, B + (int64_t)n0 * K + kc * kGemmBK, K, tid);
+    if constexpr (AT) load_tile_mnmajor<kGemmBM>(sA, A + (int64_t)kc * kGemmBK * M + m0, M, tid);
+    else load_tile_kmajor<kGemmBM>(sA, A + (int64_t)m0 * K + kc * kGemmBK, K, tid);
+    if constexpr (BT) load_tile_mnmajor<kGemmBN>(sB, B + (int64_t)kc * kGemmBK * N + n0, N, tid);
+    else load_tile_kmajor<kGemmBN>(sB, B + (int64_t)n0 * K + kc * kGemmBK, K, tid);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     if (tid == 0) {
@@ -181,13 +213,15 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_tc(const __nv_bfloat16* _
   if (!timed_out) {
     // epilogue: warp w owns TMEM lanes 32w..32w+31 = rows m0 + 32w + lane
     const int row = m0 + warp * 32 + lane;
+    float part = 0.f;
 #pragma unroll 1
     for (int c0 = 0; c0 < kGemmBN; c0 += 32) {
       float v[32];
       tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) epi(row, n0 + c0 + j, v[j]);
+      for (int j = 0; j < 32; ++j) part += epi(row, n0 + c0 + j, v[j]);
     }
+    epi_sum(epi, part);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -278,7 +312,23 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   return false;
 }
 
-template <class Epi, class TMap, int BN>
+// MN-major with 128-byte swizzle (the operand stored [K][MN]): a box of 64 MN
+// elements x 64 k is 64 rows of 128 B, in 8-row atoms of 1024 B along K (stride
+// byte offset); the next 64 MN elements are the next box (leading byte offset).
+constexpr uint32_t kMnBox = 64 * kGemmBK * 2;
+__device__ __forceinline__ uint64_t make_sdesc_sw128_mn(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)(kMnBox >> 4) << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+
+// AT (BT): A is stored [K][M] (B is stored [K][N]); the tensor core reads either
+// order, so no operand is transposed in memory first.
+template <class Epi, class TMap, int BN, bool AT, bool BT>
 __global__ void __launch_bounds__(kGemmTmaThreads, 2) k_gemm_tma(const __grid_constant__ TMap tmA,
                                                                  const __grid_constant__ TMap tmB, int M, int N, int K,
                                                                  Epi epi, int* __restrict__ err) {
@@ -317,12 +367,24 @@ __global__ void __launch_bounds__(kGemmTmaThreads, 2) k_gemm_tma(const __grid_co
       }
       const uint32_t sa = base + s * G::kStageBytes, sb = sa + G::kABytes;
       mbar_expect_tx(&full[s], G::kStageBytes);
-      tma_load_2d(sa, &tmA, kc * kGemmBK, m0, &full[s]);
-      tma_load_2d(sb, &tmB, kc * kGemmBK, n0, &full[s]);
+      if constexpr (AT) {
+#pragma unroll
+        for (int i = 0; i < kGemmBM / 64; ++i)
+          tma_load_2d(sa + i * kMnBox, &tmA, m0 + 64 * i, kc * kGemmBK, &full[s]);
+      } else {
+        tma_load_2d(sa, &tmA, kc * kGemmBK, m0, &full[s]);
+      }
+      if constexpr (BT) {
+#pragma unroll
+        for (int i = 0; i < BN / 64; ++i)
+          tma_load_2d(sb + i * kMnBox, &tmB, n0 + 64 * i, kc * kGemmBK, &full[s]);
+      } else {
+        tma_load_2d(sb, &tmB, kc * kGemmBK, n0, &full[s]);
+      }
     }
   } else if (warp == 1 && lane == 0) {
     // MMA issuer
-    constexpr uint32_t idesc = make_idesc_bf16(kGemmBM, BN);
+    constexpr uint32_t idesc = make_idesc_bf16(kGemmBM, BN, AT, BT);
     bool ok = true;
     for (int kc = 0; kc < nk; ++kc) {
       const int s = kc % G::kStages;
@@ -334,7 +396,8 @@ __global__ void __launch_bounds__(kGemmTmaThreads, 2) k_gemm_tma(const __grid_co
       const uint32_t sa = base + s * G::kStageBytes, sb = sa + G::kABytes;
 #pragma unroll
       for (int kk = 0; kk < kGemmBK / 16; ++kk)
-        umma_bf16(tmem, make_sdesc_sw128(sa + kk * 32), make_sdesc_sw128(sb + kk * 32), idesc,
+        umma_bf16(tmem, AT ? make_sdesc_sw128_mn(sa + kk * 2048) : make_sdesc_sw128(sa + kk * 32),
+                  BT ? make_sdesc_sw128_mn(sb + kk * 2048) : make_sdesc_sw128(sb + kk * 32), idesc,
                   (kc > 0 || kk > 0) ? 1u : 0u);
       umma_commit(&empty[s]);
     }
@@ -350,6 +413,7 @@ __global__ void __launch_bounds__(kGemmTmaThreads, 2) k_gemm_tma(const __grid_co
   } else {
     float* tr = reinterpret_cast<float*>(smem) + warp * (32 * 33);
     const int rg = warp & 3, row0 = m0 + rg * 32;
+    float part = 0.f;
 #pragma unroll 1
     for (int c0 = (warp >> 2) * (BN / 2); c0 < ((warp >> 2) + 1) * (BN / 2); c0 += 32) {
       float v[32];
@@ -358,9 +422,10 @@ __global__ void __launch_bounds__(kGemmTmaThreads, 2) k_gemm_tma(const __grid_co
       for (int j = 0; j < 32; ++j) tr[lane * 33 + j] = v[j];
       __syncwarp();
 #pragma unroll 4
-      for (int r = 0; r < 32; ++r) epi(row0 + r, n0 + c0 + lane, tr[r * 33 + lane]);
+      for (int r = 0; r < 32; ++r) part += epi(row0 + r, n0 + c0 + lane, tr[r * 33 + lane]);
       __syncwarp();
     }
+    epi_sum(epi, part);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();

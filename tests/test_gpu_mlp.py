@@ -60,6 +60,41 @@ def test_predict_ragged_shapes(nin, nout, B, off):
     assert ((Y - ref).abs().max() / ref.abs().max()).item() < 2 ** -5
 
 
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("nin,nout,B", [(201, 131, 129), (64, 90, 1), (258, 34, 300)])
+def test_train_step_ragged_shapes(nin, nout, B, variant):
+    """Gradients at odd feature and output counts and ragged batches, with each
+    product kernel, against FP64 autograd (BF16 operands: 2^-8 each), the loss,
+    and AdamW's first step from the gradients returned."""
+    ws = _ws()
+    nh1, nh2 = 128, 256
+    g = torch.Generator(device="cuda").manual_seed(B + nin)
+    net = ws.MLP(nin, nh1, nh2, nout, bmax=300, seed=1)
+    P = [torch.randn(*s, device="cuda", generator=g) / s[-1] ** 0.5
+         for s in [(nh1, nin), (nh1,), (nh2, nh1), (nh2,), (nout, nh2), (nout,)]]
+    net.set_params([p.cpu().numpy() for p in P])
+    X, T = torch.randn(B, nin, device="cuda", generator=g), torch.randn(B, nout, device="cuda", generator=g)
+    D = [p.double().requires_grad_() for p in P]
+    h = X.double()
+    for l in (0, 2):
+        h = torch.nn.functional.gelu(h @ D[l].T + D[l + 1])
+    ref = ((h @ D[4].T + D[5] - T.double()) ** 2).mean()
+    ref.backward()
+    try:
+        assert ws.lib.pf_gemm_set_variant(variant) == 0
+        loss = net.train_step(X, T, lr=1e-3, wd=0.1)
+    finally:
+        ws.lib.pf_gemm_set_variant(1)
+    assert net.error() == 0
+    assert abs(loss.item() / ref.item() - 1) < 2 ** -6
+    new = net.params()
+    for k, (q, d, p0, p1) in enumerate(zip(net.grads(), D, P, new)):
+        r = d.grad.cpu().numpy()
+        assert np.linalg.norm(q - r) / np.linalg.norm(r) < 2 ** -5, k
+        w = p0.cpu().numpy().astype(np.float64) * (1 - (1e-4 if k % 2 == 0 else 0.0))
+        assert np.max(np.abs(p1 - (w - 1e-3 * q / (np.abs(q) + 1e-8)))) < 1e-6, k
+
+
 def _rel(a, b):
     return float(np.linalg.norm(a - b) / max(np.linalg.norm(b), 1e-30))
 
