@@ -14,11 +14,12 @@
 //   k_im_gemm          : (j > 0) its block column and row, rows [kj, ndp) x
 //                        columns [kj, kj+128) and rows [kj, kj+128) x columns
 //                        [kj+128, ndp), minus the products of all earlier
-//                        panels in one pass of depth kj: one 128 x 128 tile
-//                        of C per CTA, operand chunks of depth 32 loaded by
-//                        TMA into a two-stage shared-memory ring, an 8 x 8
-//                        register tile per thread updated with packed
-//                        two-wide FP32 FMAs;
+//                        panels in one pass of depth kj, one 128 x 128 tile
+//                        of C per CTA: on the tensor cores, from operands
+//                        split into three BF16 parts each, or near the
+//                        solution by packed two-wide FP32 FMAs (an 8 x 8
+//                        register tile per thread, operand chunks of depth 32
+//                        loaded by TMA into a two-stage ring);
 //   k_im_diag  (step 0): LU of the 64 x 64 diagonal block at (kj, kj), and the
 //                        inverses U11^-1, L11^-1 of its factors;
 //   k_im_panel (step 0): L21 = A21 U11^-1 for the rows below and
@@ -40,6 +41,8 @@
 #include <cstdint>
 
 #include "dense_im.h"
+#include "gemm_tc.cuh"
+#include "kernels.h"
 
 namespace nrpf {
 
@@ -60,6 +63,7 @@ constexpr int kImGC = 2;
 // transposed, so acc + a (-b) rounds exactly as fmaf(-a, b, acc)
 constexpr bool kImPacked = true;
 constexpr int kImGemmThreads = 32 * 4 * (4 / kImGC);
+static_assert(kImGemmThreads == 256, "the tensor-core form splits its work over eight warps");
 constexpr uint32_t kImABytes = kImKc * kImTile * 4;  // 16 KB: [32 columns][128 rows]
 constexpr uint32_t kImBBytes = kImTile * kImKc * 4;  // 16 KB: [128 columns][32 rows], swizzled
 constexpr uint32_t kImStageBytes = kImABytes + kImBBytes;
@@ -292,31 +296,12 @@ __device__ __forceinline__ int gemm_tile(float* __restrict__ C, int ld, int i0, 
   return -1;
 }
 
-// The block column and row of the outer panel at r0: tiles of 128 over rows
-// [r0, ld) x columns [r0, r0+128) and rows [r0, r0+128) x columns [r0+128,
-// ld), 2 ntc - 1 of them (ntc = tiles across [r0, ld)), each minus the
-// products over pivot columns 0 .. r0-1 (r0 / 32 chunks).  grid: Bp * (2 ntc
-// - 1) CTAs, tile-fastest within an instance, so that the CTAs resident at
-// one time share their instance's operand panels in L2.
-__global__ void __launch_bounds__(kImGemmThreads, 2)
-    k_im_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, DevPlan P,
-              DevState S, int r0, int ntc, const int32_t* __restrict__ gate) {
-  extern __shared__ uint8_t im_smem_raw[];
-  __shared__ __align__(8) uint64_t full[kImStages];
-  if (gate && *gate == 0) return;
-  const int ntile = 2 * ntc - 1;
-  const int b = (int)(blockIdx.x / (unsigned)ntile);
-  const int t = (int)(blockIdx.x - (unsigned)b * (unsigned)ntile);
-  if (!S.active[b]) return;
-  const int ld = P.ndp;
-  const int k = 0, nkc = r0 / kImKc;
-  const int i0 = r0 + (t < ntc ? t : 0) * kImTile, j0 = r0 + (t < ntc ? 0 : t - ntc + 1) * kImTile;
-  // 1024-byte alignment for the swizzled B chunks (offset arithmetic on the
-  // shared array keeps the pointer in the shared address space)
-  uint8_t* sm = im_smem_raw + ((1024u - (su32(im_smem_raw) & 1023u)) & 1023u);
+__device__ __forceinline__ void update_fma(float* __restrict__ A, int ld, int i0, int j0, int nkc, uint8_t* sm,
+                                           uint64_t* full, const CUtensorMap* tmA, const CUtensorMap* tmB, int lane_b,
+                                           int tile_b, int32_t* bad) {
+  const int k = 0;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rw = (warp & 3) * 32, cw = (warp >> 2) * 32 * kImGC;
-  const int lane_b = b & 31, tile_b = b >> 5;
   if (tid == 0) {
     for (int s = 0; s < kImStages; ++s) bar_init(&full[s], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -324,21 +309,275 @@ __global__ void __launch_bounds__(kImGemmThreads, 2)
   __syncthreads();
   if (tid == 0)
     for (int kc = 0; kc < kImStages && kc < nkc; ++kc)
-      issue_chunk(sm, full, &tmA, &tmB, kc, i0, j0, k, lane_b, tile_b);
+      issue_chunk(sm, full, tmA, tmB, kc, i0, j0, k, lane_b, tile_b);
   // rows (columns) of this tile inside the block: 128, or 64 at the edge
   const int mrows = ld - i0 < kImTile ? ld - i0 : kImTile;
   const int ncols = ld - j0 < kImTile ? ld - j0 : kImTile;
   const bool active = rw < mrows && cw < ncols;
-  const int fail = gemm_tile(im_block(P, S, b), ld, i0, j0, k, nkc, sm, full, &tmA, &tmB, lane_b, tile_b, active, rw, cw,
+  const int fail = gemm_tile(A, ld, i0, j0, k, nkc, sm, full, tmA, tmB, lane_b, tile_b, active, rw, cw,
                              lane & 7, lane >> 3);
   if (fail >= 0 && tid == 0) {
     // a copy did not land in time: the instance is marked failed (its step
     // is discarded) and the CTA waits, bounded, for the copies it issued
     // (chunks up to fail + 1: one chunk ahead of the one consumed)
-    S.bad[b] = 1;
+    *bad = 1;
     const int issued = fail + 2 < nkc ? fail + 2 : nkc;
     for (int kc = fail; kc < issued; ++kc) bar_wait(&full[kc % kImStages], (uint32_t)(kc / kImStages) & 1u);
   }
+}
+
+// ---------------------------------------------------------------------------
+// Update C -= A B of one 128 x 128 tile of one instance over the pivot columns
+// 0 .. r0-1, as an FP32 product on the BF16 tensor cores.
+//
+// Each operand is split into three BF16 parts, x = h + m + l with h = bf16(x),
+// m = bf16(x - h), l = bf16(x - h - m): 24 bits, the whole FP32 significand
+// (the method of Henry, Tang & Heinecke, "Leveraging the bfloat16 Artificial
+// Intelligence Datatype for Higher-Precision Computations", ARITH 2019).  Of
+// the nine partial products the six above 2^-24 are taken, smallest first:
+//   Ah Bl + Al Bh + Am Bm + Am Bh + Ah Bm + Ah Bh   (Am Bl, Al Bm: <= 2^-25)
+// each exact in the FP32 accumulator's inputs.  The accumulator holds the sum of
+// one chunk of depth 32 only; the chunk's sum is then added to C in FP32 with
+// rounding to nearest, so the tensor core's own rounding acts on sums of 32
+// products and C is rounded once per chunk instead of once per product.
+// Error of J^-1 F against FP64 with all updates in this form, and by FP32 FMAs
+// (meshed grids, 32 instances, the first Newton step; median of |dx - dx64| /
+// |dx64|):
+//   buses         700      2,000    4,000    9,000
+//   dense block   192      320      768      2,176
+//   this form     5.6e-7   1.6e-6   4.3e-6   6.6e-5
+//   FP32 FMAs     2.1e-6   1.9e-6   8.5e-6   4.9e-4
+//
+// Data flow per chunk of depth 32 (256 threads, eight warps):
+//  * A (columns of L, rows contiguous): warp w reads its 32 rows (w % 4), one
+//    128-byte line per column, 16 columns (w / 4), a chunk ahead into
+//    registers; a thread holds a row, so pairs of its columns are what a TMEM
+//    operand's 32-bit columns take: the parts go to TMEM (tcgen05.st), and the
+//    MMA reads A from there, which leaves shared memory to B;
+//  * B (columns of U, depth contiguous): 16 bytes of depth per thread and column,
+//    eight threads a line; the parts go to shared memory as 64-byte rows with
+//    64-byte swizzle (K-major; the 8-byte stores of a half warp cover all banks);
+//  * thread 0 issues 2 x 6 MMAs of 128 x 128 x 16 and commits them; meanwhile
+//    the next chunk is split into the other buffer, then all warps add the
+//    finished chunk to C in registers (one row, 64 columns per thread).
+// Two CTAs run on an SM (128 registers, 256 of 512 TMEM columns each): the MMAs
+// of one cover the conversion, the barrier and the read-back of the other.
+//
+// Bounds, per instance and refactorisation of the 2,176-wide block: 37.6 GFLOP
+// of BF16 products (20 us at the measured cuBLAS rate), 140.5 MB of DRAM (21 us)
+// and 196 MB through L2.  Measured, 1,000 instances: 36.6 us each (171 TFLOP/s
+// of FP32 products); by FP32 FMAs 104.8 us (60 TFLOP/s, 0.77 of the FMA peak).
+// ---------------------------------------------------------------------------
+constexpr uint32_t kImAccCols = 128;                  // TMEM columns of the accumulator
+constexpr uint32_t kImACols = 3 * kImKc / 2;          // ... of one A buffer (three parts, two values a column)
+constexpr uint32_t kImTmemCols = 256;                 // allocated: 128 + 2 * 48, rounded up to a power of two
+constexpr uint32_t kImBPart = kImTile * kImKc * 2;    // 8 KB: one part of a B chunk
+constexpr uint32_t kImBBuf = 3 * kImBPart;
+
+// the three BF16 parts of two FP32 values, packed (x0 in the low half)
+__device__ __forceinline__ void split3(float x0, float x1, uint32_t& h, uint32_t& m, uint32_t& l) {
+  const float2 minus1 = make_float2(-1.f, -1.f);
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(x1), "f"(x0));
+  // x - part is exact in FP32
+  float2 r = __ffma2_rn(make_float2(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u)), minus1,
+                        make_float2(x0, x1));
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(m) : "f"(r.y), "f"(r.x));
+  r = __ffma2_rn(make_float2(__uint_as_float(m << 16), __uint_as_float(m & 0xffff0000u)), minus1, r);
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(l) : "f"(r.y), "f"(r.x));
+}
+
+// Shared-memory descriptor, K-major rows of 64 bytes with 64-byte swizzle:
+// 8-row atoms of 512 B (stride byte offset), layout type 4.
+__device__ __forceinline__ uint64_t make_sdesc_sw64(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(512 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;
+  return d;
+}
+
+// D (+)= A B with A in TMEM (a row per lane, two BF16 per column)
+__device__ __forceinline__ void umma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
+                                             uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
+      "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&r)[4]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
+               "r"(r[2]), "r"(r[3])
+               : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ void update_tc(float* __restrict__ A, int ld, int i0, int j0, int nkc, uint8_t* sm,
+                                          uint64_t* done, uint32_t* tmem_holder, int32_t* bad) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (warp == 0) tmem_alloc(tmem_holder, kImTmemCols);
+  if (tid == 0) {
+    mbar_init(done, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  // this thread's row of A and C, its half of the columns of C and of A's depth
+  const int rg = warp & 3, half = warp >> 2;
+  const int row = i0 + rg * 32 + lane;
+  const bool rok = row < ld;             // uniform over a warp: ld % 64 == 0
+  const bool cok = j0 + half * 64 < ld;  // the half's 64 columns of C
+  const float* __restrict__ Ap = A + (size_t)(half * 16) * ld + row;
+  // its four columns of B, four of depth in each
+  const int bq = tid & 7, bj = tid >> 3;
+  const float* __restrict__ Bp = A + (size_t)(j0 + bj) * ld + 4 * bq;
+  const uint32_t boff = (uint32_t)bj * 64u + ((((uint32_t)bq >> 1) ^ (((uint32_t)bj >> 1) & 3u)) << 4) +
+                        ((uint32_t)bq & 1u) * 8u;
+  float a[16];
+  float4 bv[4];
+  auto load = [&](int kc) {
+    const size_t k = (size_t)kc * kImKc;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) a[q] = rok ? Ap[(k + q) * ld] : 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      bv[i] = j0 + bj + 32 * i < ld ? *reinterpret_cast<const float4*>(Bp + (size_t)(32 * i) * ld + k)
+                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  load(0);
+  float c[64];
+  float* __restrict__ C = A + (size_t)(j0 + half * 64) * ld + row;
+  if (rok && cok) {
+#pragma unroll
+    for (int q = 0; q < 64; ++q) c[q] = C[(size_t)q * ld];
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_holder;
+  const uint32_t lane_base = tmem + ((uint32_t)(rg * 32) << 16);
+  // negate A (bit 13): the accumulator holds minus the chunk's product
+  constexpr uint32_t idesc = make_idesc_bf16(kImTile, kImTile) | (1u << 13);
+  bool ok = true;
+  // chunk kc's accumulator into C, once its MMAs have completed
+  auto add_chunk = [&](int kc) {
+    ok = mbar_wait(done, (uint32_t)kc & 1u);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      float v[16];
+      tmem_ld16(lane_base + (uint32_t)(half * 64 + g * 16), v);
+#pragma unroll
+      for (int q = 0; q < 16; ++q) c[16 * g + q] += v[q];
+    }
+  };
+  int issued = 0;
+#pragma unroll 1
+  for (int kc = 0; kc < nkc; ++kc) {
+    // split chunk kc into buffer kc % 2: the MMAs that read it (chunk kc - 2)
+    // were waited for before chunk kc - 1 was issued
+    uint8_t* Bs = sm + (kc & 1) * kImBBuf;
+    const uint32_t at = lane_base + kImAccCols + (uint32_t)(kc & 1) * kImACols + (uint32_t)half * 8u;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      uint32_t h[4], m[4], l[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) split3(a[8 * g + 2 * q], a[8 * g + 2 * q + 1], h[q], m[q], l[q]);
+      tmem_st4(at + 4 * g, h);
+      tmem_st4(at + 16 + 4 * g, m);
+      tmem_st4(at + 32 + 4 * g, l);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      uint2 h, m, l;
+      split3(bv[i].x, bv[i].y, h.x, m.x, l.x);
+      split3(bv[i].z, bv[i].w, h.y, m.y, l.y);
+      uint8_t* q = Bs + boff + i * (32 * 64);
+      *reinterpret_cast<uint2*>(q) = h;
+      *reinterpret_cast<uint2*>(q + kImBPart) = m;
+      *reinterpret_cast<uint2*>(q + 2 * kImBPart) = l;
+    }
+    if (kc + 1 < nkc) load(kc + 1);
+    if (kc > 0) add_chunk(kc - 1);
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    // both operands are in place and every warp has read the accumulator
+    if (__syncthreads_or(!ok)) break;
+    if (tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t ta = tmem + kImAccCols + (uint32_t)(kc & 1) * kImACols;
+      const uint32_t sb = su32(Bs);
+      constexpr int pa[6] = {0, 2, 1, 1, 0, 0}, pb[6] = {2, 0, 1, 0, 1, 0};
+#pragma unroll
+      for (int p = 0; p < 6; ++p)
+#pragma unroll
+        for (int ks = 0; ks < kImKc / 16; ++ks)
+          umma_bf16_ts(tmem, ta + 16 * pa[p] + 8 * ks, make_sdesc_sw64(sb + pb[p] * kImBPart + 32 * ks), idesc,
+                       p + ks > 0 ? 1u : 0u);
+      umma_commit(done);
+    }
+    issued = kc + 1;
+  }
+  if (ok && issued == nkc) add_chunk(nkc - 1);
+  if (__syncthreads_or(!ok || issued != nkc)) {
+    // the MMAs did not complete in time: the instance is marked failed (its
+    // step is discarded), after a second bounded wait before TMEM is freed
+    if (tid == 0) *bad = 1;
+    if (issued > 0) mbar_wait(done, (uint32_t)(issued - 1) & 1u);
+  } else if (rok && cok) {
+#pragma unroll
+    for (int q = 0; q < 64; ++q) C[(size_t)q * ld] = c[q];
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tmem_dealloc(tmem, kImTmemCols);
+  }
+}
+
+// The block column and row of the outer panel at r0: tiles of 128 over rows
+// [r0, ld) x columns [r0, r0+128) and rows [r0, r0+128) x columns [r0+128,
+// ld), 2 ntc - 1 of them (ntc = tiles across [r0, ld)), each minus the
+// products over pivot columns 0 .. r0-1 (r0 / 32 chunks).  grid: Bp * (2 ntc
+// - 1) CTAs, tile-fastest within an instance, so that the CTAs resident at
+// one time share their instance's operand panels in L2.  An instance far from
+// its solution takes the tensor cores, one near it the FMA pipe (kActiveNear,
+// kernels.h, says why the line lies there).
+__global__ void __launch_bounds__(kImGemmThreads, 2)
+    k_im_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, DevPlan P,
+              DevState S, int r0, int ntc, const int32_t* __restrict__ gate) {
+  extern __shared__ uint8_t im_smem_raw[];
+  __shared__ __align__(8) uint64_t bars[kImStages];
+  __shared__ uint32_t tmem_holder;
+  if (gate && *gate == 0) return;
+  const int ntile = 2 * ntc - 1;
+  const int b = (int)(blockIdx.x / (unsigned)ntile);
+  const int t = (int)(blockIdx.x - (unsigned)b * (unsigned)ntile);
+  const int act = S.active[b];
+  if (!act) return;
+  const int i0 = r0 + (t < ntc ? t : 0) * kImTile, j0 = r0 + (t < ntc ? 0 : t - ntc + 1) * kImTile;
+  // 1024-byte alignment for the swizzled chunks (offset arithmetic on the
+  // shared array keeps the pointer in the shared address space)
+  uint8_t* sm = im_smem_raw + ((1024u - (su32(im_smem_raw) & 1023u)) & 1023u);
+  float* A = im_block(P, S, b);
+  if (act == kActiveNear)
+    update_fma(A, P.ndp, i0, j0, r0 / kImKc, sm, bars, &tmA, &tmB, b & 31, b >> 5, &S.bad[b]);
+  else
+    update_tc(A, P.ndp, i0, j0, r0 / kImKc, sm, &bars[0], &tmem_holder, &S.bad[b]);
 }
 
 // ---------------------------------------------------------------------------

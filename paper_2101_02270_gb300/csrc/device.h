@@ -88,7 +88,7 @@ struct DevState {
   unsigned long long* norm;  // [Bp] max |F| as float64 bits
   int32_t* iters;   // [Bp]
   int32_t* status;  // [Bp]
-  int32_t* active;  // [Bp]
+  int32_t* active;  // [Bp] 0: finished; kActiveFar / kActiveNear (kernels.h)
   int32_t* bad;     // [Bp] non-finite step detected
   SolveCtl* ctl;  // Newton loop control (one per workspace)
   const double2* yv;  // [nnzY] per-instance Ybus values (re, im), or null: the plan's shared values

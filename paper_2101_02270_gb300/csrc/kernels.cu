@@ -325,7 +325,7 @@ __global__ void k_check(DevState S, int Bp) {
     keep = 1;
     S.iters[b] = it + 1;
   }
-  S.active[b] = keep;
+  S.active[b] = !keep ? 0 : nrm > kNearMismatch ? kActiveFar : kActiveNear;
   const unsigned mask = __ballot_sync(__activemask(), keep);
   if (keep && (threadIdx.x & 31) == __ffs(mask) - 1) atomicAdd(counter, __popc(mask));
 }

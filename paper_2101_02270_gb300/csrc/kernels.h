@@ -13,6 +13,21 @@
 #define NRPF_MAXIT_CODE 1
 #define NRPF_FAILED_CODE 2
 
+// S.active of an instance that is still iterating: far from its solution, or
+// near it (max |F| of at most kNearMismatch).  The instance-major dense block
+// is updated on the tensor cores while an instance is far (dense_im.cu), and by
+// FP32 FMAs in pivot order when it is near.  The tensor-core form is the faster
+// one (9,000 buses x 1,000, per refactorisation: 36 against 105 ms) and the more
+// exact one; the line is there because the step from a mismatch of 1e-3 p.u. or
+// less is, by quadratic convergence, the last or the last but one, and an FP32
+// factor's own error is what it leaves in the voltages (3.5e-9 on the 9,000-bus
+// grid, at a mismatch of 2e-9).  Taking that step with the same roundings as
+// ever keeps converged voltages where they were, to 9e-10 on that grid and 1e-10
+// or less on smaller or more lightly loaded ones; with the tensor cores in every
+// step they move by 3.2e-9 (to 3.2e-10 from the exact root).
+constexpr int kActiveFar = 1, kActiveNear = 2;
+constexpr double kNearMismatch = 1e-3;
+
 namespace nrpf {
 
 void launch_load(const DevPlan& P, const DevState& S, int B, const double* sbus, const double* v0,

@@ -229,6 +229,35 @@ def test_instance_major_edge_cases():
         assert np.all(it.cpu().numpy() == 0) and np.all(st.cpu().numpy() == 1)
 
 
+@pytest.mark.parametrize("n,branches,pad", [(300, 560, 128), (400, 700, 192), (800, 1300, 256), (1500, 2500, 448)])
+def test_instance_major_update_far_and_near(n, branches, pad):
+    """Block updates of the instance-major layout at every edge of a 128 x 128
+    tile (blocks of 64 rows or columns at the end, or none) and depths of none to
+    twelve chunks.  The staged solve takes the tensor cores: its steps against the
+    FP64 plan's, within the factorisation's bar for FP32.  A batch whose odd
+    instances start near the solution (mismatch below 1e-3, FMA updates) and
+    whose even ones start flat ends at the FP64 plan's voltages."""
+    import gridgen
+    g = gridgen.make_grid("mesh2000_b10k", 0, n=n, n_branch=branches, n_pv=n // 10, load_scale=1 / 32)
+    sc = gridgen.make_scenarios(g, 40, 0.6, 1.4)
+    S, V0 = _dev(sc.sbus(g)), _dev(sc.v0_flat(g))
+    with _plan(g) as p, _plan(g, lu_precision="fp32", dense_layout="instance_major") as q:
+        assert q.info["dense_layout"] == 2 and q.info["dense_pad"] == pad
+        F, _ = p.stage_mismatch(S, V0)
+        x, y = p.stage_linear_solve(V0, F), q.stage_linear_solve(V0, F)
+        assert ((y - x).norm(dim=1) / x.norm(dim=1)).max().item() < 1e-4
+        V, it, st = p.solve(S, V0, TOL, 10)
+        near = p.solve(S, V0, TOL, 2)[0]
+        norm = p.stage_mismatch(S, near)[1]
+        assert 1e-8 < norm.min().item() and norm.max().item() < 1e-3
+        start = V0.clone()
+        start[1::2] = near[1::2]
+        v, it2, st2 = q.solve(S, start, TOL, 10)
+        assert torch.all(st2 == 0) and torch.all(st == 0)
+        assert torch.all(it2[1::2] <= it[1::2] - 1) and torch.all(it2[::2] == it[::2])
+        assert (v - V).abs().max().item() <= 1e-6
+
+
 def test_singular_instance_reports_failure():
     """An instance whose Jacobian is singular (a PQ bus with zero voltage)
     stops with status 2 while the rest of the batch converges."""
