@@ -869,85 +869,161 @@ __global__ void k_bwd_level(DevPlan P, DevState S, int r0, int r1, const int32_t
   X[(size_t)i * kTile] = acc / LU[(size_t)P.dp[i] * kTile];
 }
 
-
-// Dense block solves with one tile's right-hand side held in shared memory.
-// CTA = one tile (32 instances) x kSolveWarps warps.  Forward (unit lower) and
-// backward (upper) substitution by blocks of SB columns: warp 0 solves the
-// SB x SB diagonal block, then every warp updates its share of the remaining
-// rows with SB multiply-adds each (the row updates of a block are independent).
-constexpr int kSolveWarps = 8;
-
-template <typename T, int SB, bool SMEM>
-__global__ void __launch_bounds__(32 * kSolveWarps) k_dense_solve_smem(DevPlan P, DevState S,
-                                                                       const int32_t* __restrict__ gate) {
+// Dense block solves, one CTA of NW warps per tile (32 instances), the tile's
+// right-hand side in shared memory when it fits.  Forward (unit lower) and
+// backward (upper) substitution by blocks of SB columns: as soon as a block of
+// x is known, warp 0 updates the next block's SB rows and solves them against
+// their SB x SB diagonal block, in registers, while the other warps update the
+// rows beyond (independent multiply-adds), so that the serial part of a block
+// hides behind the rest of it and one barrier per block suffices.  Backward, the
+// last warp has the reciprocals of the pivots ready two blocks ahead: an FP64
+// division on the serial part costs as much as ten of its multiply-adds.
+// Reads the block once (592 KB per instance of the 2,000-bus FP64 plan) and is
+// bound by latency and barriers: what matters is loads in flight.  A warp takes
+// four rows of a column in FP32 (one 16-byte load per lane), two in FP64, for
+// all SB columns at once.  NW: 32 while every tile can have an SM of its own
+// (one CTA of 1,024 threads per SM), else 16 (FP64: 10, for its registers) and
+// three CTAs per SM.  Measured per
+// solve with 8 warps, a row at a time, the diagonal block in between (two
+// barriers per block), and in this form:
+//   FP64, 272 wide:  1 tile 1.07 -> 0.76 ms, 60 tiles 1.95 -> 0.90 ms, 313 tiles 2.44 -> 2.01 ms
+//   FP32, 320 wide: 11 tiles 1.26 -> 0.31 ms, 313 tiles 1.36 -> 0.87 ms
+// (FP64: the pipe takes 16 cycles per multiply-add of a warp, 0.6 ms per tile and
+// SM.)
+template <typename T, int SB, bool SMEM, int NW>
+__global__ void __launch_bounds__(32 * NW, NW == 32 ? 1 : 3) k_dense_solve_smem(DevPlan P, DevState S,
+                                                                               const int32_t* __restrict__ gate) {
+  constexpr int U = DenseGroup<T>::G == 4 ? 4 : 2;  // rows per step of a warp
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ T rec[2][SB][kTile];  // reciprocal pivots of two blocks
   if (gate && *gate == 0) return;
   const int lane = threadIdx.x, warp = threadIdx.y;
   const int tile = blockIdx.x;
   if (!__syncthreads_or(S.active[tile * kTile + lane])) return;
   const T* __restrict__ Ab = reinterpret_cast<const T*>(S.lu) + ((size_t)tile * P.NLU + P.NS) * kTile;
-  const size_t cstride = (size_t)P.ndp * kTile;
-  auto A = [&](int r, int c) -> T {
-    if constexpr (DenseGroup<T>::G == 1)
-      return Ab[(size_t)c * cstride + (size_t)r * kTile + lane];
-    else
-      return Ab[dense_off<T>(r, c, P.ndp, lane)];
-  };
   T* __restrict__ X = reinterpret_cast<T*>(S.x) + ((size_t)tile * P.mp + P.s) * kTile + lane;
   const int ld = P.ndp;
+  // rows r .. r+U-1 of column c (r a multiple of U)
+  auto ldu = [&](int r, int c, T(&v)[U]) {
+    if constexpr (U == 4) {
+      ld4(Ab, r, c, ld, lane, v);
+    } else {
+#pragma unroll
+      for (int i = 0; i < U; ++i) v[i] = Ab[dense_off<T>(r + i, c, ld, lane)];
+    }
+  };
   // the tile's right-hand side: in shared memory when it fits, else in place
   // in global memory (same blocked algorithm, L2-resident per tile)
   T* xs = SMEM ? reinterpret_cast<T*>(smem_raw) : X - lane;  // xs[r * 32 + lane]
-  if (SMEM) {
-    for (int r = warp; r < ld; r += kSolveWarps) xs[r * kTile + lane] = X[(size_t)r * kTile];
-    __syncthreads();
-  }
-  for (int k0 = 0; k0 < ld; k0 += SB) {
+  if (SMEM)
+    for (int r = warp; r < ld; r += NW) xs[r * kTile + lane] = X[(size_t)r * kTile];
+  // rows r .. r+U-1 minus the block's columns k0 .. k0+SB-1 times xb
+  auto update = [&](int r, int k0, const T(&xb)[SB], T(&acc)[U]) {
+#pragma unroll
+    for (int i = 0; i < U; ++i) acc[i] = xs[(r + i) * kTile + lane];
+#pragma unroll
+    for (int c = 0; c < SB; ++c) {
+      T v[U];
+      ldu(r, k0 + c, v);
+#pragma unroll
+      for (int i = 0; i < U; ++i) acc[i] -= v[i] * xb[c];
+    }
+  };
+  // warp 0: rows k .. k+SB-1 of the block before (columns k0 .., or none when
+  // k0 < 0), then their own diagonal block
+  auto head = [&](int k, int k0, const T(&xb)[SB], bool upper) {
+    T x[SB];
+#pragma unroll
+    for (int g = 0; g < SB / U; ++g) {
+      T acc[U];
+      if (k0 >= 0) {
+        update(k + U * g, k0, xb, acc);
+      } else {
+#pragma unroll
+        for (int i = 0; i < U; ++i) acc[i] = xs[(k + U * g + i) * kTile + lane];
+      }
+#pragma unroll
+      for (int i = 0; i < U; ++i) x[U * g + i] = acc[i];
+    }
+    if (!upper) {
+#pragma unroll
+      for (int c = 0; c < SB - 1; ++c)
+#pragma unroll
+        for (int g = (c + 1) / U; g < SB / U; ++g) {
+          T v[U];
+          ldu(k + U * g, k + c, v);
+#pragma unroll
+          for (int i = 0; i < U; ++i)
+            if (U * g + i > c) x[U * g + i] -= v[i] * x[c];
+        }
+    } else {
+#pragma unroll
+      for (int c = SB - 1; c >= 0; --c)
+#pragma unroll
+        for (int g = c / U; g >= 0; --g) {
+          T v[U];
+          ldu(k + U * g, k + c, v);
+#pragma unroll
+          for (int i = U - 1; i >= 0; --i) {
+            if (U * g + i == c) x[c] *= rec[(k / SB) & 1][c][lane];
+            if (U * g + i < c) x[U * g + i] -= v[i] * x[c];
+          }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < SB; ++r) xs[(k + r) * kTile + lane] = x[r];
+  };
+  auto reciprocals = [&](int k) {
+    T d[SB];
+#pragma unroll
+    for (int c = 0; c < SB; ++c) d[c] = Ab[dense_off<T>(k + c, k + c, ld, lane)];
+#pragma unroll
+    for (int c = 0; c < SB; ++c) rec[(k / SB) & 1][c][lane] = (T)1 / d[c];
+  };
+  if (warp == NW - 1) reciprocals(ld - SB);
+  if (warp == NW - 2 && ld > SB) reciprocals(ld - 2 * SB);
+  T xb[SB];
+#pragma unroll
+  for (int c = 0; c < SB; ++c) xb[c] = (T)0;
+  __syncthreads();
+  if (warp == 0) head(0, -1, xb, false);
+  __syncthreads();
+  for (int k0 = 0; k0 + SB < ld; k0 += SB) {
+#pragma unroll
+    for (int c = 0; c < SB; ++c) xb[c] = xs[(k0 + c) * kTile + lane];
     if (warp == 0) {
+      head(k0 + SB, k0, xb, false);
+    } else {
+      for (int r = k0 + 2 * SB + U * (warp - 1); r < ld; r += U * (NW - 1)) {
+        T acc[U];
+        update(r, k0, xb, acc);
 #pragma unroll
-      for (int c = 0; c < SB; ++c) {
-        const T xc = xs[(k0 + c) * kTile + lane];
-#pragma unroll
-        for (int r = c + 1; r < SB; ++r)
-          xs[(k0 + r) * kTile + lane] -= A(k0 + r, k0 + c) * xc;
+        for (int i = 0; i < U; ++i) xs[(r + i) * kTile + lane] = acc[i];
       }
     }
     __syncthreads();
-    T xb[SB];
-#pragma unroll
-    for (int c = 0; c < SB; ++c) xb[c] = xs[(k0 + c) * kTile + lane];
-    for (int r = k0 + SB + warp; r < ld; r += kSolveWarps) {
-      T acc = xs[r * kTile + lane];
-#pragma unroll
-      for (int c = 0; c < SB; ++c) acc -= A(r, k0 + c) * xb[c];
-      xs[r * kTile + lane] = acc;
-    }
-    __syncthreads();
   }
-  for (int k0 = ld - SB; k0 >= 0; k0 -= SB) {
-    if (warp == 0) {
-#pragma unroll
-      for (int c = SB - 1; c >= 0; --c) {
-        const T xc = xs[(k0 + c) * kTile + lane] / A(k0 + c, k0 + c);
-        xs[(k0 + c) * kTile + lane] = xc;
-#pragma unroll
-        for (int r = 0; r < c; ++r) xs[(k0 + r) * kTile + lane] -= A(k0 + r, k0 + c) * xc;
-      }
-    }
-    __syncthreads();
-    T xb[SB];
+  if (warp == 0) head(ld - SB, -1, xb, true);
+  __syncthreads();
+  for (int k0 = ld - SB; k0 > 0; k0 -= SB) {
 #pragma unroll
     for (int c = 0; c < SB; ++c) xb[c] = xs[(k0 + c) * kTile + lane];
-    for (int r = warp; r < k0; r += kSolveWarps) {
-      T acc = xs[r * kTile + lane];
+    if (warp == 0) {
+      head(k0 - SB, k0, xb, true);
+    } else {
+      // block k0's have been used, and block k0 - 2 SB takes their place
+      if (warp == NW - 1 && k0 >= 2 * SB) reciprocals(k0 - 2 * SB);
+      for (int r = U * (warp - 1); r < k0 - SB; r += U * (NW - 1)) {
+        T acc[U];
+        update(r, k0, xb, acc);
 #pragma unroll
-      for (int c = 0; c < SB; ++c) acc -= A(r, k0 + c) * xb[c];
-      xs[r * kTile + lane] = acc;
+        for (int i = 0; i < U; ++i) xs[(r + i) * kTile + lane] = acc[i];
+      }
     }
     __syncthreads();
   }
   if (SMEM)
-    for (int r = warp; r < ld; r += kSolveWarps) X[(size_t)r * kTile] = xs[r * kTile + lane];
+    for (int r = warp; r < ld; r += NW) X[(size_t)r * kTile] = xs[r * kTile + lane];
 }
 
 // ---------------------------------------------------------------------------
@@ -1202,23 +1278,32 @@ void launch_factor(const DevPlan& P, const DevState& S, const std::vector<int32_
 // Dense solve with the tile's right-hand side in shared memory, when it fits.
 constexpr size_t kSolveSmemMax = 200 * 1024;
 
-template <typename T, int SB>
-static void launch_dense_solve_smem(const DevPlan& P, const DevState& S, const int32_t* gate, cudaStream_t st,
-                                    Recorder* rec, size_t smem) {
+template <typename T, int SB, int NW>
+static void launch_dense_solve_nw(const DevPlan& P, const DevState& S, const int32_t* gate, cudaStream_t st,
+                                  Recorder* rec, size_t smem) {
   static bool configured[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    cudaFuncSetAttribute(k_dense_solve_smem<T, SB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_dense_solve_smem<T, SB, true, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)kSolveSmemMax);
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   if (smem <= kSolveSmemMax)
     NRPF_LAUNCH(rec, K_DENSE_SOLVE, st,
-                k_dense_solve_smem<T, SB, true><<<S.Bp / kTile, dim3(32, kSolveWarps), smem, st>>>(P, S, gate));
+                k_dense_solve_smem<T, SB, true, NW><<<S.Bp / kTile, dim3(32, NW), smem, st>>>(P, S, gate));
   else
     NRPF_LAUNCH(rec, K_DENSE_SOLVE, st,
-                k_dense_solve_smem<T, SB, false><<<S.Bp / kTile, dim3(32, kSolveWarps), 0, st>>>(P, S, gate));
+                k_dense_solve_smem<T, SB, false, NW><<<S.Bp / kTile, dim3(32, NW), 0, st>>>(P, S, gate));
+}
+
+template <typename T, int SB>
+static void launch_dense_solve_smem(const DevPlan& P, const DevState& S, const int32_t* gate, cudaStream_t st,
+                                    Recorder* rec, size_t smem) {
+  if (S.Bp / kTile <= 152)
+    launch_dense_solve_nw<T, SB, 32>(P, S, gate, st, rec, smem);
+  else
+    launch_dense_solve_nw<T, SB, (sizeof(T) == 8 ? 10 : 16)>(P, S, gate, st, rec, smem);
 }
 
 template <typename T>

@@ -258,6 +258,22 @@ def test_instance_major_update_far_and_near(n, branches, pad):
         assert (v - V).abs().max().item() <= 1e-6
 
 
+@pytest.mark.parametrize("lu,panel", [("fp64", 4), ("fp64", 8), ("fp32", 4), ("fp32", 16)])
+@pytest.mark.parametrize("B", [152 * 32, 152 * 32 + 1, 304 * 32 + 1, 456 * 32 + 1])
+def test_instances_do_not_depend_on_the_batch(lu, panel, B):
+    """The shapes chosen by the number of tiles (dense solves and level
+    schedules) keep every instance's operations: a scenario's result in a batch
+    of any size is, bit for bit, the one it has in a batch of 64."""
+    g, S, V0 = case("mesh30_b64", batch=64)
+    idx = np.arange(B) % 64
+    with _plan(g, lu_precision=lu, panel=panel) as p:
+        v, it, st = p.solve(_dev(S), _dev(V0), TOL, 10)
+        v2, it2, st2 = p.solve(_dev(S[idx]), _dev(V0[idx]), TOL, 10)
+    k = torch.from_numpy(idx).cuda()
+    assert torch.all(st == 0)
+    assert torch.equal(v2, v[k]) and torch.equal(it2, it[k]) and torch.equal(st2, st[k])
+
+
 def test_singular_instance_reports_failure():
     """An instance whose Jacobian is singular (a PQ bus with zero voltage)
     stops with status 2 while the rest of the batch converges."""
