@@ -119,6 +119,9 @@ int ensure_capacity(pf_plan* p, int B) {
   // inverse pivots of the current diagonal block (interleaved dense block),
   // or U11^-1 and L11^-1 of the current 64 x 64 block (instance-major)
   AL(p->dp.dim ? (size_t)2 * 64 * 64 * Bp * sizeof(float) : (size_t)std::max(h.kb, 1) * Bp * w, inv, void*);
+  if (p->dp.n_fac_lvl > 0) {
+    AL((size_t)h.s * Bp * w, dinv, void*);
+  }
   AL((size_t)Bp * sizeof(unsigned long long), norm, unsigned long long*);
   AL((size_t)Bp * 4, iters, int32_t*);
   AL((size_t)Bp * 4, status, int32_t*);
@@ -464,6 +467,15 @@ int pf_plan_create(int n, const int32_t* rowptr, const int32_t* colidx, const do
       return rc;
     }
     d.schur_task = reinterpret_cast<const int4*>(tasks);
+    const int32_t* ops = nullptr;
+    if ((rc = upload(p, h.fac_lvl_ptr, &d.fac_lvl_ptr)) || (rc = upload(p, h.fac_task, &d.fac_task)) ||
+        (rc = upload(p, h.fac_op, &ops))) {
+      pf_plan_destroy(p);
+      return rc;
+    }
+    d.fac_op = reinterpret_cast<const int2*>(ops);
+    d.n_fac_lvl = std::max((int)h.fac_lvl_ptr.size() - 1, 0);
+    d.n_fac_task = std::max((int)h.fac_task.size() - 1, 0);
     d.n_schur = (int)(h.schur_task.size() / 4);
   }
   if (o.max_batch > 0 && (rc = ensure_capacity(p, o.max_batch))) {

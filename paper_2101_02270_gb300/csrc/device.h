@@ -42,6 +42,11 @@ struct DevPlan {
   const int32_t* dst;
   const int32_t* dp;           // [m] diagonal position (-1 for dense columns)
   const int64_t* ce;           // [m] segment end
+  // the same by entries (plan.h); n_fac_lvl = 0: by columns
+  const int32_t* fac_lvl_ptr;
+  const int32_t* fac_task;
+  const int2* fac_op;
+  int n_fac_lvl, n_fac_task;
   // Schur complement of the sparse columns into the dense block
   const int4* schur_task;     // {dense column, 32-row chunk, first entry, end}
   const int32_t* schur_ent;   // (L(i, k) position << 5) | row in chunk
@@ -85,6 +90,7 @@ struct DevState {
   void* x;       // [mp] right-hand side / solution (LU precision)
   void* lu;      // [NLU] LU values (LU precision)
   void* inv;     // [kb] inverse pivots of the current dense diagonal block
+  void* dinv;    // [s] inverse pivots of the sparse columns (LU precision)
   unsigned long long* norm;  // [Bp] max |F| as float64 bits
   int32_t* iters;   // [Bp]
   int32_t* status;  // [Bp]

@@ -439,6 +439,135 @@ __global__ void __launch_bounds__(32 * kLWarps) k_lu_sparse_level(DevPlan P, Dev
   }
 }
 
+// ---------------------------------------------------------------------------
+// The level schedules in one launch each.  A tile belongs to a cluster of C
+// CTAs, whose warps share the tasks of a level and meet at the cluster's barrier
+// (C = 1: the CTA's) before the next: one launch per level costs 3 to 4 us, most
+// of it the launch and the chain of gate, schedule and value loads, and the
+// 2,000-bus FP64 plan has 31 + 31 + 30 levels per iteration.
+// C: as many CTAs (a power of two, at most 8, of 1,024 threads) as the tiles leave
+// SMs for and a level has tasks for, 32 to a CTA: within one CTA the values stay
+// in L1 and the barrier is cheap.  With more tiles than SMs one smaller CTA each,
+// so that all are resident at once (64 registers: 2, 3, 4 CTAs of 512, 320, 256
+// threads per SM).
+// ---------------------------------------------------------------------------
+struct LevelShape {
+  int cluster, threads;
+};
+inline LevelShape level_shape(int tiles, int tasks, int levels) {
+  if (tiles > 456) return {1, 256};
+  if (tiles > 304) return {1, 320};
+  if (tiles > 152) return {1, 512};
+  int c = 8;
+  while (c > 1 && (c * tiles > 152 || (int64_t)16 * c * levels >= tasks)) c /= 2;
+  return {c, 1024};
+}
+
+__device__ __forceinline__ void level_barrier(int cluster) {
+  if (cluster > 1)
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  else
+    __syncthreads();
+}
+
+// Sparse refactorisation by entries (plan.h: fac_*), every level.  A warp takes a
+// task of up to 16 operations (or one longer entry): 32 operations come with one
+// coalesced load and are handed out by shuffles, and the values of eight are in
+// flight together; the entry being formed stays in a register and takes its
+// subtractions in ascending k, exactly as the left-looking columns do.  The
+// operations of a warp's next task are loaded ahead, across the barrier too, so
+// that a level's chain is value, arithmetic, store, barrier.  By columns
+// (k_lu_sparse_level, a launch per level) a task reads, changes and writes the
+// whole column once per k, each waiting for the one before.  Per refactorisation
+// of the 2,000-bus plans, by columns and by entries:
+//   FP64: 1 tile 2.68, 0.65 ms; 60 tiles 4.24, 1.74 ms; 313 tiles 7.57, 8.9 ms
+//   FP32: 11 tiles 0.86, 0.22 ms; 313 tiles 2.60, 2.41 ms
+// so FP64 with more tiles than SMs keeps the columns.
+template <typename T>
+__global__ void __launch_bounds__(1024) k_sparse_factor(DevPlan P, DevState S, int cluster,
+                                                        const int32_t* __restrict__ gate) {
+  if (gate && *gate == 0) return;
+  const int lane = threadIdx.x & 31;
+  const int tile = blockIdx.x / cluster;
+  if (!tile_active(S, tile, lane)) return;  // uniform over the cluster
+  const int W = cluster * (blockDim.x >> 5);
+  const int w = (blockIdx.x % cluster) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  T* LU = reinterpret_cast<T*>(S.lu) + (size_t)tile * P.NLU * kTile + lane;
+  T* DI = reinterpret_cast<T*>(S.dinv) + (size_t)tile * P.s * kTile + lane;
+  const int32_t* __restrict__ lvl = P.fac_lvl_ptr;
+  const int total = lvl[P.n_fac_lvl];
+  int nt = w, nq0 = 0, nq1 = 0;  // the task loaded ahead: its operations, 32 of them in nop
+  int2 nop = make_int2(0, 0);
+  auto fetch = [&](int t) {
+    nt = t;
+    if (t < total) {
+      nq0 = P.fac_task[t];
+      nq1 = P.fac_task[t + 1];
+      nop = P.fac_op[min(nq0 + lane, nq1 - 1)];
+    }
+  };
+  fetch(w);
+  int t1 = lvl[1], t2 = P.n_fac_lvl > 1 ? lvl[2] : t1;
+  for (int l = 0, t0 = 0; l < P.n_fac_lvl; ++l) {
+    int t = t0 + w;
+    if (t >= t1) fetch(t1 + w);
+    while (t < t1) {
+      if (nt != t) fetch(t);
+      const int q0 = nq0, q1 = nq1;
+      int2 op = nop;
+      t += W;
+      fetch(t < t1 ? t : t1 + w);
+      T acc = (T)0, scale = (T)0;
+      int pos = 0, kind = 0, col = 0;
+      auto finish = [&] {
+        if (kind == 2) acc *= scale;
+        if (kind == 3) DI[(size_t)col * kTile] = (T)1 / acc;
+        if (kind) LU[(size_t)pos * kTile] = acc;
+      };
+      for (int qb = q0; qb < q1; qb += 32) {
+        const int cnt = min(32, q1 - qb);
+        if (qb > q0) op = P.fac_op[min(qb + lane, q1 - 1)];
+        for (int i = 0; i < cnt; i += 8) {
+          T a[8], b[8];
+          int x[8], y[8];
+#pragma unroll
+          for (int z = 0; z < 8; ++z) {
+            x[z] = __shfl_sync(0xffffffffu, op.x, i + z);
+            y[z] = __shfl_sync(0xffffffffu, op.y, i + z);
+            if (i + z < cnt) {
+              a[z] = LU[(size_t)(x[z] >> 2) * kTile];
+              const int k = x[z] & 3;
+              if (k == 0) b[z] = LU[(size_t)y[z] * kTile];
+              else if (k == 2) b[z] = DI[(size_t)y[z] * kTile];
+            }
+          }
+#pragma unroll
+          for (int z = 0; z < 8; ++z) {
+            if (i + z < cnt) {
+              const int k = x[z] & 3;
+              if (k == 0) {
+                acc -= a[z] * b[z];
+              } else {
+                finish();
+                acc = a[z];
+                scale = b[z];
+                pos = x[z] >> 2;
+                kind = k;
+                col = y[z];
+              }
+            }
+          }
+        }
+      }
+      finish();
+    }
+    t0 = t1;
+    t1 = t2;
+    if (l + 3 <= P.n_fac_lvl) t2 = lvl[l + 3];
+    level_barrier(cluster);
+  }
+}
+
 // Schur complement of the sparse columns into the dense block, after the
 // sparse levels (every U(k, j) is then final).  A warp per (dense column j,
 // chunk of 32 dense rows) and tile: the rows live in shared memory (one
@@ -869,6 +998,84 @@ __global__ void k_bwd_level(DevPlan P, DevState S, int r0, int r1, const int32_t
   X[(size_t)i * kTile] = acc / LU[(size_t)P.dp[i] * kTile];
 }
 
+// All levels of the forward (BWD: backward) schedule in one launch (see
+// k_sparse_factor): a warp per row, its entries in the order of the list, four
+// products' loads in flight; the warp's next row and that row's first four
+// entries are loaded ahead, across the barrier too.
+template <typename T, bool BWD>
+__global__ void __launch_bounds__(1024) k_subst(DevPlan P, DevState S, int cluster, const int32_t* __restrict__ gate) {
+  if (gate && *gate == 0) return;
+  const int lane = threadIdx.x & 31;
+  const int tile = blockIdx.x / cluster;
+  if (!tile_active(S, tile, lane)) return;  // uniform over the cluster
+  const int W = cluster * (blockDim.x >> 5);
+  const int w = (blockIdx.x % cluster) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const T* __restrict__ LU = reinterpret_cast<const T*>(S.lu) + (size_t)tile * P.NLU * kTile + lane;
+  T* X = reinterpret_cast<T*>(S.x) + (size_t)tile * P.mp * kTile + lane;
+  const int nl = BWD ? P.n_bw_lvl : P.n_fw_lvl;
+  const int32_t* __restrict__ lvl = BWD ? P.bw_lvl_ptr : P.fw_lvl_ptr;
+  const int32_t* __restrict__ rows = BWD ? P.bw_rows : P.fw_rows;
+  const int32_t* __restrict__ ptr = BWD ? P.bw_ptr : P.fw_ptr;
+  const int32_t* __restrict__ pos = BWD ? P.bw_pos : P.fw_pos;
+  const int32_t* __restrict__ col = BWD ? P.bw_col : P.fw_col;
+  const int total = lvl[nl];
+  int nr = 0, ni = 0, ne0 = 0, ne1 = 0, np[4], nc[4];  // the row loaded ahead
+  auto fetch = [&](int r) {
+    nr = r;
+    if (r < total) {
+      ni = rows[r];
+      ne0 = ptr[r];
+      ne1 = ptr[r + 1];
+#pragma unroll
+      for (int z = 0; z < 4; ++z)
+        if (ne0 + z < ne1) {
+          np[z] = pos[ne0 + z];
+          nc[z] = col[ne0 + z];
+        }
+    }
+  };
+  fetch(w);
+  int r1 = lvl[1], r2 = nl > 1 ? lvl[2] : r1;
+  for (int l = 0, r0 = 0; l < nl; ++l) {
+    int r = r0 + w;
+    if (r >= r1) fetch(r1 + w);
+    while (r < r1) {
+      if (nr != r) fetch(r);
+      const int i = ni, e1 = ne1;
+      int e = ne0;
+      T acc = X[(size_t)i * kTile], a[4], b[4];
+      const T d = BWD ? LU[(size_t)P.dp[i] * kTile] : (T)1;
+      const int n0 = min(e1 - e, 4);
+#pragma unroll
+      for (int z = 0; z < 4; ++z)
+        if (z < n0) {
+          a[z] = LU[(size_t)np[z] * kTile];
+          b[z] = X[(size_t)nc[z] * kTile];
+        }
+      r += W;
+      fetch(r < r1 ? r : r1 + w);
+#pragma unroll
+      for (int z = 0; z < 4; ++z)
+        if (z < n0) acc -= a[z] * b[z];
+      for (e += n0; e + 4 <= e1; e += 4) {
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          a[z] = LU[(size_t)pos[e + z] * kTile];
+          b[z] = X[(size_t)col[e + z] * kTile];
+        }
+#pragma unroll
+        for (int z = 0; z < 4; ++z) acc -= a[z] * b[z];
+      }
+      for (; e < e1; ++e) acc -= LU[(size_t)pos[e] * kTile] * X[(size_t)col[e] * kTile];
+      X[(size_t)i * kTile] = BWD ? acc / d : acc;
+    }
+    r0 = r1;
+    r1 = r2;
+    if (l + 3 <= nl) r2 = lvl[l + 3];
+    level_barrier(cluster);
+  }
+}
+
 // Dense block solves, one CTA of NW warps per tile (32 instances), the tile's
 // right-hand side in shared memory when it fits.  Forward (unit lower) and
 // backward (upper) substitution by blocks of SB columns: as soon as a block of
@@ -1246,11 +1453,32 @@ static void launch_dense_outer(const DevPlan& P, const DevState& S, int k, const
   }
 }
 
+// one of the level kernels, a cluster per tile
+template <typename K>
+static void launch_levels(K kernel, int cls, const DevPlan& P, const DevState& S, int tasks, int levels,
+                          const int32_t* gate, cudaStream_t st, Recorder* rec) {
+  const int tiles = S.Bp / kTile;
+  const LevelShape sh = level_shape(tiles, tasks, levels);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(tiles * sh.cluster));
+  cfg.blockDim = dim3((unsigned)sh.threads);
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)sh.cluster;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = sh.cluster > 1 ? 1 : 0;
+  NRPF_LAUNCH(rec, cls, st, cudaLaunchKernelEx(&cfg, kernel, P, S, sh.cluster, gate));
+}
+
 template <typename T>
 void launch_factor(const DevPlan& P, const DevState& S, const std::vector<int32_t>& lvl_ptr,
                    const int32_t* gate, cudaStream_t st, Recorder* rec) {
   const int tiles = S.Bp / kTile;
-  for (size_t l = 0; l + 1 < lvl_ptr.size(); ++l) {
+  if (P.n_fac_lvl > 0 && (sizeof(T) == 4 || tiles <= 152))
+    launch_levels(k_sparse_factor<T>, K_LU_SPARSE, P, S, P.n_fac_task, P.n_fac_lvl, gate, st, rec);
+  else for (size_t l = 0; l + 1 < lvl_ptr.size(); ++l) {
     int c0 = lvl_ptr[l], c1 = lvl_ptr[l + 1];
     if (c1 <= c0) continue;
     NRPF_LAUNCH(rec, K_LU_SPARSE, st,
@@ -1309,13 +1537,7 @@ static void launch_dense_solve_smem(const DevPlan& P, const DevState& S, const i
 template <typename T>
 void launch_solve(const DevPlan& P, const DevState& S, const std::vector<int32_t>& fw_lvl,
                   const std::vector<int32_t>& bw_lvl, const int32_t* gate, cudaStream_t st, Recorder* rec) {
-  const int tiles = S.Bp / kTile;
-  for (size_t l = 0; l + 1 < fw_lvl.size(); ++l) {
-    int r0 = fw_lvl[l], r1 = fw_lvl[l + 1];
-    if (r1 > r0)
-      NRPF_LAUNCH(rec, K_FWD, st,
-                  k_fwd_level<T><<<grid2(r1 - r0, 4, tiles), dim3(32, 4), 0, st>>>(P, S, r0, r1, gate));
-  }
+  if (P.n_fw_lvl > 0) launch_levels(k_subst<T, false>, K_FWD, P, S, fw_lvl.back(), P.n_fw_lvl, gate, st, rec);
   if (sizeof(T) == 4 && P.dim) {
     if (P.ndp > 0) launch_dense_im_solve(P, S, gate, st, rec);
   } else if (P.ndp > 0) {
@@ -1325,12 +1547,7 @@ void launch_solve(const DevPlan& P, const DevState& S, const std::vector<int32_t
     else
       launch_dense_solve_smem<T, 4>(P, S, gate, st, rec, smem);
   }
-  for (size_t l = 0; l + 1 < bw_lvl.size(); ++l) {
-    int r0 = bw_lvl[l], r1 = bw_lvl[l + 1];
-    if (r1 > r0)
-      NRPF_LAUNCH(rec, K_BWD, st,
-                  k_bwd_level<T><<<grid2(r1 - r0, 4, tiles), dim3(32, 4), 0, st>>>(P, S, r0, r1, gate));
-  }
+  if (P.n_bw_lvl > 0) launch_levels(k_subst<T, true>, K_BWD, P, S, bw_lvl.back(), P.n_bw_lvl, gate, st, rec);
 }
 
 template <typename T>

@@ -320,6 +320,59 @@ int build_plan(int n, const int32_t* rowptr, const int32_t* colidx, const double
       if (level[j] == l && (j < s || P.col_upd_ptr[j + 1] > P.col_upd_ptr[j])) P.lu_lvl_cols.push_back(j);
     P.lu_lvl_ptr[l + 1] = (int32_t)P.lu_lvl_cols.size();
   }
+  // ---- the refactorisation by entries ----
+  // (not for schedules whose lists would take gigabytes: those keep the columns)
+  if (s > 0 && P.dst.size() <= ((size_t)1 << 26) && P.NS < ((int64_t)1 << 29)) {
+    std::vector<int32_t> first((size_t)P.NS + 1, 0);  // products of each entry
+    for (int32_t d : P.dst) ++first[(size_t)d + 1];
+    for (int64_t p = 0; p < P.NS; ++p) first[p + 1] += first[p];
+    std::vector<std::pair<int32_t, int32_t>> prod(P.dst.size());
+    std::vector<int32_t> fill(first.begin(), first.end() - 1);
+    for (const Upd& u : P.upd)  // columns ascending, and k ascending within each
+      for (int q = 0; q < u.llen; ++q) prod[fill[P.dst[u.dst_off + q]]++] = {u.lsrc + q, u.ukj};
+    std::vector<int32_t> lev((size_t)P.NS, -1);  // -1: the Jacobian's value stands
+    std::vector<int32_t> col((size_t)P.NS);
+    int nl = 0;
+    for (int j = 0; j < m; ++j)
+      for (int64_t p = P.cs[j]; p < P.ce[j]; ++p) {
+        col[p] = j;
+        int32_t l = -1;
+        for (int32_t q = first[p]; q < first[p + 1]; ++q)
+          l = std::max(l, std::max(lev[prod[q].first], lev[prod[q].second]) + 1);
+        if (j < s && p == P.dp[j]) l = std::max(l, 0);
+        if (j < s && p > P.dp[j]) l = std::max(l, lev[P.dp[j]] + 1);
+        lev[p] = l;
+        nl = std::max(nl, l + 1);
+      }
+    std::vector<std::vector<int32_t>> at(nl);
+    for (int64_t p = 0; p < P.NS; ++p)
+      if (lev[p] >= 0) at[lev[p]].push_back((int32_t)p);
+    constexpr int kTaskOps = 16;  // short entries share a task up to this many operations
+    P.fac_lvl_ptr.assign(1, 0);
+    P.fac_task.assign(1, 0);
+    for (auto& es : at) {
+      auto ops = [&](int32_t p) { return 1 + first[p + 1] - first[p]; };
+      std::stable_sort(es.begin(), es.end(), [&](int32_t a, int32_t b) { return ops(a) > ops(b); });
+      int used = 0;
+      for (int32_t p : es) {
+        if (used > 0 && used + ops(p) > kTaskOps) {
+          P.fac_task.push_back((int32_t)(P.fac_op.size() / 2));
+          used = 0;
+        }
+        const int j = col[p];
+        const int kind = j >= s || p < P.dp[j] ? 1 : p == P.dp[j] ? 3 : 2;
+        P.fac_op.push_back((p << 2) | kind);
+        P.fac_op.push_back(j);
+        for (int32_t q = first[p]; q < first[p + 1]; ++q) {
+          P.fac_op.push_back(prod[q].first << 2);
+          P.fac_op.push_back(prod[q].second);
+        }
+        used += ops(p);
+      }
+      if (used > 0) P.fac_task.push_back((int32_t)(P.fac_op.size() / 2));
+      P.fac_lvl_ptr.push_back((int32_t)P.fac_task.size() - 1);
+    }
+  }
   // rows of each Schur task's chunk that hold a Jacobian entry
   if (P.nd > 0) {
     const int nch = (P.ndp + 31) / 32;

@@ -45,6 +45,17 @@ struct HostPlan {
   std::vector<int32_t> col_upd_ptr;              // [m+1] into upd
   std::vector<Upd> upd;
   std::vector<int32_t> dst;
+  // ---- the same refactorisation by entries (empty: too large, see plan.cpp) ----
+  // Every entry (i, j) of the sparse segments that changes is A(i, j) minus its
+  // products L(i, k) U(k, j), ascending k, then (L entries) times the inverse
+  // pivot of column j.  Entries depend on entries, not on columns, so a level
+  // holds all that can be computed at once.  A task is one entry or a few short
+  // ones, as a run of operations fac_op[2q], fac_op[2q+1]:
+  //   (position << 2 | kind, j): begins an entry, kind 1 U, 2 L, 3 diagonal
+  //   (position of L(i, k) << 2, position of U(k, j)): a product of it
+  std::vector<int32_t> fac_lvl_ptr;  // [levels+1] into the tasks
+  std::vector<int32_t> fac_task;     // [tasks+1] into the operations
+  std::vector<int32_t> fac_op;
   // ---- Schur complement of the sparse columns into the dense block ----
   // The updates of a dense column j by sparse columns k keep only their rows
   // < s in the level schedule (they finish U(k, j)); the rows >= s are applied
