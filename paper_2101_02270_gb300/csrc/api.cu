@@ -16,6 +16,7 @@
 #include "handle.h"
 #include "kernels.h"
 #include "plan.h"
+#include "small_solve.h"
 
 using nrpf::DevPlan;
 using nrpf::DevState;
@@ -155,11 +156,16 @@ void enqueue_body(pf_plan* p, const DevState& S, cudaStream_t st, nrpf::Recorder
   const HostPlan& h = p->hp;
   const int32_t* prev = nrpf::ctl_prev(S);
   const int32_t* cur = nrpf::ctl_cur(S);
-  nrpf::launch_prepare_lu<T>(P, S, prev, st, rec, false);
+  const bool small = P.n_sm_lvl > 0;  // one kernel for the whole linear solve
+  nrpf::launch_prepare_lu<T>(P, S, prev, st, rec, small);
   nrpf::launch_mismatch<T>(P, S, 1, prev, st, rec);
   nrpf::launch_check(S, st, rec);
-  nrpf::launch_factor<T>(P, S, h.lu_lvl_ptr, cur, st, rec);
-  nrpf::launch_solve<T>(P, S, h.fw_lvl_ptr, h.bw_lvl_ptr, cur, st, rec);
+  if (small) {
+    nrpf::launch_small_solve<T>(P, S, cur, st, rec);
+  } else {
+    nrpf::launch_factor<T>(P, S, h.lu_lvl_ptr, cur, st, rec);
+    nrpf::launch_solve<T>(P, S, h.fw_lvl_ptr, h.bw_lvl_ptr, cur, st, rec);
+  }
   nrpf::launch_update<T>(P, S, cur, st, rec);
   nrpf::launch_iter_tail(S, cond, graph, st, rec);
 }
@@ -476,6 +482,18 @@ int pf_plan_create(int n, const int32_t* rowptr, const int32_t* colidx, const do
     d.fac_op = reinterpret_cast<const int2*>(ops);
     d.n_fac_lvl = std::max((int)h.fac_lvl_ptr.size() - 1, 0);
     d.n_fac_task = std::max((int)h.fac_task.size() - 1, 0);
+    // the whole-solve schedule, where eight instances' values fit in this precision
+    if (nrpf::small_solve_fits(h, p->lu_precision == NRPF_LU_FP32 ? 4 : 8)) {
+      if ((rc = upload(p, h.sm_lvl_ptr, &d.sm_lvl_ptr)) || (rc = upload(p, h.sm_task, &d.sm_task)) ||
+          (rc = upload(p, h.sm_op, &ops))) {
+        pf_plan_destroy(p);
+        return rc;
+      }
+      d.sm_op = reinterpret_cast<const int2*>(ops);
+      d.n_sm_lvl = (int)h.sm_lvl_ptr.size() - 1;
+      d.n_sm_task = (int)h.sm_task.size() - 1;
+      d.n_sm_op = (int)(h.sm_op.size() / 2);
+    }
     d.n_schur = (int)(h.schur_task.size() / 4);
   }
   if (o.max_batch > 0 && (rc = ensure_capacity(p, o.max_batch))) {

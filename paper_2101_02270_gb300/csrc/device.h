@@ -14,6 +14,17 @@ namespace nrpf {
 // (float64) or 128-byte (float32) segment.
 constexpr int kTile = 32;
 
+// Layout of the dense block inside a tile's LU array.  FP64: element (r, c)
+// of the ndp x ndp block at (c * ndp + r) * 32 + lane.  FP32: four
+// consecutive rows of a column stay together per lane,
+// (c * ndp + (r & ~3)) * 32 + lane * 4 + (r & 3), so a lane reads rows
+// r..r+3 (r % 4 == 0) as one 16-byte vector and a warp's access is still one
+// contiguous 512-byte segment.  ndp is a multiple of the panel width (>= 4).
+template <typename T>
+struct DenseGroup {
+  static constexpr int G = sizeof(T) == 4 ? 4 : 1;
+};
+
 struct DevUpd {
   int32_t ukj, lsrc, llen, dst_off;
 };
@@ -53,6 +64,11 @@ struct DevPlan {
   const int32_t* schur_u;     // U(k, j) position of the entry
   const uint32_t* schur_jmask; // rows of the chunk holding a Jacobian entry
   int n_schur;
+  // the whole linear solve of a small plan (plan.h; n_sm_lvl = 0: not small)
+  const int32_t* sm_lvl_ptr;
+  const int32_t* sm_task;
+  const int2* sm_op;
+  int n_sm_lvl, n_sm_task, n_sm_op;
   // FS/BS
   const int32_t* fw_rows; const int32_t* fw_ptr; const int32_t* fw_pos; const int32_t* fw_col;
   const int32_t* bw_rows; const int32_t* bw_ptr; const int32_t* bw_pos; const int32_t* bw_col;
@@ -100,5 +116,19 @@ struct DevState {
   const double2* yv;  // [nnzY] per-instance Ybus values (re, im), or null: the plan's shared values
   const void* im_maps;  // host pointer to the workspace's DenseImMaps (instance-major plans), never read on the device
 };
+
+// offset of LU position p of lane `lane` within its tile's array (positions
+// >= NS are in the dense block: interleaved, grouped by four rows in FP32, or
+// instance-major when P.dim is set, lane l's block then at NS * 32 + l * ndp^2)
+template <typename T>
+__device__ __forceinline__ size_t lu_off(const DevPlan& P, int64_t p, int lane) {
+  constexpr int G = DenseGroup<T>::G;
+  const int64_t NS = P.NS;
+  if (p < NS) return (size_t)p * kTile + lane;
+  const int64_t q = p - NS;
+  if (P.dim) return (size_t)NS * kTile + (size_t)lane * (size_t)P.ndp * (size_t)P.ndp + (size_t)q;
+  if (G == 1) return (size_t)p * kTile + lane;
+  return (size_t)NS * kTile + (size_t)(q & ~(int64_t)(G - 1)) * kTile + (size_t)lane * G + (size_t)(q & (G - 1));
+}
 
 }  // namespace nrpf

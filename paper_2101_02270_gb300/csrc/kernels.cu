@@ -22,35 +22,10 @@ __device__ __forceinline__ bool tile_active(const DevState& S, int tile, int lan
   return __any_sync(0xffffffffu, S.active[tile * kTile + lane] != 0);
 }
 
-// Layout of the dense block inside a tile's LU array.  FP64: element (r, c)
-// of the ndp x ndp block at (c * ndp + r) * 32 + lane.  FP32: four
-// consecutive rows of a column stay together per lane,
-// (c * ndp + (r & ~3)) * 32 + lane * 4 + (r & 3), so a lane reads rows
-// r..r+3 (r % 4 == 0) as one 16-byte vector and a warp's access is still one
-// contiguous 512-byte segment.  ndp is a multiple of the panel width (>= 4).
-template <typename T>
-struct DenseGroup {
-  static constexpr int G = sizeof(T) == 4 ? 4 : 1;
-};
-
 template <typename T>
 __device__ __forceinline__ size_t dense_off(int r, int c, int ld, int lane) {
   constexpr int G = DenseGroup<T>::G;
   return ((size_t)c * ld + (r & ~(G - 1))) * kTile + (size_t)lane * G + (r & (G - 1));
-}
-
-// offset of LU position p of lane `lane` within its tile's array (positions
-// >= NS are in the dense block: interleaved, grouped by four rows in FP32, or
-// instance-major when P.dim is set, lane l's block then at NS * 32 + l * ndp^2)
-template <typename T>
-__device__ __forceinline__ size_t lu_off(const DevPlan& P, int64_t p, int lane) {
-  constexpr int G = DenseGroup<T>::G;
-  const int64_t NS = P.NS;
-  if (p < NS) return (size_t)p * kTile + lane;
-  const int64_t q = p - NS;
-  if (P.dim) return (size_t)NS * kTile + (size_t)lane * (size_t)P.ndp * (size_t)P.ndp + (size_t)q;
-  if (G == 1) return (size_t)p * kTile + lane;
-  return (size_t)NS * kTile + (size_t)(q & ~(int64_t)(G - 1)) * kTile + (size_t)lane * G + (size_t)(q & (G - 1));
 }
 
 // ---------------------------------------------------------------------------
@@ -141,14 +116,16 @@ __global__ void k_store(DevPlan P, DevState S, int B, double2* __restrict__ v_ou
 //   dP_i/d|V_k| = Re W_ik / |V_k|, dQ_i/d|V_k| = Im W_ik / |V_k|
 //   dP_i/dth_i = -Q_i - B_ii |V_i|^2,  dQ_i/dth_i = P_i - G_ii |V_i|^2
 //   dP_i/d|V_i| = P_i/|V_i| + G_ii |V_i|, dQ_i/d|V_i| = Q_i/|V_i| - B_ii |V_i|
-// Block: 32 lanes x kWarps warps; each warp walks kBusPerWarp buses.
+// Block: 32 lanes x kWarps warps; each warp walks `per` buses, eight, which
+// amortises the block's reduction, or fewer while that fills the GPU: a bus is a
+// chain of index, value and FP64 arithmetic, 4 us of it, so that eight in a row
+// took 33 us on 30 buses and 66 us on one tile of 2,000 (now 11 and 18 us).
 // The right-hand side receives -F at the permuted row of each equation.
 // ---------------------------------------------------------------------------
 constexpr int kMWarps = 8;
-constexpr int kBusPerWarp = 8;
 
 template <typename T>
-__global__ void __launch_bounds__(32 * kMWarps) k_mismatch_jac(DevPlan P, DevState S, int jac,
+__global__ void __launch_bounds__(32 * kMWarps) k_mismatch_jac(DevPlan P, DevState S, int jac, int per,
                                                                const int32_t* __restrict__ gate) {
   __shared__ double red[kMWarps][32];
   const int lane = threadIdx.x, warp = threadIdx.y;
@@ -173,8 +150,8 @@ __global__ void __launch_bounds__(32 * kMWarps) k_mismatch_jac(DevPlan P, DevSta
     }
   };
   double nrm = 0.0;
-  const int ibeg = (blockIdx.x * kMWarps + warp) * kBusPerWarp;
-  for (int ii = 0; ii < kBusPerWarp; ++ii) {
+  const int ibeg = (blockIdx.x * kMWarps + warp) * per;
+  for (int ii = 0; ii < per; ++ii) {
     const int i = ibeg + ii;
     if (i >= P.n) break;
     const int bt = P.bus_type[i];
@@ -1350,8 +1327,12 @@ void launch_store(const DevPlan& P, const DevState& S, int B, double* v_out, int
 template <typename T>
 void launch_mismatch(const DevPlan& P, const DevState& S, int jac, const int32_t* gate, cudaStream_t st,
                      Recorder* rec) {
-  dim3 g((P.n + kMWarps * kBusPerWarp - 1) / (kMWarps * kBusPerWarp), S.Bp / kTile);
-  NRPF_LAUNCH(rec, K_MISMATCH, st, k_mismatch_jac<T><<<g, dim3(32, kMWarps), 0, st>>>(P, S, jac, gate));
+  const int tiles = S.Bp / kTile;
+  auto blocks = [&](int per) { return (P.n + kMWarps * per - 1) / (kMWarps * per); };
+  int per = 8;
+  while (per > 1 && (int64_t)blocks(per) * tiles < 4 * 152) per /= 2;
+  NRPF_LAUNCH(rec, K_MISMATCH, st,
+              k_mismatch_jac<T><<<dim3(blocks(per), tiles), dim3(32, kMWarps), 0, st>>>(P, S, jac, per, gate));
 }
 
 void launch_load_y(const DevPlan& P, const DevState& S, int B, const double* y, cudaStream_t st, Recorder* rec) {

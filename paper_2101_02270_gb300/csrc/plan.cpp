@@ -390,6 +390,90 @@ int build_plan(int n, const int32_t* rowptr, const int32_t* colidx, const double
   }
   P.lu_fma = fma;
 
+  // ---- the whole linear solve by entries ----
+  // for plans whose values, of eight instances in the smaller precision, fit the
+  // shared memory of a CTA
+  const int64_t nval = P.NS + (int64_t)P.nd * P.nd + 2 * (int64_t)m;
+  if (m > 0 && nval <= kSmallValues) {
+    // value index of (r, c), and the structure of each column below the diagonal
+    // (by symmetry also of each row of U right of it)
+    auto at = [&](int r, int c) -> int32_t {
+      if (r >= s && c >= s) return (int32_t)(P.NS + (int64_t)(c - s) * P.nd + (r - s));
+      return (int32_t)P.pos(r, c);
+    };
+    auto below = [&](int k) {
+      std::vector<int> v;
+      if (k < s) v = Lpat[k];
+      else for (int r = k + 1; r < m; ++r) v.push_back(r);
+      return v;
+    };
+    const int32_t vx = (int32_t)(P.NS + (int64_t)P.nd * P.nd), vd = vx + m;
+    struct Entry {
+      int32_t value, kind, col, level;
+      std::vector<std::pair<int32_t, int32_t>> prod;
+    };
+    std::vector<Entry> es;
+    std::vector<int32_t> of(nval, -1);  // entry that forms a value
+    std::vector<std::vector<std::pair<int32_t, int32_t>>> prod(vd);
+    std::vector<std::vector<int>> str(m);
+    for (int k = 0; k < m; ++k) {
+      str[k] = below(k);
+      for (int i : str[k]) {
+        const int32_t l = at(i, k);
+        for (int j : str[k]) {
+          const int32_t p = at(i, j);
+          if (p < 0) { err = "internal: fill pattern not closed"; return NRPF_ERR_PATTERN; }
+          prod[p].push_back({l, at(k, j)});
+        }
+        prod[vx + i].push_back({l, vx + k});
+      }
+    }
+    auto level_of = [&](int32_t v) { return of[v] < 0 ? -1 : es[of[v]].level; };
+    auto add = [&](int32_t value, int kind, int32_t col, std::vector<std::pair<int32_t, int32_t>> pr) {
+      int l = of[value] >= 0 ? es[of[value]].level : -1;  // backward: after the forward value
+      for (auto& q : pr) l = std::max(l, std::max(level_of(q.first), level_of(q.second)));
+      if (kind == 2) l = std::max(l, level_of(col));
+      of[value] = (int32_t)es.size();
+      if (kind == 3) of[col] = of[value];
+      es.push_back(Entry{value, kind, col, l + 1, std::move(pr)});
+    };
+    for (int j = 0; j < m; ++j) {
+      // column j: U and diagonal in ascending rows, then L; then the right-hand
+      // side's entry j
+      for (int k = 0; k < j; ++k) {
+        const int32_t p = at(k, j);
+        if (p >= 0 && !prod[p].empty()) add(p, 1, 0, std::move(prod[p]));
+      }
+      add(at(j, j), 3, vd + j, std::move(prod[at(j, j)]));
+      for (int i : str[j]) add(at(i, j), 2, vd + j, std::move(prod[at(i, j)]));
+      if (!prod[vx + j].empty()) add(vx + j, 1, 0, std::move(prod[vx + j]));
+    }
+    for (int i = m - 1; i >= 0; --i) {
+      std::vector<std::pair<int32_t, int32_t>> pr;
+      for (int j : str[i]) pr.push_back({at(i, j), vx + j});
+      add(vx + i, 2, vd + i, std::move(pr));
+    }
+    int nl = 0;
+    for (auto& e : es) nl = std::max(nl, e.level + 1);
+    std::vector<std::vector<int>> by(nl);
+    for (size_t e = 0; e < es.size(); ++e) by[es[e].level].push_back((int)e);
+    P.sm_lvl_ptr.assign(1, 0);
+    P.sm_task.assign(1, 0);
+    for (auto& v : by) {
+      std::stable_sort(v.begin(), v.end(), [&](int a, int b) { return es[a].prod.size() > es[b].prod.size(); });
+      for (int e : v) {
+        P.sm_op.push_back((es[e].value << 2) | es[e].kind);
+        P.sm_op.push_back(es[e].col);
+        for (auto& q : es[e].prod) {
+          P.sm_op.push_back(q.first << 2);
+          P.sm_op.push_back(q.second);
+        }
+        P.sm_task.push_back((int32_t)(P.sm_op.size() / 2));
+      }
+      P.sm_lvl_ptr.push_back((int32_t)P.sm_task.size() - 1);
+    }
+  }
+
   // ---- forward substitution (unit L), rows by level; all rows gather the
   //      contributions of sparse columns, the dense block follows ----
   {

@@ -16,6 +16,10 @@ struct Upd {
   int32_t dst_off;  // offset into HostPlan::dst
 };
 
+// Values per instance up to which a plan gets the whole-solve schedule: eight
+// instances in FP32 then take 200 KB of shared memory.
+constexpr int64_t kSmallValues = 6400;
+
 struct HostPlan {
   // ---- problem ----
   int n = 0, m = 0, npv = 0, npq = 0, nslack = 0;
@@ -56,6 +60,13 @@ struct HostPlan {
   std::vector<int32_t> fac_lvl_ptr;  // [levels+1] into the tasks
   std::vector<int32_t> fac_task;     // [tasks+1] into the operations
   std::vector<int32_t> fac_op;
+  // ---- the whole linear solve by entries, for small plans (empty: not small) ----
+  // Values of one instance: the NS sparse positions, the nd x nd dense block
+  // (column-major, no padding), the right-hand side [m], the inverse pivots [m].
+  // Operations as above over these values, for the LU of all columns (the
+  // right-hand side is one more column: its forward substitution) and for the
+  // backward substitution (kind 2: scaled by the inverse pivot at value j).
+  std::vector<int32_t> sm_lvl_ptr, sm_task, sm_op;
   // ---- Schur complement of the sparse columns into the dense block ----
   // The updates of a dense column j by sparse columns k keep only their rows
   // < s in the level schedule (they finish U(k, j)); the rows >= s are applied

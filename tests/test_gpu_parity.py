@@ -414,3 +414,24 @@ def test_host_batch_back_to_back_calls():
     for S, o in zip((S1, S2, S1), outs):
         Vo, ito, sto = _oracle_solve(g, S, V0)
         _compare_newton(g, o[0].numpy(), o[1].numpy(), o[2].numpy(), Vo, ito, sto, S)
+
+
+@pytest.mark.parametrize("n,branches,lu", [(8, 10, "fp64"), (60, 85, "fp64"), (110, 140, "fp64"), (110, 140, "fp32"),
+                                           (170, 215, "fp32"), (260, 330, "fp32")])
+@pytest.mark.parametrize("B", [1, 33, 152 * 16 + 3])
+def test_small_plan_solve(n, branches, lu, B):
+    """Small plans solve each Newton step in one CTA's shared memory (32, 16 or 8
+    instances of it, with and without the schedule there) and the next larger
+    ones do not: voltages, iterations and status are the oracle's on sampled
+    instances of every size."""
+    import gridgen
+    g = gridgen.make_grid("mesh2000_b10k", 0, n=n, n_branch=branches, n_pv=max(1, n // 10), load_scale=1 / 16)
+    sc = gridgen.make_scenarios(g, B, 0.6, 1.4)
+    S, V0 = sc.sbus(g), sc.v0_flat(g)
+    with _plan(g, lu_precision=lu) as p:
+        v, it, st = p.solve(_dev(S), _dev(V0), TOL, 10)
+        Vg, itg, stg = v.cpu().numpy(), it.cpu().numpy(), st.cpu().numpy()
+    assert np.all(stg == 0)
+    idx = sorted({0, B // 2, B - 1})
+    Vo, ito, sto = _oracle_solve(g, S, V0, idx=idx)
+    _compare_newton(g, Vg[idx], itg[idx], stg[idx], Vo, ito, sto, S[idx], check_iters=lu == "fp64")
