@@ -123,6 +123,17 @@ int ensure_capacity(pf_plan* p, int B) {
   if (p->dp.n_fac_lvl > 0) {
     AL((size_t)h.s * Bp * w, dinv, void*);
   }
+  // Operands of the FP64 trailing update in fixed point (7 % of the workspace):
+  // where they would be the memory that is missing, the update stays in FP64
+  if (p->lu_precision == NRPF_LU_FP64 && h.kb == 8 && h.ndp > 16) {
+    void* d = nullptr;
+    if (cudaMalloc(&d, nrpf::dense_limb_bytes(p->dp, Bp)) == cudaSuccess) {
+      p->ws_allocs.push_back(d);
+      s.limb = d;
+    } else {
+      cudaGetLastError();
+    }
+  }
   AL((size_t)Bp * sizeof(unsigned long long), norm, unsigned long long*);
   AL((size_t)Bp * 4, iters, int32_t*);
   AL((size_t)Bp * 4, status, int32_t*);

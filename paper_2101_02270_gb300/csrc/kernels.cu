@@ -2,6 +2,7 @@
 // kTile = 32 interleaved instances: lane = instance within the tile, so all
 // plan indices are warp-uniform (broadcast loads) and all value accesses are
 // contiguous across the warp.
+#include <algorithm>
 #include <cfloat>
 #include <cstdint>
 #include <vector>
@@ -937,6 +938,191 @@ __global__ void __launch_bounds__(128, UpdOcc<T, TS>::value) k_dense_update(DevP
 }
 
 // ---------------------------------------------------------------------------
+// FP64 trailing update of depth 16 in integer arithmetic.  An FP64 multiply-add
+// of a warp holds its quarter of the SM for 64 cycles; a 32 x 32 + 64-bit integer
+// one (mad.wide) takes two.  The update is therefore made in fixed point:
+//  * k_dense_limbs: the 16 entries of each row of L21 become integers of 55 bits
+//    and sign, X = x 2^(1077 - E), E the largest (biased) exponent among them,
+//    rounded to nearest; likewise each column of U12.  X = hi 2^28 + lo, both
+//    signed 28 bits.
+//  * k_dense_update_fixed: sum of hi hi and of hi lo + lo hi over the 16 products
+//    in two 64-bit integers, exactly (lo lo, 2^-56 of the scale, is left out);
+//    then hh + hl / 2^28, rounded, is converted and subtracted once, C <- C - T s
+//    with the power of two s = 2^(Ea + Eb - 1075 - 1023).
+// Error of an entry: 2^-55 of the largest product of its row and column per
+// operand, against 16 roundings of 2^-53 of the entry itself by multiply-adds.
+// Backward error of staged FP64 solves, max norm |J x - b| / (|J| |x| + |b|),
+// median of 16 instances, by multiply-adds and in this form (meshed grids):
+//   buses (dense)  700 (136)  1,300 (240)  2,000 (272)  2,000 (448)  3,000 (544)
+//   multiply-adds  5.3e-17    6.4e-17      8.1e-17      1.7e-16      1.4e-16
+//   this form      4.0e-17    5.1e-17      6.2e-17      1.1e-16      9.1e-17
+// Bounds: 48 mad.wide per entry and 16 products, four cycles each on the pipe that
+// makes them (79 ms for four refactorisations of 10,000 272-wide blocks), and two
+// FP64 instructions, conversion and subtraction (53 ms); measured 121 ms, where
+// multiply-adds took 397. Loading the operands through registers instead of one
+// bulk copy per side took 138 ms; more warps per CTA were no faster.
+// A row or column with an infinity or NaN makes every entry it meets NaN.
+// ---------------------------------------------------------------------------
+constexpr int kFixK = 16;
+constexpr int kFixBad = 0x4000;  // exponent of a row with an infinity or NaN
+
+// S.limb, per tile and in groups of four rows of L21 (then of four columns of
+// U12): int4 [2][ndp/4][kFixK][2][32], a lane's int4 = (hi, lo) of two rows, so
+// that a group's operands are one run at constant offsets; then int4
+// [2][ndp/4][32], the four exponents, already at their place in an FP64's high
+// word (L21's with the bias of the product taken off).
+__host__ __device__ __forceinline__ size_t limb_vecs(int ndp) {  // int4 per tile
+  return (size_t)(ndp / 4) * 2 * kTile * (2 * kFixK + 1);
+}
+
+__global__ void __launch_bounds__(128) k_dense_limbs(DevPlan P, DevState S, int k, const int32_t* __restrict__ gate) {
+  if (gate && *gate == 0) return;
+  const int lane = threadIdx.x, tile = blockIdx.y, ld = P.ndp;
+  if (!tile_active(S, tile, lane)) return;
+  const int r0 = k + kFixK, n = ld - r0;
+  const int t = blockIdx.x * blockDim.y + threadIdx.y;
+  if (t >= 2 * n) return;
+  const bool row = t < n;
+  const int i = r0 + (row ? t : t - n), g = (row ? 0 : ld / 4) + i / 4;
+  const double* __restrict__ A = reinterpret_cast<const double*>(S.lu) + ((size_t)tile * P.NLU + P.NS) * kTile + lane;
+  int4* base = reinterpret_cast<int4*>(S.limb) + (size_t)tile * limb_vecs(ld);
+  int2* out = reinterpret_cast<int2*>(base + ((size_t)g * kFixK * 2 + (i & 2) / 2) * kTile + lane) + (i & 1);
+  int32_t* eo = reinterpret_cast<int32_t*>(base + ((size_t)(ld / 4) * 2 * kFixK * 2 + g) * kTile + lane) + (i & 3);
+  long long x[kFixK];
+  int em = 0;
+#pragma unroll
+  for (int p = 0; p < kFixK; ++p) {
+    const size_t e = row ? (size_t)(k + p) * ld + i : (size_t)i * ld + k + p;
+    x[p] = __double_as_longlong(A[e * kTile]);
+    em = max(em, (int)(x[p] >> 52) & 0x7ff);
+  }
+#pragma unroll
+  for (int p = 0; p < kFixK; ++p) {
+    const int ex = (int)(x[p] >> 52) & 0x7ff, d = em - ex;
+    const long long m = ((x[p] & 0xfffffffffffffll) | 0x10000000000000ll) << 2;
+    long long v = d == 0 ? m : (m + (1ll << (min(d, 60) - 1))) >> min(d, 60);
+    if (ex == 0) v = 0;  // zero, and what is below the normal range
+    if ((x[p] < 0) != row) v = -v;  // the rows of L21 negated: the sums are subtracted
+    const int lo = (int)((unsigned)v << 4) >> 4;
+    out[(size_t)p * 2 * kTile * 2] = make_int2((int)((v - lo) >> 28), lo);
+  }
+  // an all-zero row: any exponent that keeps the scale of a zero sum normal
+  const int e = em == 0x7ff ? kFixBad : em == 0 ? 1075 : em;
+  *eo = row ? e - 1075 : e;
+}
+
+__device__ __forceinline__ void mad_wide(long long& c, int a, int b) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
+}
+
+// A warp per 4 x 4 entries, 2 x 2 warps per CTA.  The CTA's operands, two groups of
+// rows and two of columns with all their 16 depths, are two runs of 32 KB: two bulk
+// copies bring them to shared memory, and three CTAs per SM cover each other's
+// copies, integer work and conversions.
+constexpr int kFixWR = 2, kFixWC = 2;  // warps (groups of four rows, of four columns) per CTA
+constexpr size_t kFixGroup = (size_t)kFixK * 2 * kTile * sizeof(int4);  // 16 KB
+constexpr size_t kFixSmem = (kFixWR + kFixWC) * kFixGroup;
+constexpr uint32_t kFixSpinLimit = 1u << 20;
+
+__global__ void __launch_bounds__(32 * kFixWR * kFixWC, 3) k_dense_update_fixed(DevPlan P, DevState S, int k,
+                                                               const int32_t* __restrict__ gate) {
+  extern __shared__ __align__(128) unsigned char fix_smem[];
+  __shared__ __align__(8) uint64_t bar;
+  if (gate && *gate == 0) return;
+  const int lane = threadIdx.x, w = threadIdx.y, tile = blockIdx.y, ld = P.ndp;
+  if (!tile_active(S, tile, lane)) return;  // uniform over the CTA
+  const int ng = (ld - k - kFixK) / 4, nb = (ng + kFixWR - 1) / kFixWR;  // groups of rows (and of columns)
+  const int gi0 = kFixWR * (int)(blockIdx.x % nb), gj0 = kFixWC * (int)(blockIdx.x / nb);
+  const int gi = gi0 + w % kFixWR, gj = gj0 + w / kFixWR;
+  const int g0 = (k + kFixK) / 4, G = ld / 4;
+  const int4* base = reinterpret_cast<const int4*>(S.limb) + (size_t)tile * limb_vecs(ld);
+  const uint32_t sb = static_cast<uint32_t>(__cvta_generic_to_shared(&bar));
+  const uint32_t sm = static_cast<uint32_t>(__cvta_generic_to_shared(fix_smem));
+  if (lane == 0 && w == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sb) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    const uint32_t na = (uint32_t)(min(kFixWR, ng - gi0) * kFixGroup), nbt = (uint32_t)(min(kFixWC, ng - gj0) * kFixGroup);
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sb), "r"(na + nbt) : "memory");
+    auto copy = [&](uint32_t dst, const int4* src, uint32_t bytes) {
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                   "l"(src), "r"(bytes), "r"(sb)
+                   : "memory");
+    };
+    copy(sm, base + (size_t)(g0 + gi0) * kFixK * 2 * kTile, na);
+    copy(sm + kFixWR * (uint32_t)kFixGroup, base + (size_t)(G + g0 + gj0) * kFixK * 2 * kTile, nbt);
+  }
+  const bool mine = gi < ng && gj < ng;
+  int4 ea = make_int4(0, 0, 0, 0), eb = ea;
+  double c[4][4];
+  double* __restrict__ C = reinterpret_cast<double*>(S.lu) +
+                           ((size_t)tile * P.NLU + P.NS + (size_t)(4 * (g0 + gj)) * ld + 4 * (g0 + gi)) * kTile + lane;
+  if (mine) {
+    ea = base[((size_t)2 * G * kFixK * 2 + g0 + gi) * kTile + lane];
+    eb = base[((size_t)2 * G * kFixK * 2 + G + g0 + gj) * kTile + lane];
+  }
+  long long hh[4][4], hl[4][4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      hh[r][q] = 0;
+      hl[r][q] = 1ll << 27;  // rounds hl / 2^28
+    }
+  __syncthreads();  // the barrier is initialised
+  uint32_t ok = 0;
+  for (uint32_t spins = 0; !ok && spins < kFixSpinLimit; ++spins)
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(sb)
+        : "memory");
+  if (__syncthreads_or(!ok)) {  // a copy did not land in time: the step is discarded
+    S.bad[tile * kTile + lane] = 1;
+    return;
+  }
+  if (!mine) return;
+  const int4* la = reinterpret_cast<const int4*>(fix_smem + (w % kFixWR) * kFixGroup) + lane;
+  const int4* lb = reinterpret_cast<const int4*>(fix_smem + (kFixWR + w / kFixWR) * kFixGroup) + lane;
+#pragma unroll
+  for (int p = 0; p < kFixK; ++p) {
+    const int4 a[2] = {la[(2 * p) * kTile], la[(2 * p + 1) * kTile]};
+    const int4 b[2] = {lb[(2 * p) * kTile], lb[(2 * p + 1) * kTile]};
+    const int ah[4] = {a[0].x, a[0].z, a[1].x, a[1].z}, al[4] = {a[0].y, a[0].w, a[1].y, a[1].w};
+    const int bh[4] = {b[0].x, b[0].z, b[1].x, b[1].z}, bl[4] = {b[0].y, b[0].w, b[1].y, b[1].w};
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        mad_wide(hh[r][q], ah[r], bh[q]);
+        mad_wide(hl[r][q], ah[r], bl[q]);
+      }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) mad_wide(hl[r][q], al[r], bh[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) c[r][q] = C[((size_t)q * ld + r) * kTile];
+  const int er[4] = {ea.x, ea.y, ea.z, ea.w}, ec[4] = {eb.x, eb.y, eb.z, eb.w};
+  // the scales are normal numbers unless values are near FP64's limits
+  const int lo = min(min(er[0], er[1]), min(er[2], er[3])) + min(min(ec[0], ec[1]), min(ec[2], ec[3]));
+  const int hi = max(max(er[0], er[1]), max(er[2], er[3])) + max(max(ec[0], ec[1]), max(ec[2], ec[3]));
+  const bool normal = lo > 0 && hi < 2047;
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const long long t = hh[r][q] + (hl[r][q] >> 28);
+      const int e = er[r] + ec[q];
+      int s = e << 20;
+      if (!normal) s = e >= 2047 ? (e >= kFixBad - 1075 ? 0x7ff80000 : 0x7ff00000) : e <= 0 ? 0 : s;
+      C[((size_t)q * ld + r) * kTile] = fma((double)t, __hiloint2double(s, 0), c[r][q]);
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Forward / backward substitution (Sec. 4.3.3).  Row-oriented gathers per
 // level instead of the paper's atomicAdd scatter: every row writes only its
 // own entry, so the result is deterministic.
@@ -1475,6 +1661,31 @@ void launch_factor(const DevPlan& P, const DevState& S, const std::vector<int32_
       return;
     }
   }
+  if constexpr (sizeof(T) == 8) {
+    if (S.limb && P.kb == 8) {
+      // two panels of eight, then one trailing update of depth 16
+      static bool configured[64] = {};
+      int dev = 0;
+      cudaGetDevice(&dev);
+      if (dev < 0 || dev >= 64 || !configured[dev]) {
+        cudaFuncSetAttribute(k_dense_update_fixed, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
+        if (dev >= 0 && dev < 64) configured[dev] = true;
+      }
+      for (int k = 0; k < P.ndp; k += kFixK) {
+        const int rest = P.ndp - k - kFixK, kend = std::min(k + kFixK, P.ndp);
+        for (int ki = k; ki < kend; ki += 8) launch_dense_step<T, 8>(P, S, ki, kend, P.ndp, gate, st, rec);
+        if (rest <= 0) continue;
+        NRPF_LAUNCH(rec, K_DENSE_UPDATE, st,
+                    k_dense_limbs<<<grid2(2 * rest, 4, tiles), dim3(32, 4), 0, st>>>(P, S, k, gate));
+        NRPF_LAUNCH(rec, K_DENSE_UPDATE, st,
+                    k_dense_update_fixed<<<dim3((unsigned)(((rest / 4 + kFixWR - 1) / kFixWR) *
+                                                           ((rest / 4 + kFixWC - 1) / kFixWC)),
+                                                (unsigned)tiles),
+                                           dim3(32, kFixWR * kFixWC), kFixSmem, st>>>(P, S, k, gate));
+      }
+      return;
+    }
+  }
   for (int k = 0; k < P.ndp; k += P.kb) {
     if (P.kb == 4) launch_dense_step<T, 4>(P, S, k, P.ndp, P.ndp, gate, st, rec);
     else if (P.kb == 8) launch_dense_step<T, 8>(P, S, k, P.ndp, P.ndp, gate, st, rec);
@@ -1483,6 +1694,8 @@ void launch_factor(const DevPlan& P, const DevState& S, const std::vector<int32_
     else launch_dense_outer<T, 64>(P, S, k, gate, st, rec);
   }
 }
+
+size_t dense_limb_bytes(const DevPlan& P, int Bp) { return limb_vecs(P.ndp) * sizeof(int4) * (size_t)(Bp / kTile); }
 
 // Dense solve with the tile's right-hand side in shared memory, when it fits.
 constexpr size_t kSolveSmemMax = 200 * 1024;

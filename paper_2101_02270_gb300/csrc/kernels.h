@@ -71,6 +71,9 @@ template <typename T>
 // identity padding of the dense block.
 void launch_prepare_lu(const DevPlan& P, const DevState& S, const int32_t* gate, cudaStream_t st,
                        Recorder* rec = nullptr, bool whole = true);
+// Bytes of S.limb, the fixed-point operands of the FP64 trailing update, for a
+// workspace of Bp instances.
+size_t dense_limb_bytes(const DevPlan& P, int Bp);
 template <typename T>
 void launch_factor(const DevPlan& P, const DevState& S, const std::vector<int32_t>& lvl_ptr,
                    const int32_t* gate, cudaStream_t st, Recorder* rec = nullptr);
