@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/nrpf.h"
+#include "dense_cluster.h"
 #include "device.h"
 #include "handle.h"
 #include "kernels.h"
@@ -174,8 +175,9 @@ void enqueue_body(pf_plan* p, const DevState& S, cudaStream_t st, nrpf::Recorder
   if (small) {
     nrpf::launch_small_solve<T>(P, S, cur, st, rec);
   } else {
-    nrpf::launch_factor<T>(P, S, h.lu_lvl_ptr, cur, st, rec);
-    nrpf::launch_solve<T>(P, S, h.fw_lvl_ptr, h.bw_lvl_ptr, cur, st, rec);
+    const bool dense = !nrpf::dense_cluster_fits(P, S, sizeof(T));
+    nrpf::launch_factor<T>(P, S, h.lu_lvl_ptr, cur, st, rec, dense);
+    nrpf::launch_solve<T>(P, S, h.fw_lvl_ptr, h.bw_lvl_ptr, cur, st, rec, dense);
   }
   nrpf::launch_update<T>(P, S, cur, st, rec);
   nrpf::launch_iter_tail(S, cond, graph, st, rec);

@@ -7,6 +7,7 @@
 #include <cstdint>
 #include <vector>
 
+#include "dense_cluster.h"
 #include "dense_im.h"
 #include "device.h"
 #include "kernels.h"
@@ -1641,7 +1642,7 @@ static void launch_levels(K kernel, int cls, const DevPlan& P, const DevState& S
 
 template <typename T>
 void launch_factor(const DevPlan& P, const DevState& S, const std::vector<int32_t>& lvl_ptr,
-                   const int32_t* gate, cudaStream_t st, Recorder* rec) {
+                   const int32_t* gate, cudaStream_t st, Recorder* rec, bool dense) {
   const int tiles = S.Bp / kTile;
   if (P.n_fac_lvl > 0 && (sizeof(T) == 4 || tiles <= 152))
     launch_levels(k_sparse_factor<T>, K_LU_SPARSE, P, S, P.n_fac_task, P.n_fac_lvl, gate, st, rec);
@@ -1655,6 +1656,7 @@ void launch_factor(const DevPlan& P, const DevState& S, const std::vector<int32_
   if (P.n_schur > 0)
     NRPF_LAUNCH(rec, K_SCHUR, st,
                 k_schur<T><<<grid2(P.n_schur, kSchurWarps, tiles), dim3(32, kSchurWarps), 0, st>>>(P, S, gate));
+  if (!dense) return;
   if constexpr (sizeof(T) == 4) {
     if (P.dim) {
       if (P.ndp > 0) launch_dense_im_factor(P, S, *reinterpret_cast<const DenseImMaps*>(S.im_maps), gate, st, rec);
@@ -1730,9 +1732,12 @@ static void launch_dense_solve_smem(const DevPlan& P, const DevState& S, const i
 
 template <typename T>
 void launch_solve(const DevPlan& P, const DevState& S, const std::vector<int32_t>& fw_lvl,
-                  const std::vector<int32_t>& bw_lvl, const int32_t* gate, cudaStream_t st, Recorder* rec) {
+                  const std::vector<int32_t>& bw_lvl, const int32_t* gate, cudaStream_t st, Recorder* rec,
+                  bool dense) {
   if (P.n_fw_lvl > 0) launch_levels(k_subst<T, false>, K_FWD, P, S, fw_lvl.back(), P.n_fw_lvl, gate, st, rec);
-  if (sizeof(T) == 4 && P.dim) {
+  if (!dense) {
+    launch_dense_cluster<T>(P, S, gate, st, rec);
+  } else if (sizeof(T) == 4 && P.dim) {
     if (P.ndp > 0) launch_dense_im_solve(P, S, gate, st, rec);
   } else if (P.ndp > 0) {
     const size_t smem = (size_t)P.ndp * kTile * sizeof(T);
@@ -1777,9 +1782,9 @@ void launch_lu_out(const DevPlan& P, const DevState& S, int B, const int64_t* ma
   template void launch_prepare_lu<T>(const DevPlan&, const DevState&, const int32_t*, cudaStream_t,          \
                                      Recorder*, bool);                                                       \
   template void launch_factor<T>(const DevPlan&, const DevState&, const std::vector<int32_t>&,               \
-                                 const int32_t*, cudaStream_t, Recorder*);                                   \
+                                 const int32_t*, cudaStream_t, Recorder*, bool);                             \
   template void launch_solve<T>(const DevPlan&, const DevState&, const std::vector<int32_t>&,                \
-                                const std::vector<int32_t>&, const int32_t*, cudaStream_t, Recorder*);       \
+                                const std::vector<int32_t>&, const int32_t*, cudaStream_t, Recorder*, bool); \
   template void launch_update<T>(const DevPlan&, const DevState&, const int32_t*, cudaStream_t, Recorder*);  \
   template void launch_rhs_in<T>(const DevPlan&, const DevState&, int, const double*, cudaStream_t);         \
   template void launch_rhs_out<T>(const DevPlan&, const DevState&, int, double*, cudaStream_t);              \

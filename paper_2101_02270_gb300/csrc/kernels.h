@@ -74,13 +74,16 @@ void launch_prepare_lu(const DevPlan& P, const DevState& S, const int32_t* gate,
 // Bytes of S.limb, the fixed-point operands of the FP64 trailing update, for a
 // workspace of Bp instances.
 size_t dense_limb_bytes(const DevPlan& P, int Bp);
+// dense = false: the sparse part and the Schur tasks only.
 template <typename T>
 void launch_factor(const DevPlan& P, const DevState& S, const std::vector<int32_t>& lvl_ptr,
-                   const int32_t* gate, cudaStream_t st, Recorder* rec = nullptr);
+                   const int32_t* gate, cudaStream_t st, Recorder* rec = nullptr, bool dense = true);
+// dense = false: the dense block is factorised and solved between the levels, by
+// a cluster of CTAs per instance (dense_cluster.h).
 template <typename T>
 void launch_solve(const DevPlan& P, const DevState& S, const std::vector<int32_t>& fw_lvl,
                   const std::vector<int32_t>& bw_lvl, const int32_t* gate, cudaStream_t st,
-                  Recorder* rec = nullptr);
+                  Recorder* rec = nullptr, bool dense = true);
 template <typename T>
 void launch_update(const DevPlan& P, const DevState& S, const int32_t* gate, cudaStream_t st,
                    Recorder* rec = nullptr);

@@ -462,3 +462,29 @@ def test_fp64_update_in_fixed_point(n, branches, spread):
         J = permuted_dense(colptr, rowidx, A[k], m)[np.ix_(pos, pos)]
         r = np.abs(J @ x[k] - b[k]).max()
         assert r <= 1e-14 * (np.abs(J).sum(1).max() * np.abs(x[k]).max() + np.abs(b[k]).max()), r
+
+
+@pytest.mark.parametrize("n,branches,lu,kw", [(260, 330, "fp64", {}), (260, 330, "fp64", {"panel": 16}),
+                                              (420, 590, "fp64", {}), (420, 590, "fp32", {}),
+                                              (420, 590, "fp32", {"dense_layout": "instance_major"}),
+                                              (420, 590, "fp32", {"panel": 8}), (1500, 2000, "fp64", {})])
+@pytest.mark.parametrize("B", [1, 33, 64, 65])
+def test_dense_block_by_clusters(n, branches, lu, kw, B):
+    """Up to two tiles, the dense block is factorised and solved by a cluster of
+    CTAs per instance: blocks of a few to many columns for the eight CTAs, every
+    storage of the block, and the first batch beyond, against the oracle; an
+    instance with a NaN injection fails alone."""
+    import gridgen
+    g = gridgen.make_grid("mesh2000_b10k", 0, n=n, n_branch=branches, n_pv=n // 10, load_scale=1 / 16)
+    sc = gridgen.make_scenarios(g, B, 0.6, 1.4)
+    S, V0 = sc.sbus(g), sc.v0_flat(g)
+    bad = B - 2 if B > 2 else -1
+    if bad >= 0:
+        S[bad, 5] = np.nan
+    with _plan(g, lu_precision=lu, **kw) as p:
+        v, it, st = p.solve(_dev(S), _dev(V0), TOL, 10)
+        Vg, itg, stg = v.cpu().numpy(), it.cpu().numpy(), st.cpu().numpy()
+    assert np.array_equal(np.flatnonzero(stg), [bad] if bad >= 0 else []) and (bad < 0 or stg[bad] == 2)
+    idx = sorted({0, B // 2, B - 1})
+    Vo, ito, sto = _oracle_solve(g, S, V0, idx=idx)
+    _compare_newton(g, Vg[idx], itg[idx], stg[idx], Vo, ito, sto, S[idx], check_iters=lu == "fp64")
