@@ -360,11 +360,10 @@ __global__ void k_set_ones(DevPlan P, DevState S, const int32_t* __restrict__ ga
   T* X = reinterpret_cast<T*>(S.x) + (size_t)tile * P.mp * kTile;
   // padding columns nd .. ndp-1 of the dense block: whole identity columns
   // (the refactorisation does not zero the dense block)
-  for (int q = threadIdx.y; q < P.n_one * P.ndp; q += blockDim.y) {
-    const int t = q / P.ndp, r = q % P.ndp;
+  const int t = blockIdx.x;  // a block per padding column
+  for (int r = threadIdx.y; r < P.ndp; r += blockDim.y)
     LU[lu_off<T>(P, P.NS + (int64_t)(P.nd + t) * P.ndp + r, lane)] = (T)(r == P.nd + t ? 1 : 0);
-  }
-  for (int t = threadIdx.y; t < P.n_one; t += blockDim.y) X[(size_t)(P.m + t) * kTile + lane] = (T)0;
+  if (threadIdx.y == 0) X[(size_t)(P.m + t) * kTile + lane] = (T)0;
 }
 
 // ---------------------------------------------------------------------------
@@ -699,6 +698,53 @@ __global__ void k_dense_diag(DevPlan P, DevState S, int k, const int32_t* __rest
   for (int c = 0; c < KB; ++c)
 #pragma unroll
     for (int r = 0; r < KB; ++r) A[dense_off<T>(k + r, k + c, ld, lane)] = D[r][c];
+}
+
+// The 16 x 16 block (the step of the FP32 panels) does not fit a thread's
+// registers: one CTA per tile, eight warps with two rows each, r = w and w + 8, in
+// registers, the pivot row published in shared memory, one barrier per pivot.  As
+// one warp per tile with the block in 256 registers, mostly spilled, it took 18 us
+// on 11 tiles; now 4.
+constexpr int kDiagWarps = 8;
+template <typename T>
+__global__ void __launch_bounds__(32 * kDiagWarps) k_dense_diag16(DevPlan P, DevState S, int k,
+                                                                  const int32_t* __restrict__ gate) {
+  constexpr int KB = 16;
+  __shared__ T prow[2][KB][kTile];
+  if (gate && *gate == 0) return;
+  const int lane = threadIdx.x, w = threadIdx.y, tile = blockIdx.x;
+  if (!tile_active(S, tile, lane)) return;  // uniform over the CTA
+  T* __restrict__ A = reinterpret_cast<T*>(S.lu) + ((size_t)tile * P.NLU + P.NS) * kTile;  // dense block
+  T* __restrict__ inv = reinterpret_cast<T*>(S.inv) + (size_t)tile * KB * kTile + lane;
+  const int ld = P.ndp;
+  T d[2][KB];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int c = 0; c < KB; ++c) d[h][c] = A[dense_off<T>(k + w + 8 * h, k + c, ld, lane)];
+#pragma unroll
+  for (int c = 0; c < KB; ++c) {
+    if (w == (c & 7)) {
+#pragma unroll
+      for (int cc = c; cc < KB; ++cc) prow[c & 1][cc][lane] = d[c >> 3][cc];
+    }
+    __syncthreads();
+    const T ip = (T)1 / prow[c & 1][c][lane];
+    if (w == (c & 7)) inv[c * kTile] = ip;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (w + 8 * h > c) {
+        const T l = d[h][c] * ip;
+        d[h][c] = l;
+#pragma unroll
+        for (int cc = c + 1; cc < KB; ++cc) d[h][cc] -= l * prow[c & 1][cc][lane];
+      }
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int c = 0; c < KB; ++c) A[dense_off<T>(k + w + 8 * h, k + c, ld, lane)] = d[h][c];
 }
 
 // four consecutive rows r .. r+3 (r a multiple of 4) of dense column c for
@@ -1570,7 +1616,7 @@ void launch_prepare_lu(const DevPlan& P, const DevState& S, const int32_t* gate,
     if (sizeof(T) == 4 && P.dim)
       launch_dense_im_set_ones(P, S, gate, st, rec);
     else
-      NRPF_LAUNCH(rec, K_ONES, st, k_set_ones<T><<<dim3(1, S.Bp / kTile), dim3(32, 8), 0, st>>>(P, S, gate));
+      NRPF_LAUNCH(rec, K_ONES, st, k_set_ones<T><<<dim3(P.n_one, S.Bp / kTile), dim3(32, 8), 0, st>>>(P, S, gate));
   }
 }
 
@@ -1583,8 +1629,11 @@ static void launch_dense_step(const DevPlan& P, const DevState& S, int k, int ke
                               cudaStream_t st, Recorder* rec) {
   const int tiles = S.Bp / kTile;
   const int rows = P.ndp - k - KB;
-  NRPF_LAUNCH(rec, K_DENSE_DIAG, st,
-              k_dense_diag<T, KB><<<(tiles + 3) / 4, dim3(32, 4), 0, st>>>(P, S, k, gate));
+  if constexpr (KB == 16)
+    NRPF_LAUNCH(rec, K_DENSE_DIAG, st, k_dense_diag16<T><<<tiles, dim3(32, kDiagWarps), 0, st>>>(P, S, k, gate));
+  else
+    NRPF_LAUNCH(rec, K_DENSE_DIAG, st,
+                k_dense_diag<T, KB><<<(tiles + 3) / 4, dim3(32, 4), 0, st>>>(P, S, k, gate));
   if (rows > 0) {
     const int cols = cend - k - KB;
     NRPF_LAUNCH(rec, K_DENSE_PANEL, st,
