@@ -373,6 +373,7 @@ constexpr uint32_t kImACols = 3 * kImKc / 2;          // ... of one A buffer (th
 constexpr uint32_t kImTmemCols = 256;                 // allocated: 128 + 2 * 48, rounded up to a power of two
 constexpr uint32_t kImBPart = kImTile * kImKc * 2;    // 8 KB: one part of a B chunk
 constexpr uint32_t kImBBuf = 3 * kImBPart;
+constexpr size_t kImGemmTcSmem = 2 * (size_t)kImBBuf + 1024;
 
 // the three BF16 parts of two FP32 values, packed (x0 in the low half)
 __device__ __forceinline__ void split3(float x0, float x1, uint32_t& h, uint32_t& m, uint32_t& l) {
@@ -556,28 +557,49 @@ __device__ __forceinline__ void update_tc(float* __restrict__ A, int ld, int i0,
 // - 1) CTAs, tile-fastest within an instance, so that the CTAs resident at
 // one time share their instance's operand panels in L2.  An instance far from
 // its solution takes the tensor cores, one near it the FMA pipe (kActiveNear,
-// kernels.h, says why the line lies there).
-__global__ void __launch_bounds__(kImGemmThreads, 2)
-    k_im_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, DevPlan P,
-              DevState S, int r0, int ntc, const int32_t* __restrict__ gate) {
-  extern __shared__ uint8_t im_smem_raw[];
-  __shared__ __align__(8) uint64_t bars[kImStages];
-  __shared__ uint32_t tmem_holder;
-  if (gate && *gate == 0) return;
+// kernels.h, says why the line lies there): two kernels, whose CTAs leave at once
+// where the instance is the other's.  In one kernel the FMA form's 97 KB of shared
+// memory per CTA left the tensor-core form, whose operands come through L1, 34 KB
+// of it: 49 ms per refactorisation of 1,000 instances of the 9,000-bus grid, 37
+// alone.
+struct ImTile {
+  float* A;
+  int b, i0, j0;
+};
+
+__device__ __forceinline__ ImTile im_tile(const DevPlan& P, const DevState& S, int r0, int ntc) {
   const int ntile = 2 * ntc - 1;
   const int b = (int)(blockIdx.x / (unsigned)ntile);
   const int t = (int)(blockIdx.x - (unsigned)b * (unsigned)ntile);
-  const int act = S.active[b];
-  if (!act) return;
-  const int i0 = r0 + (t < ntc ? t : 0) * kImTile, j0 = r0 + (t < ntc ? 0 : t - ntc + 1) * kImTile;
-  // 1024-byte alignment for the swizzled chunks (offset arithmetic on the
-  // shared array keeps the pointer in the shared address space)
-  uint8_t* sm = im_smem_raw + ((1024u - (su32(im_smem_raw) & 1023u)) & 1023u);
-  float* A = im_block(P, S, b);
-  if (act == kActiveNear)
-    update_fma(A, P.ndp, i0, j0, r0 / kImKc, sm, bars, &tmA, &tmB, b & 31, b >> 5, &S.bad[b]);
-  else
-    update_tc(A, P.ndp, i0, j0, r0 / kImKc, sm, &bars[0], &tmem_holder, &S.bad[b]);
+  return {im_block(P, S, b), b, r0 + (t < ntc ? t : 0) * kImTile, r0 + (t < ntc ? 0 : t - ntc + 1) * kImTile};
+}
+
+// 1024-byte alignment for the swizzled chunks (offset arithmetic on the shared
+// array keeps the pointer in the shared address space)
+__device__ __forceinline__ uint8_t* align1024(uint8_t* p) { return p + ((1024u - (su32(p) & 1023u)) & 1023u); }
+
+__global__ void __launch_bounds__(kImGemmThreads, 2) k_im_gemm(const __grid_constant__ CUtensorMap tmA,
+                                                               const __grid_constant__ CUtensorMap tmB, DevPlan P,
+                                                               DevState S, int r0, int ntc,
+                                                               const int32_t* __restrict__ gate) {
+  extern __shared__ uint8_t im_smem_raw[];
+  __shared__ __align__(8) uint64_t bars[kImStages];
+  if (gate && *gate == 0) return;
+  const ImTile t = im_tile(P, S, r0, ntc);
+  if (S.active[t.b] != kActiveNear) return;
+  update_fma(t.A, P.ndp, t.i0, t.j0, r0 / kImKc, align1024(im_smem_raw), bars, &tmA, &tmB, t.b & 31, t.b >> 5,
+             &S.bad[t.b]);
+}
+
+__global__ void __launch_bounds__(kImGemmThreads, 2) k_im_gemm_tc(DevPlan P, DevState S, int r0, int ntc,
+                                                                  const int32_t* __restrict__ gate) {
+  extern __shared__ uint8_t im_smem_raw[];
+  __shared__ __align__(8) uint64_t bar;
+  __shared__ uint32_t tmem_holder;
+  if (gate && *gate == 0) return;
+  const ImTile t = im_tile(P, S, r0, ntc);
+  if (S.active[t.b] != kActiveFar) return;
+  update_tc(t.A, P.ndp, t.i0, t.j0, r0 / kImKc, align1024(im_smem_raw), &bar, &tmem_holder, &S.bad[t.b]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1077,6 +1099,7 @@ void launch_dense_im_factor(const DevPlan& P, const DevState& S, const DenseImMa
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || !configured[dev]) {
     cudaFuncSetAttribute(k_im_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImGemmSmem);
+    cudaFuncSetAttribute(k_im_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImGemmTcSmem);
     cudaFuncSetAttribute(k_im_diag<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImDiagSmemPre);
     cudaFuncSetAttribute(k_im_panel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImPanelSmem);
     cudaFuncSetAttribute(k_im_panel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImPanelSmemPre);
@@ -1109,9 +1132,11 @@ void launch_dense_im_factor(const DevPlan& P, const DevState& S, const DenseImMa
   // panels before it
   auto gemm = [&](int r0) {
     const int ntc = (ld - r0 + kImTile - 1) / kImTile;
+    const unsigned grid = Bp * (unsigned)(2 * ntc - 1);
     NRPF_LAUNCH(rec, K_DENSE_UPDATE, st,
-                k_im_gemm<<<Bp * (unsigned)(2 * ntc - 1), kImGemmThreads, kImGemmSmem, st>>>(maps.a, maps.b, P, S,
-                                                                                            r0, ntc, gate));
+                k_im_gemm_tc<<<grid, kImGemmThreads, kImGemmTcSmem, st>>>(P, S, r0, ntc, gate));
+    NRPF_LAUNCH(rec, K_DENSE_UPDATE, st,
+                k_im_gemm<<<grid, kImGemmThreads, kImGemmSmem, st>>>(maps.a, maps.b, P, S, r0, ntc, gate));
   };
   // Left-looking by outer panels: panel j's block column and row first take
   // the products of panels 0 .. j-1 (depth kj, each entry's subtractions in
