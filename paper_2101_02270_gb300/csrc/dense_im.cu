@@ -73,7 +73,7 @@ constexpr size_t kImGemmSmem = (size_t)kImStages * kImStageBytes + 2 * (size_t)k
 // for a hardware-defined time window)
 constexpr uint32_t kImSpinLimit = 1u << 20;
 
-constexpr int kImDiagThreads = 512;
+constexpr int kImDiagThreads = 128;
 constexpr int kImSolveThreads = 256;
 constexpr int kPitch = 68;  // shared row pitch (floats) of 64-wide blocks: rows stay 16-byte aligned
 
@@ -603,48 +603,61 @@ __global__ void __launch_bounds__(kImGemmThreads, 2) k_im_gemm_tc(DevPlan P, Dev
 }
 
 // ---------------------------------------------------------------------------
-// LU of the 64 x 64 diagonal block at (ki, ki), one CTA per instance, and the
-// inverses of its factors.  With PRE, the block first receives the product
-// L(ki:ki+64, k:k+64) U(k:k+64, ki:ki+64) of the outer panel's first step.
-// Unblocked right-looking elimination: the pivot column is scaled by the
-// reciprocal of the pivot, then the trailing block takes the rank-1 update,
-// and the same row operations on an identity block give L11^-1.  A backward
-// sweep over the rows of [U | I] then gives U11^-1.  Both go to the instance's
-// slot of S.inv as
+// LU of the 64 x 64 diagonal block at (ki, ki), one CTA of 128 threads per
+// instance, and the inverses of its factors.  With PRE, the block first receives
+// the product L(ki:ki+64, k:k+64) U(k:k+64, ki:ki+64) of the outer panel's first
+// step.  Unblocked elimination in the order of right-looking LU (every entry takes
+// its products in ascending pivot order), then
 //   ui[q * 64 + c] = U11^-1(q, c),  li[q * 64 + r] = L11^-1(r, q)
-// (zero outside the triangles), the operands the panel kernel multiplies by.
-// Thread (tr, tc) = (tid / R, tid % R), R = 8 threads per row, holds in
-// registers the entries of row tr in the columns c = tc + R i (i < 64 / R) of
-// D, of L11^-1 and of U11^-1.  Per pivot p the threads of row p publish their
-// row to a double-buffered shared row (one barrier per pivot), the multiplier
-// of row tr comes from its owner by a shuffle among the row's R lanes, and
-// every update is unrolled.  Measured on the 9,000-bus block: R = 4 (256
-// threads) 184 ms per step, stalled on instruction fetch (the unrolled pivot
-// loops); R = 8 179 ms; R = 16 304 ms; a pivot loop not unrolled, 558 ms.
-// Shared memory (dynamic, PRE only): W1[q][r] = L(ki + r, k + q), W2[c][q] =
-// U(k + q, ki + c).
+// (zero outside the triangles) to the instance's slot of S.inv, the operands the
+// panel kernel multiplies by.
+//
+// Thread (ti, tj) = (tid % 16, tid / 16) holds rows 4 ti .. 4 ti + 3 of columns
+// 8 tj .. 8 tj + 7 in registers.  A block of eight pivots is then one tj, half a
+// warp, which factorises its 64 x 8 panel by shuffles alone; the two row groups of
+// the block finish their rows of U likewise; and a rank-8 update in registers
+// takes the rest: two barriers per eight pivots.  The inverses go column by column,
+// a thread each (64 for L11^-1, 64 for U11^-1), eight rows at a time: the columns
+// are independent and need no barrier.  Both share one 64 x 64 array, one its lower
+// and one its upper triangle; 42 KB and 20 warps on an SM.
+// What bounds it is issue and latency within a CTA, so small CTAs, five per SM.  With
+// 512 threads, eight per row, two barriers per pivot (one for each of the sweeps)
+// and two CTAs per SM 200,000 blocks took 24.7 ms; now 14.0 ms (15.1 ms before the
+// two products went to packed FMAs, pairs of rows in a register pair; the factors are
+// kept negated in shared memory so that those need no negation), every rounding the
+// same.
 // ---------------------------------------------------------------------------
-constexpr size_t kImDiagSmemPre = 2 * 64 * kPitch * sizeof(float);
+constexpr int kXPitch = 65;
+constexpr size_t kImDiagSmem = (64 * kPitch + 64 * kXPitch + 4 * 8 * 64 + 64) * sizeof(float);
+static_assert(2 * 64 * kPitch <= 64 * kPitch + 64 * kXPitch + 4 * 8 * 64, "PRE operands fit before the rest");
 
 template <bool PRE>
-__global__ void __launch_bounds__(kImDiagThreads, 2) k_im_diag(DevPlan P, DevState S, int k, int ki,
-                                                                        const int32_t* __restrict__ gate) {
-  constexpr int R = kImDiagThreads / 64;  // threads per row
-  constexpr int NC = 64 / R;              // columns per thread
+__global__ void __launch_bounds__(kImDiagThreads, 5) k_im_diag(DevPlan P, DevState S, int k, int ki,
+                                                               const int32_t* __restrict__ gate) {
   extern __shared__ __align__(16) float diag_smem[];
-  __shared__ float prow[2][64], pli[2][64], invd[64];
+  float(*M)[kPitch] = reinterpret_cast<float(*)[kPitch]>(diag_smem);                    // M[c][r]: minus L, minus U / pivots
+  float(*X)[kXPitch] = reinterpret_cast<float(*)[kXPitch]>(diag_smem + 64 * kPitch);    // X[r][c]: the inverses
+  float(*Lp)[8][64] = reinterpret_cast<float(*)[8][64]>(diag_smem + 64 * kPitch + 64 * kXPitch);  // [2]: L(r, p)
+  float(*Up)[8][64] = Lp + 2;                                                           // [2]: U(p, c)
+  float* invd = diag_smem + 64 * kPitch + 64 * kXPitch + 4 * 8 * 64;
   if (gate && *gate == 0) return;
   const int b = blockIdx.x;
   if (!S.active[b]) return;
-  const int ld = P.ndp, tid = threadIdx.x, tc = tid % R, tr = tid / R;
-  const int src0 = tid & 31 & ~(R - 1);  // lane of (tr, 0)
+  const int ld = P.ndp, tid = threadIdx.x, ti = tid & 15, tj = tid >> 4;
   float* __restrict__ A = im_block(P, S, b);
-  float d[NC];
+  float2 w2[2][8];  // row 4 ti + a, column 8 tj + c at w2[a / 2][c], pairs of rows packed
+#define v(a, c) ((a) & 1 ? w2[(a) >> 1][c].y : w2[(a) >> 1][c].x)
 #pragma unroll
-  for (int i = 0; i < NC; ++i) d[i] = A[(size_t)(ki + tc + R * i) * ld + ki + tr];
+  for (int c = 0; c < 8; ++c) {
+    const float4 q = *reinterpret_cast<const float4*>(A + (size_t)(ki + 8 * tj + c) * ld + ki + 4 * ti);
+    v(0, c) = q.x;
+    v(1, c) = q.y;
+    v(2, c) = q.z;
+    v(3, c) = q.w;
+  }
   if (PRE) {
-    float(*W1)[kPitch] = reinterpret_cast<float(*)[kPitch]>(diag_smem);
-    float(*W2)[kPitch] = reinterpret_cast<float(*)[kPitch]>(diag_smem + 64 * kPitch);
+    float(*W1)[kPitch] = reinterpret_cast<float(*)[kPitch]>(diag_smem);                 // W1[q][r] = L(ki + r, k + q)
+    float(*W2)[kPitch] = reinterpret_cast<float(*)[kPitch]>(diag_smem + 64 * kPitch);   // W2[c][q] = U(k + q, ki + c)
 #pragma unroll
     for (int j = 0; j < 64 * 16 / kImDiagThreads; ++j) {
       const int e = tid + j * kImDiagThreads, c = e >> 4, r4 = 4 * (e & 15);
@@ -653,82 +666,172 @@ __global__ void __launch_bounds__(kImDiagThreads, 2) k_im_diag(DevPlan P, DevSta
     }
     cp16_wait_all();
     __syncthreads();
-    // D(tr, c) minus the products in ascending q
 #pragma unroll 1
     for (int q = 0; q < 64; q += 4) {
-      const float l0 = W1[q][tr], l1 = W1[q + 1][tr], l2 = W1[q + 2][tr], l3 = W1[q + 3][tr];
+      float4 l[4];
 #pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        const float4 u = *reinterpret_cast<const float4*>(&W2[tc + R * i][q]);
-        d[i] = fmaf(-l0, u.x, d[i]);
-        d[i] = fmaf(-l1, u.y, d[i]);
-        d[i] = fmaf(-l2, u.z, d[i]);
-        d[i] = fmaf(-l3, u.w, d[i]);
+      for (int z = 0; z < 4; ++z) l[z] = *reinterpret_cast<const float4*>(&W1[q + z][4 * ti]);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const float4 u = *reinterpret_cast<const float4*>(&W2[8 * tj + c][q]);
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          const float2 nu = make_float2(-comp(u, z), -comp(u, z));
+          w2[0][c] = __ffma2_rn(make_float2(l[z].x, l[z].y), nu, w2[0][c]);
+          w2[1][c] = __ffma2_rn(make_float2(l[z].z, l[z].w), nu, w2[1][c]);
+        }
       }
     }
+    __syncthreads();  // M, X and the rest overwrite the operands
   }
-  float li[NC];
+#pragma unroll 1
+  for (int kb = 0; kb < 8; ++kb) {
+    float(*L)[64] = Lp[kb & 1], (*U)[64] = Up[kb & 1];
+    if (tj >> 1 == kb >> 1) {  // the warp whose half holds the panel
+      // pivot p: row 8 kb + p, held by row group 2 kb + p / 4 of this half warp
 #pragma unroll
-  for (int i = 0; i < NC; ++i) li[i] = (tc + R * i == tr) ? 1.f : 0.f;
+      for (int p = 0; p < 8; ++p) {
+        float row[8];
 #pragma unroll
-  for (int p = 0; p < 64; ++p) {
-    const int buf = p & 1;
-    if (tr == p) {
+        for (int c = 0; c < 8; ++c)
+          if (c >= p) row[c] = __shfl_sync(0xffffffffu, v(p & 3, c), 2 * kb + (p >> 2), 16);
+        if (tj == kb) {
+          const float inv = 1.f / row[p];
+          if (ti == 0) invd[8 * kb + p] = inv;
 #pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        prow[buf][tc + R * i] = d[i];
-        pli[buf][tc + R * i] = li[i];
+          for (int a = 0; a < 4; ++a)
+            if (4 * ti + a > 8 * kb + p) {
+              const float l = v(a, p) * inv;
+              v(a, p) = l;
+#pragma unroll
+              for (int c = p + 1; c < 8; ++c) v(a, c) = fmaf(-l, row[c], v(a, c));
+            }
+        }
+      }
+      if (tj == kb) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          *reinterpret_cast<float4*>(&L[c][4 * ti]) = make_float4(v(0, c), v(1, c), v(2, c), v(3, c));
       }
     }
     __syncthreads();
-    const float lraw = __shfl_sync(0xffffffffu, d[p / R], src0 | (p % R));  // D(tr, p)
-    if (tr > p) {
-      const float inv = 1.f / prow[buf][p];
-      const float l = lraw * inv;
-      if (tc == p % R) d[p / R] = l;
+    if ((tj | 1) > kb) {  // a warp with columns to the right
+      // rows of U: row p to the rows of its block below it
 #pragma unroll
-      for (int i = 0; i < NC; ++i)
-        if (tc + R * i > p) d[i] = fmaf(-l, prow[buf][tc + R * i], d[i]);
+      for (int p = 0; p < 7; ++p) {
+        float u[8];
 #pragma unroll
-      for (int i = 0; i < NC; ++i)
-        if (tc + R * i <= p) li[i] = fmaf(-l, pli[buf][tc + R * i], li[i]);
+        for (int c = 0; c < 8; ++c) u[c] = __shfl_sync(0xffffffffu, v(p & 3, c), 2 * kb + (p >> 2), 16);
+        if (tj > kb && ti >> 1 == kb) {
+#pragma unroll
+          for (int a = 0; a < 4; ++a)
+            if (4 * (ti & 1) + a > p) {
+              const float l = L[p][4 * ti + a];
+#pragma unroll
+              for (int c = 0; c < 8; ++c) v(a, c) = fmaf(-l, u[c], v(a, c));
+            }
+        }
+      }
+      if (tj > kb && ti >> 1 == kb) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          float4* o = reinterpret_cast<float4*>(&U[4 * (ti & 1) + a][8 * tj]);
+          o[0] = make_float4(v(a, 0), v(a, 1), v(a, 2), v(a, 3));
+          o[1] = make_float4(v(a, 4), v(a, 5), v(a, 6), v(a, 7));
+        }
+      }
+    }
+    __syncthreads();
+    if (tj > kb && ti >> 1 > kb) {
+#pragma unroll
+      for (int p = 0; p < 8; ++p) {
+        const float4 l = *reinterpret_cast<const float4*>(&L[p][4 * ti]);
+        const float4 u0 = *reinterpret_cast<const float4*>(&U[p][8 * tj]);
+        const float4 u1 = *reinterpret_cast<const float4*>(&U[p][8 * tj + 4]);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const float u = -(c < 4 ? comp(u0, c) : comp(u1, c - 4));
+          const float2 nu = make_float2(u, u);
+          w2[0][c] = __ffma2_rn(make_float2(l.x, l.y), nu, w2[0][c]);
+          w2[1][c] = __ffma2_rn(make_float2(l.z, l.w), nu, w2[1][c]);
+        }
+      }
     }
   }
-  float* __restrict__ inv_out = reinterpret_cast<float*>(S.inv) + (size_t)b * 8192;
+  // the factors out; in M, negated, with U's column c over pivot c
 #pragma unroll
-  for (int i = 0; i < NC; ++i) {
-    A[(size_t)(ki + tc + R * i) * ld + ki + tr] = d[i];
-    inv_out[4096 + (tc + R * i) * 64 + tr] = li[i];  // li[q][r] = L11^-1(r, q)
-    if (tc + R * i == tr) invd[tr] = 1.f / d[i];
+  for (int c = 0; c < 8; ++c) {
+    const int col = 8 * tj + c;
+    *reinterpret_cast<float4*>(A + (size_t)(ki + col) * ld + ki + 4 * ti) =
+        make_float4(v(0, c), v(1, c), v(2, c), v(3, c));
+    const float inv = invd[col];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) M[col][4 * ti + a] = -(4 * ti + a < col ? v(a, c) * inv : v(a, c));
   }
-  float ui[NC];
-#pragma unroll
-  for (int i = 0; i < NC; ++i) ui[i] = (tc + R * i == tr) ? 1.f : 0.f;
+#undef v
+  for (int e = tid; e < 64 * kXPitch; e += kImDiagThreads) X[0][e] = 0.f;
   __syncthreads();
-  // row p of [U | I], still unscaled, goes to the rows above it; then row p
-  // is scaled by 1 / U(p, p)
+  // Column c of L11^-1: x_i -= L(i, p) x_p, p ascending; of U11^-1, not yet scaled by
+  // the pivots of its rows: x_i -= (U(i, p) / pivot p) x_p, p descending.
+  {
+    const bool low = tid < 64;
+    const int c = tid & 63;
+    auto get = [&](int r) { return r == c ? 1.f : (low ? r > c : r < c) ? X[r][c] : 0.f; };
+    auto put = [&](int r, float x) {
+      if (low ? r > c : r < c) X[r][c] = x;
+    };
+#pragma unroll 1
+    for (int z = 0; z < 8; ++z) {
+      const int pb = 8 * (low ? z : 7 - z);  // this block's first row
+      float x[8];
 #pragma unroll
-  for (int p = 63; p >= 0; --p) {
-    const int buf = p & 1;
-    if (tr == p) {
+      for (int r = 0; r < 8; ++r) x[r] = get(pb + r);
+      if (low) {
 #pragma unroll
-      for (int i = 0; i < NC; ++i) prow[buf][tc + R * i] = ui[i];
-    }
-    __syncthreads();
-    const float uraw = __shfl_sync(0xffffffffu, d[p / R], src0 | (p % R));  // U(tr, p)
-    if (tr < p) {
-      const float u = uraw * invd[p];
+        for (int p = 0; p < 8; ++p)
 #pragma unroll
-      for (int i = 0; i < NC; ++i)
-        if (tc + R * i >= p) ui[i] = fmaf(-u, prow[buf][tc + R * i], ui[i]);
-    } else if (tr == p) {
+          for (int r = p + 1; r < 8; ++r) x[r] = fmaf(M[pb + p][pb + r], x[p], x[r]);
+      } else {
 #pragma unroll
-      for (int i = 0; i < NC; ++i)
-        if (tc + R * i >= p) ui[i] *= invd[p];
+        for (int p = 7; p >= 0; --p)
+#pragma unroll
+          for (int r = 0; r < p; ++r) x[r] = fmaf(M[pb + p][pb + r], x[p], x[r]);
+      }
+#pragma unroll
+      for (int r = 0; r < 8; ++r) put(pb + r, x[r]);
+#pragma unroll 1
+      for (int y = z + 1; y < 8; ++y) {
+        const int ib = 8 * (low ? y : 7 - y);
+        float2 w[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) w[r] = make_float2(get(ib + 2 * r), get(ib + 2 * r + 1));
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          // p ascending (descending) with q; the block's column p of M, rows ib ..
+          const float xp = low ? x[q] : x[7 - q];
+          const float* m = &M[pb + (low ? q : 7 - q)][ib];
+          const float4 m0 = *reinterpret_cast<const float4*>(m), m1 = *reinterpret_cast<const float4*>(m + 4);
+          const float2 x2 = make_float2(xp, xp);
+          w[0] = __ffma2_rn(make_float2(m0.x, m0.y), x2, w[0]);
+          w[1] = __ffma2_rn(make_float2(m0.z, m0.w), x2, w[1]);
+          w[2] = __ffma2_rn(make_float2(m1.x, m1.y), x2, w[2]);
+          w[3] = __ffma2_rn(make_float2(m1.z, m1.w), x2, w[3]);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          put(ib + 2 * r, w[r].x);
+          put(ib + 2 * r + 1, w[r].y);
+        }
+      }
     }
   }
-#pragma unroll
-  for (int i = 0; i < NC; ++i) inv_out[tr * 64 + tc + R * i] = ui[i];  // ui[q][c] = U11^-1(q, c)
+  __syncthreads();
+  float* __restrict__ inv_out = reinterpret_cast<float*>(S.inv) + (size_t)b * 8192;
+  for (int e = tid; e < 4096; e += kImDiagThreads) {
+    const int q = e >> 6, c = e & 63;
+    inv_out[e] = c > q ? X[q][c] * invd[q] : c == q ? invd[q] : 0.f;     // U11^-1(q, c)
+    inv_out[4096 + e] = c > q ? X[c][q] : c == q ? 1.f : 0.f;            // L11^-1(c, q)
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1100,7 +1203,8 @@ void launch_dense_im_factor(const DevPlan& P, const DevState& S, const DenseImMa
   if (dev < 0 || dev >= 64 || !configured[dev]) {
     cudaFuncSetAttribute(k_im_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImGemmSmem);
     cudaFuncSetAttribute(k_im_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImGemmTcSmem);
-    cudaFuncSetAttribute(k_im_diag<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImDiagSmemPre);
+    cudaFuncSetAttribute(k_im_diag<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImDiagSmem);
+    cudaFuncSetAttribute(k_im_diag<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImDiagSmem);
     cudaFuncSetAttribute(k_im_panel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImPanelSmem);
     cudaFuncSetAttribute(k_im_panel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kImPanelSmemPre);
     if (dev >= 0 && dev < 64) configured[dev] = true;
@@ -1110,7 +1214,7 @@ void launch_dense_im_factor(const DevPlan& P, const DevState& S, const DenseImMa
   // the two 64-wide steps of the outer panel at k
   auto outer = [&](int k) {
     NRPF_LAUNCH(rec, K_DENSE_DIAG, st,
-                k_im_diag<false><<<Bp, kImDiagThreads, 0, st>>>(P, S, k, k, gate));
+                k_im_diag<false><<<Bp, kImDiagThreads, kImDiagSmem, st>>>(P, S, k, k, gate));
     int nr = ld - k - 64;
     if (nr > 0) {
       const int nch = (nr + 127) / 128;
@@ -1119,7 +1223,7 @@ void launch_dense_im_factor(const DevPlan& P, const DevState& S, const DenseImMa
     }
     if (ld - k < kImOuter) return;  // a last outer panel of 64
     NRPF_LAUNCH(rec, K_DENSE_DIAG, st,
-                k_im_diag<true><<<Bp, kImDiagThreads, kImDiagSmemPre, st>>>(P, S, k, k + 64, gate));
+                k_im_diag<true><<<Bp, kImDiagThreads, kImDiagSmem, st>>>(P, S, k, k + 64, gate));
     nr = ld - k - kImOuter;
     if (nr > 0) {
       const int nch = (nr + 127) / 128;
