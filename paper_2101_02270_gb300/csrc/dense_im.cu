@@ -1060,10 +1060,12 @@ __global__ void __launch_bounds__(kImPanelThreads2, 3) k_im_panel(DevPlan P, Dev
 // thread updates its rows below (above) the block with the block's 64
 // entries, reading the matrix columns contiguously across the CTA.  The solve
 // reads each instance's block once and is bound by how many loads are in
-// flight: at most 40 registers per thread let six CTAs (six instances) run on
-// an SM instead of four, which halved its time on the 9,000-bus block.
+// flight, and by the last wave: at most 32 registers per thread let eight CTAs (eight
+// instances) run on an SM.  On 1,000 blocks of 2,176 (18.9 GB per solve) six CTAs of 40
+// registers took 4.7 ms, two waves, the second nearly empty; eight take 3.2 ms
+// (5.9 TB/s).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kImSolveThreads, 6) k_im_dsolve(DevPlan P, DevState S,
+__global__ void __launch_bounds__(kImSolveThreads, 8) k_im_dsolve(DevPlan P, DevState S,
                                                               const int32_t* __restrict__ gate) {
   extern __shared__ float xs[];                  // [ndp]
   __shared__ float T[64][65];                    // T[c][r]
