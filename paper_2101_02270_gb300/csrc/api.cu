@@ -449,6 +449,7 @@ int pf_plan_create(int n, const int32_t* rowptr, const int32_t* colidx, const do
   const HostPlan& h = p->hp;
   DevPlan& d = p->dp;
   d.n = h.n; d.m = h.m; d.s = h.s; d.nd = h.nd; d.ndp = h.ndp; d.kb = h.kb; d.mp = h.s + h.ndp;
+  d.nde = p->lu_precision == NRPF_LU_FP32 && !d.dim && h.kb > 16 ? std::min(h.ndp, (h.nd + 15) / 16 * 16) : h.ndp;
   d.NS = h.NS; d.NLU = h.NLU; d.nnzY = (int)h.colidx.size();
   d.n_one = (int)h.one_pos.size();
   d.n_lu_lvl = (int)h.lu_lvl_ptr.size() - 1;

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(kCluThreads) k_dense_cluster(DevPlan P, DevSta
   if (gate && *gate == 0) return;
   const int b = blockIdx.x / kClu, rank = blockIdx.x % kClu;
   if (!S.active[b]) return;  // uniform over the cluster
-  const int ld = P.ndp, nblk = ld / kCluNb, nl = (nblk + kClu - 1) / kClu;
+  const int ld = P.nde, nblk = ld / kCluNb, nl = (nblk + kClu - 1) / kClu;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int W = kCluThreads / 32;
   T* A = reinterpret_cast<T*>(clu_raw);            // [nl * 8 columns][ld]
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kCluThreads) k_dense_cluster(DevPlan P, DevSta
   for (int lb = 0; lb * kClu + rank < nblk; ++lb)
     for (int q = tid; q < kCluNb * ld; q += kCluThreads) {
       const int c = (lb * kClu + rank) * kCluNb + q / ld, r = q % ld;
-      A[(size_t)lb * kCluNb * ld + q] = G[lu_off<T>(P, P.NS + (int64_t)c * ld + r, b & 31)];
+      A[(size_t)lb * kCluNb * ld + q] = G[lu_off<T>(P, P.NS + (int64_t)c * P.ndp + r, b & 31)];
     }
   if (rank == 0)
     for (int r = tid; r < ld; r += kCluThreads) y[r] = X[(size_t)r * kTile];
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(kCluThreads) k_dense_cluster(DevPlan P, DevSta
 }  // namespace
 
 bool dense_cluster_fits(const DevPlan& P, const DevState& S, size_t width) {
-  return P.ndp >= 2 * kCluNb && P.ndp % kCluNb == 0 && S.Bp <= kCluTiles * kTile && clu_smem(P.ndp, width) <= kCluSmem;
+  return P.nde >= 2 * kCluNb && P.nde % kCluNb == 0 && S.Bp <= kCluTiles * kTile && clu_smem(P.nde, width) <= kCluSmem;
 }
 
 template <typename T>
@@ -225,7 +225,7 @@ void launch_dense_cluster(const DevPlan& P, const DevState& S, const int32_t* ga
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(S.Bp * kClu));
   cfg.blockDim = dim3(kCluThreads);
-  cfg.dynamicSmemBytes = clu_smem(P.ndp, sizeof(T));
+  cfg.dynamicSmemBytes = clu_smem(P.nde, sizeof(T));
   cfg.stream = st;
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;

@@ -32,6 +32,10 @@ struct DevUpd {
 // Read-only plan arrays on the device (copied once by pf_plan_create).
 struct DevPlan {
   int n, m, s, nd, ndp, kb, mp;  // mp = s + ndp (rhs length incl. padding)
+  // columns of the dense block that are worked on, ndp its leading dimension: nd
+  // rounded up to the 16 of the FP32 kernels' steps where ndp is rounded further
+  // (their outer panels), ndp otherwise
+  int nde;
   int dim;  // 1: instance-major dense block (FP32 LU; see dense_im.h), 0: interleaved
   int64_t NS, NLU;
   int nnzY;

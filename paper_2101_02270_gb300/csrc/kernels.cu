@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "dense_cluster.h"
+#include "dense_il.h"
 #include "dense_im.h"
 #include "device.h"
 #include "kernels.h"
@@ -349,7 +350,7 @@ __global__ void k_zero16(uint4* __restrict__ p, size_t n16, size_t stride16, int
 }
 
 // Identity on the padding of the dense block, and zero right-hand side on
-// its padding rows (m .. s+ndp-1): no other kernel writes those rows, and a
+// its padding rows (m .. s+nde-1): no other kernel writes those rows, and a
 // stale non-finite value there would leak into real rows as 0 * NaN during
 // the backward substitution.
 template <typename T>
@@ -358,10 +359,10 @@ __global__ void k_set_ones(DevPlan P, DevState S, const int32_t* __restrict__ ga
   const int tile = blockIdx.y, lane = threadIdx.x;
   T* LU = reinterpret_cast<T*>(S.lu) + (size_t)tile * P.NLU * kTile;
   T* X = reinterpret_cast<T*>(S.x) + (size_t)tile * P.mp * kTile;
-  // padding columns nd .. ndp-1 of the dense block: whole identity columns
+  // padding columns nd .. nde-1 of the dense block: whole identity columns
   // (the refactorisation does not zero the dense block)
   const int t = blockIdx.x;  // a block per padding column
-  for (int r = threadIdx.y; r < P.ndp; r += blockDim.y)
+  for (int r = threadIdx.y; r < P.nde; r += blockDim.y)
     LU[lu_off<T>(P, P.NS + (int64_t)(P.nd + t) * P.ndp + r, lane)] = (T)(r == P.nd + t ? 1 : 0);
   if (threadIdx.y == 0) X[(size_t)(P.m + t) * kTile + lane] = (T)0;
 }
@@ -640,7 +641,7 @@ __global__ void __launch_bounds__(32 * kSchurWarps, sizeof(T) == 8 ? 7 : 10) k_s
 #pragma unroll
     for (int g = 0; g < 8; ++g) {
       const int r0 = 32 * task.y + 4 * g;
-      if (r0 >= P.ndp) break;
+      if (r0 >= P.nde) break;
       float4* q = A4 + ((size_t)task.x * P.ndp + r0) * 8 + lane;
       const uint32_t jb = jm >> (4 * g) & 0xFu;
       float4 v = jb ? *q : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -700,11 +701,9 @@ __global__ void k_dense_diag(DevPlan P, DevState S, int k, const int32_t* __rest
     for (int r = 0; r < KB; ++r) A[dense_off<T>(k + r, k + c, ld, lane)] = D[r][c];
 }
 
-// The 16 x 16 block (the step of the FP32 panels) does not fit a thread's
-// registers: one CTA per tile, eight warps with two rows each, r = w and w + 8, in
-// registers, the pivot row published in shared memory, one barrier per pivot.  As
-// one warp per tile with the block in 256 registers, mostly spilled, it took 18 us
-// on 11 tiles; now 4.
+// The 16 x 16 block does not fit a thread's registers: one CTA per tile, eight warps
+// with two rows each, r = w and w + 8, in registers, the pivot row published in shared
+// memory, one barrier per pivot.
 constexpr int kDiagWarps = 8;
 template <typename T>
 __global__ void __launch_bounds__(32 * kDiagWarps) k_dense_diag16(DevPlan P, DevState S, int k,
@@ -904,7 +903,7 @@ __global__ void __launch_bounds__(128, UpdOcc<T, TS>::value) k_dense_update(DevP
         acc2[2 * h][c] = make_float2(v.x, v.y);
         acc2[2 * h + 1][c] = make_float2(v.z, v.w);
       }
-#pragma unroll(KB > 16 ? 2 : KB / 4)
+#pragma unroll
     for (int pp = 0; pp < KB / 4; ++pp) {
       float4 bq[TS];  // rows k+4pp .. k+4pp+3 of columns j0 .. j0+7 (U12)
 #pragma unroll
@@ -1319,7 +1318,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 32 ? 1 : 3) k_dense_solve_smem(
   if (!__syncthreads_or(S.active[tile * kTile + lane])) return;
   const T* __restrict__ Ab = reinterpret_cast<const T*>(S.lu) + ((size_t)tile * P.NLU + P.NS) * kTile;
   T* __restrict__ X = reinterpret_cast<T*>(S.x) + ((size_t)tile * P.mp + P.s) * kTile + lane;
-  const int ld = P.ndp;
+  const int ld = P.ndp, n = P.nde;
   // rows r .. r+U-1 of column c (r a multiple of U)
   auto ldu = [&](int r, int c, T(&v)[U]) {
     if constexpr (U == 4) {
@@ -1333,7 +1332,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 32 ? 1 : 3) k_dense_solve_smem(
   // in global memory (same blocked algorithm, L2-resident per tile)
   T* xs = SMEM ? reinterpret_cast<T*>(smem_raw) : X - lane;  // xs[r * 32 + lane]
   if (SMEM)
-    for (int r = warp; r < ld; r += NW) xs[r * kTile + lane] = X[(size_t)r * kTile];
+    for (int r = warp; r < n; r += NW) xs[r * kTile + lane] = X[(size_t)r * kTile];
   // rows r .. r+U-1 minus the block's columns k0 .. k0+SB-1 times xb
   auto update = [&](int r, int k0, const T(&xb)[SB], T(&acc)[U]) {
 #pragma unroll
@@ -1397,21 +1396,21 @@ __global__ void __launch_bounds__(32 * NW, NW == 32 ? 1 : 3) k_dense_solve_smem(
 #pragma unroll
     for (int c = 0; c < SB; ++c) rec[(k / SB) & 1][c][lane] = (T)1 / d[c];
   };
-  if (warp == NW - 1) reciprocals(ld - SB);
-  if (warp == NW - 2 && ld > SB) reciprocals(ld - 2 * SB);
+  if (warp == NW - 1) reciprocals(n - SB);
+  if (warp == NW - 2 && n > SB) reciprocals(n - 2 * SB);
   T xb[SB];
 #pragma unroll
   for (int c = 0; c < SB; ++c) xb[c] = (T)0;
   __syncthreads();
   if (warp == 0) head(0, -1, xb, false);
   __syncthreads();
-  for (int k0 = 0; k0 + SB < ld; k0 += SB) {
+  for (int k0 = 0; k0 + SB < n; k0 += SB) {
 #pragma unroll
     for (int c = 0; c < SB; ++c) xb[c] = xs[(k0 + c) * kTile + lane];
     if (warp == 0) {
       head(k0 + SB, k0, xb, false);
     } else {
-      for (int r = k0 + 2 * SB + U * (warp - 1); r < ld; r += U * (NW - 1)) {
+      for (int r = k0 + 2 * SB + U * (warp - 1); r < n; r += U * (NW - 1)) {
         T acc[U];
         update(r, k0, xb, acc);
 #pragma unroll
@@ -1420,9 +1419,9 @@ __global__ void __launch_bounds__(32 * NW, NW == 32 ? 1 : 3) k_dense_solve_smem(
     }
     __syncthreads();
   }
-  if (warp == 0) head(ld - SB, -1, xb, true);
+  if (warp == 0) head(n - SB, -1, xb, true);
   __syncthreads();
-  for (int k0 = ld - SB; k0 > 0; k0 -= SB) {
+  for (int k0 = n - SB; k0 > 0; k0 -= SB) {
 #pragma unroll
     for (int c = 0; c < SB; ++c) xb[c] = xs[(k0 + c) * kTile + lane];
     if (warp == 0) {
@@ -1440,7 +1439,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 32 ? 1 : 3) k_dense_solve_smem(
     __syncthreads();
   }
   if (SMEM)
-    for (int r = warp; r < ld; r += NW) X[(size_t)r * kTile] = xs[r * kTile + lane];
+    for (int r = warp; r < n; r += NW) X[(size_t)r * kTile] = xs[r * kTile + lane];
 }
 
 // ---------------------------------------------------------------------------
@@ -1615,8 +1614,8 @@ void launch_prepare_lu(const DevPlan& P, const DevState& S, const int32_t* gate,
   if (P.n_one > 0) {
     if (sizeof(T) == 4 && P.dim)
       launch_dense_im_set_ones(P, S, gate, st, rec);
-    else
-      NRPF_LAUNCH(rec, K_ONES, st, k_set_ones<T><<<dim3(P.n_one, S.Bp / kTile), dim3(32, 8), 0, st>>>(P, S, gate));
+    else if (P.nde > P.nd)
+      NRPF_LAUNCH(rec, K_ONES, st, k_set_ones<T><<<dim3(P.nde - P.nd, S.Bp / kTile), dim3(32, 8), 0, st>>>(P, S, gate));
   }
 }
 
@@ -1652,7 +1651,7 @@ static void launch_dense_step(const DevPlan& P, const DevState& S, int k, int ke
   }
 }
 
-// Outer panel of width KBO (two-level blocking): 16-wide steps factorise the
+// FP64, outer panel of width KBO (two-level blocking): 16-wide steps factorise the
 // outer panel's columns and its rows to the right (U12), each step updating
 // only that L-shaped region; then one trailing update of depth KBO (one pass
 // over the trailing block per KBO columns instead of per 16).
@@ -1663,7 +1662,7 @@ static void launch_dense_outer(const DevPlan& P, const DevState& S, int k, const
   for (int ki = k; ki < k + KBO; ki += 16) launch_dense_step<T, 16>(P, S, ki, k + KBO, P.ndp, gate, st, rec);
   const int rest = P.ndp - k - KBO;
   if (rest > 0) {
-    constexpr int TS = sizeof(T) == 4 ? 8 : 4;
+    constexpr int TS = 4;
     NRPF_LAUNCH(rec, K_DENSE_UPDATE, st,
                 k_dense_update<T, KBO, TS><<<grid2((int64_t)(rest / TS) * (rest / TS), 4, tiles), dim3(32, 4), 0,
                                              st>>>(P, S, k, P.ndp, P.ndp, gate));
@@ -1711,6 +1710,10 @@ void launch_factor(const DevPlan& P, const DevState& S, const std::vector<int32_
       if (P.ndp > 0) launch_dense_im_factor(P, S, *reinterpret_cast<const DenseImMaps*>(S.im_maps), gate, st, rec);
       return;
     }
+    if (P.kb >= 16) {  // narrower panels only where a plan asks for them
+      launch_dense_il_factor(P, S, gate, st, rec);
+      return;
+    }
   }
   if constexpr (sizeof(T) == 8) {
     if (S.limb && P.kb == 8) {
@@ -1740,9 +1743,11 @@ void launch_factor(const DevPlan& P, const DevState& S, const std::vector<int32_
   for (int k = 0; k < P.ndp; k += P.kb) {
     if (P.kb == 4) launch_dense_step<T, 4>(P, S, k, P.ndp, P.ndp, gate, st, rec);
     else if (P.kb == 8) launch_dense_step<T, 8>(P, S, k, P.ndp, P.ndp, gate, st, rec);
-    else if (P.kb == 16) launch_dense_step<T, 16>(P, S, k, P.ndp, P.ndp, gate, st, rec);
-    else if (P.kb == 32) launch_dense_outer<T, 32>(P, S, k, gate, st, rec);
-    else launch_dense_outer<T, 64>(P, S, k, gate, st, rec);
+    if constexpr (sizeof(T) == 8) {
+      if (P.kb == 16) launch_dense_step<T, 16>(P, S, k, P.ndp, P.ndp, gate, st, rec);
+      else if (P.kb == 32) launch_dense_outer<T, 32>(P, S, k, gate, st, rec);
+      else if (P.kb == 64) launch_dense_outer<T, 64>(P, S, k, gate, st, rec);
+    }
   }
 }
 
@@ -1789,8 +1794,8 @@ void launch_solve(const DevPlan& P, const DevState& S, const std::vector<int32_t
   } else if (sizeof(T) == 4 && P.dim) {
     if (P.ndp > 0) launch_dense_im_solve(P, S, gate, st, rec);
   } else if (P.ndp > 0) {
-    const size_t smem = (size_t)P.ndp * kTile * sizeof(T);
-    if (P.ndp % 8 == 0)
+    const size_t smem = (size_t)P.nde * kTile * sizeof(T);
+    if (P.nde % 8 == 0)
       launch_dense_solve_smem<T, 8>(P, S, gate, st, rec, smem);
     else
       launch_dense_solve_smem<T, 4>(P, S, gate, st, rec, smem);

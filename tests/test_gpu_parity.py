@@ -488,3 +488,27 @@ def test_dense_block_by_clusters(n, branches, lu, kw, B):
     idx = sorted({0, B // 2, B - 1})
     Vo, ito, sto = _oracle_solve(g, S, V0, idx=idx)
     _compare_newton(g, Vg[idx], itg[idx], stg[idx], Vo, ito, sto, S[idx], check_iters=lu == "fp64")
+
+
+@pytest.mark.parametrize("n,branches", [(30, 40), (60, 85), (150, 210), (230, 330), (420, 590), (700, 980), (900, 1300)])
+@pytest.mark.parametrize("panel", [16, 32, 64])
+def test_interleaved_fp32_block_by_panels(n, branches, panel):
+    """The interleaved FP32 dense block, one 16-wide step up to several outer
+    panels of 64, with a last panel of every number of steps and stored with more
+    or less padding: staged solves are backward stable, |J x - b| at most 90 units
+    of FP32 rounding times (|J| |x| + |b|) in the max norm."""
+    import gridgen
+    g = gridgen.make_grid("mesh2000_b10k", 0, n=n, n_branch=branches, n_pv=max(1, n // 10), load_scale=1 / 16)
+    B = 36
+    V = _dev(perturbed(np.broadcast_to(g.v_set.astype(complex), (B, g.n)).copy()))
+    with _plan(g, lu_precision="fp32", panel=panel, dense_layout="interleaved") as p, _plan(g) as q:
+        m = p.info["m"]
+        rhs = torch.randn(B, m, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+        x = p.stage_linear_solve(V, rhs).cpu().numpy()
+        pos, colptr, rowidx = q.pattern()
+        A = q.stage_factor(V, factor=False).cpu().numpy()
+    b = rhs.cpu().numpy()
+    for k in range(0, B, 5):
+        J = permuted_dense(colptr, rowidx, A[k], m)[np.ix_(pos, pos)]
+        r = np.abs(J @ x[k] - b[k]).max()
+        assert r <= 90 * 2.0**-24 * (np.abs(J).sum(1).max() * np.abs(x[k]).max() + np.abs(b[k]).max()), r
