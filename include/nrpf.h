@@ -53,7 +53,9 @@ extern "C" {
 #define NRPF_ORDER_NATURAL 1     /* bus order as given (tests)                  */
 #define NRPF_DENSE_AUTO 0        /* instance-major for FP32 LU with a dense block
                                     of at least NRPF_DENSE_IM_MIN unknowns and
-                                    panel 64, interleaved otherwise            */
+                                    panel 64, interleaved otherwise (solves of
+                                    at most 512 instances then still factorise
+                                    an FP32 block of panel 64 instance-major)  */
 #define NRPF_DENSE_INTERLEAVED 1 /* dense block interleaved across the 32
                                     instances of a tile (one lane each)        */
 #define NRPF_DENSE_INSTANCE_MAJOR 2 /* each instance's dense block its own

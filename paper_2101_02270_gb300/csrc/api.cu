@@ -34,6 +34,20 @@ int default_order_tries(int n) { return std::max(8, std::min(128, 512000 / std::
 constexpr double kSparseWeightFp64 = 1.5;
 constexpr double kSparseWeightFp32 = 15.0;
 
+// A solve of up to 16 tiles of a plan whose FP32 block is interleaved, for its size
+// and not by request, factorises it in the instance-major form all the same: its few and large
+// kernels (14 launches of a 320-wide factorisation against 59) cost less than the
+// interleaved ones there, whose multiply-adds are as fast but which have a lane per
+// instance and wait for each other.  Both forms are FP32 LU without pivoting; the
+// instance-major one's linear solves are nearer to FP64 (2,000 buses, first Newton
+// step: 1.6e-6 against 1.9e-6; 1,000 buses: 1.8e-6 against 5.3e-6).  Whole solves,
+// interleaved / instance-major, ms:
+//   instances         96           333          512          768          1,024
+//   500 (115 wide)    1.46 / 1.19  1.59 / 1.40  1.68 / 1.62  1.97 / 2.10  2.23 / 2.40
+//   1,000 (224)       2.23 / 1.84  3.02 / 2.94  3.40 / 3.38  3.93 / 4.34  4.48 / 5.02
+//   2,000 (308)       4.24 / 3.22  6.49 / 5.48  8.94 / 8.08  9.45 / 9.04  10.9 / 10.6
+constexpr int kFewTiles = 16;
+
 #define CK(call)                                   \
   do {                                             \
     cudaError_t e_ = (call);                       \
@@ -82,6 +96,7 @@ void free_ws(pf_plan* p) {
   p->yv_cap = 0;
   for (void* a : p->ws_allocs) cudaFree(a);
   p->ws_allocs.clear();
+  p->few_inv = nullptr;
   p->capacity = 0;
   p->st = DevState{};
 }
@@ -143,6 +158,18 @@ int ensure_capacity(pf_plan* p, int B) {
   AL(sizeof(nrpf::SolveCtl), ctl, nrpf::SolveCtl*);
 #undef AL
   CK(cudaMemset(s.ctl, 0, sizeof(nrpf::SolveCtl)));
+  // Solves of up to kFewTiles factorise an interleaved FP32 block instance-major;
+  // without the memory for the inverses they keep to the layout
+  if (p->few_im) {
+    void* d = nullptr;
+    const size_t n = (size_t)std::min(Bp, kFewTiles * kTile);
+    if (cudaMalloc(&d, n * 2 * 64 * 64 * sizeof(float)) != cudaSuccess) {
+      cudaGetLastError();
+    } else {
+      p->ws_allocs.push_back(d);
+      if (nrpf::make_dense_im_maps(p->dp, s.lu, Bp, &p->im_maps)) p->few_inv = d;
+    }
+  }
   if (p->dp.dim && h.ndp > 0) {
     // TMA descriptors of this workspace's dense blocks
     if (!nrpf::make_dense_im_maps(p->dp, s.lu, Bp, &p->im_maps)) {
@@ -162,20 +189,26 @@ int ensure_capacity(pf_plan* p, int B) {
 // refactorisation, FS/BS and update (gated by this check), and the tail that
 // advances the loop control.
 template <typename T>
-void enqueue_body(pf_plan* p, const DevState& S, cudaStream_t st, nrpf::Recorder* rec,
+void enqueue_body(pf_plan* p, DevState S, cudaStream_t st, nrpf::Recorder* rec,
                   cudaGraphConditionalHandle cond, int graph) {
-  const DevPlan& P = p->dp;
+  DevPlan P = p->dp;
   const HostPlan& h = p->hp;
   const int32_t* prev = nrpf::ctl_prev(S);
   const int32_t* cur = nrpf::ctl_cur(S);
   const bool small = P.n_sm_lvl > 0;  // one kernel for the whole linear solve
+  const bool dense = !nrpf::dense_cluster_fits(P, S, sizeof(T));
+  if (!small && dense && p->few_inv && S.Bp <= kFewTiles * kTile) {
+    P.dim = 1;
+    P.nde = P.ndp;
+    S.inv = p->few_inv;
+    S.im_maps = &p->im_maps;
+  }
   nrpf::launch_prepare_lu<T>(P, S, prev, st, rec, small);
   nrpf::launch_mismatch<T>(P, S, 1, prev, st, rec);
   nrpf::launch_check(S, st, rec);
   if (small) {
     nrpf::launch_small_solve<T>(P, S, cur, st, rec);
   } else {
-    const bool dense = !nrpf::dense_cluster_fits(P, S, sizeof(T));
     nrpf::launch_factor<T>(P, S, h.lu_lvl_ptr, cur, st, rec, dense);
     nrpf::launch_solve<T>(P, S, h.fw_lvl_ptr, h.bw_lvl_ptr, cur, st, rec, dense);
   }
@@ -441,6 +474,7 @@ int pf_plan_create(int n, const int32_t* rowptr, const int32_t* colidx, const do
   // kernels to pay (a 128 x 128 tile of C per CTA)
   p->dp.dim = o.dense_layout == NRPF_DENSE_INSTANCE_MAJOR ||
               (o.dense_layout == NRPF_DENSE_AUTO && im_ok && p->hp.nd >= NRPF_DENSE_IM_MIN);
+  p->few_im = o.dense_layout == NRPF_DENSE_AUTO && im_ok && !p->dp.dim && p->hp.nd > 0;
   if (p->host_only) {
     *out = p;
     return NRPF_OK;

@@ -23,6 +23,8 @@ struct pf_plan {
   std::vector<void*> ws_allocs;
   int64_t* d_pattern_map = nullptr;  // CCS pattern -> LU element
   nrpf::DenseImMaps im_maps{};       // TMA descriptors of the workspace (instance-major dense block)
+  bool few_im = false;               // solves of few instances factorise the block instance-major
+  void* few_inv = nullptr;           // inverse diagonal factors for that, or null
   int64_t pattern_nnz = 0;
   nrpf::Recorder rec;
   // Newton loop as a graph: one iteration captured as the body of a WHILE

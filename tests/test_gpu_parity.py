@@ -512,3 +512,31 @@ def test_interleaved_fp32_block_by_panels(n, branches, panel):
         J = permuted_dense(colptr, rowidx, A[k], m)[np.ix_(pos, pos)]
         r = np.abs(J @ x[k] - b[k]).max()
         assert r <= 90 * 2.0**-24 * (np.abs(J).sum(1).max() * np.abs(x[k]).max() + np.abs(b[k]).max()), r
+
+
+@pytest.mark.parametrize("n,branches", [(300, 400), (420, 590), (1000, 1500)])
+def test_few_instances_of_an_interleaved_block(n, branches):
+    """Up to 512 instances a solve factorises an FP32 block that is interleaved
+    for its size in the instance-major form.  One workspace, batches on both sides
+    of the limits, staged solves (interleaved) in between: every solve has the
+    oracle's voltages, a NaN injection fails alone, and a batch solved again after
+    the others has the same result, bit for bit."""
+    import gridgen
+    g = gridgen.make_grid("mesh2000_b10k", 0, n=n, n_branch=branches, n_pv=n // 10, load_scale=1 / 16)
+    sc = gridgen.make_scenarios(g, 513, 0.6, 1.4)
+    S, V0 = sc.sbus(g), sc.v0_flat(g)
+    S[40, 5] = np.nan
+    idx = [0, 39, 41, 64]
+    Vo, ito, sto = _oracle_solve(g, S, V0, idx=idx)
+    first = {}
+    with _plan(g, lu_precision="fp32") as p:
+        assert p.info["dense_layout"] == 1
+        for B in (513, 65, 512, 513, 65):
+            v, it, st = p.solve(_dev(S[:B]), _dev(V0[:B]), TOL, 10)
+            Vg, itg, stg = v.cpu().numpy(), it.cpu().numpy(), st.cpu().numpy()
+            assert np.array_equal(np.flatnonzero(stg), [40]) and stg[40] == 2
+            _compare_newton(g, Vg[idx], itg[idx], stg[idx], Vo, ito, sto, S[idx], check_iters=False)
+            f = first.setdefault(B, (Vg, itg))
+            assert np.array_equal(f[0], Vg, equal_nan=True) and np.array_equal(f[1], itg)
+            x = p.stage_linear_solve(v[:36], torch.ones(36, p.info["m"], dtype=torch.float64, device="cuda"))
+            assert torch.isfinite(x).all()
