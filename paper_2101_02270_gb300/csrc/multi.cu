@@ -11,11 +11,23 @@
 // launch's dynamic shared memory, otherwise in a private global slot.  The
 // memset of the counter and the kernel are captured once in a CUDA graph and
 // replayed.  Plans must have no dense block (create them with dense_frac >= 1).
+//
+// What bounds it: the FP64 pipe (436 instructions per bus, 32 scenarios and Newton
+// iteration of mismatch and update, each 64 cycles of a quarter of an SM: 4 ms for 256
+// feeders of 20 to 400 buses x 100 scenarios) and the latency of the levels' chains of
+// index, value and store, which the other CTAs of an SM cover.  So: no magnitude or
+// finiteness test in FP64, no FP64 instruction with few lanes (four entries in flight
+// per lane, predicated, took 8.7 ms), few registers (64: sixteen CTAs of four warps),
+// the plan's pointers in registers and its arrays read as constants (a store to the
+// state made every one of them be read again), and items in the order of their time.
+// That case, FP32 / FP64 LU: 7.4 / 9.2 ms before these, 6.6 / 8.7 with the reads, 6.1 /
+// 8.1 with the order, 5.9 / 7.9 ms without the tests.
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
 #include <cstdint>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -60,12 +72,19 @@ inline size_t state_bytes(const nrpf::HostPlan& h, int S, size_t w) {
   return (b + 255) / 256 * 256;
 }
 
+// Magnitudes and finiteness without the FP64 pipe, which is the busiest one here
+__device__ __forceinline__ unsigned long long magnitude(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ bool finite(float x) { return fabsf(x) <= FLT_MAX; }
+__device__ __forceinline__ bool finite(double x) { return magnitude(x) < 0x7ff0000000000000ull; }
+
 // One item's whole Newton loop.  base: its state (shared or global memory).
 template <typename T>
 __device__ __forceinline__ void run_item(const DevMulti& M, const Item& it, char* base, const double2* __restrict__ sbus,
                                          const double2* __restrict__ v0, double tol, int maxit,
                                          double2* __restrict__ vout, int32_t* __restrict__ iters_out,
-                                         uint8_t* __restrict__ status_out, double* s_red, int* s_bad) {
+                                         uint8_t* __restrict__ status_out, unsigned long long* s_red, int* s_bad) {
   const int lane = threadIdx.x, warp = threadIdx.y, W = blockDim.y;
   const int tid = warp * 32 + lane, nthr = 32 * W;
   const int ls = M.log_s, S = 1 << ls;
@@ -83,6 +102,12 @@ __device__ __forceinline__ void run_item(const DevMulti& M, const Item& it, char
   double* qsp = psp + (size_t)n * S;
   T* X = reinterpret_cast<T*>(qsp + (size_t)n * S);
   T* LU = X + (size_t)P.mp * S;
+  // the plan's arrays, in registers: a store to the state does not make them change
+  const int8_t* __restrict__ bus_type = P.bus_type;
+  const int32_t *__restrict__ rowptr = P.rowptr, *__restrict__ colidx = P.colidx;
+  const double *__restrict__ yre = P.yre, *__restrict__ yim = P.yim;
+  const int4* __restrict__ jmap = reinterpret_cast<const int4*>(P.jmap);
+  const int32_t *__restrict__ rhs_p = P.rhs_p, *__restrict__ rhs_q = P.rhs_q, *__restrict__ ydiag = P.ydiag;
   auto at = [&](int64_t e) -> int64_t { return (e << ls) + sc; };
   const bool valid = sc < it.nb;
   const int64_t gbase = M.in_off[it.plan] + (int64_t)(it.b0 + sc) * n;
@@ -111,23 +136,27 @@ __device__ __forceinline__ void run_item(const DevMulti& M, const Item& it, char
   __syncthreads();
   for (int itn = 0;; ++itn) {
     // ---- zero the LU values, then mismatch + Jacobian (Alg. 1, Sec. 3.1.2) ----
-    for (int64_t e = tid; e < P.NLU * S; e += nthr) LU[e] = (T)0;
+    {
+      const int64_t nz = P.NLU * S;
+      for (int64_t e = tid; e < nz; e += nthr) LU[e] = (T)0;
+    }
     __syncthreads();
-    double nrm = 0.0;
+    unsigned long long nrm = 0;  // max |F| as bits, which order as the magnitudes do (NaN last)
     for (int i = wk; i < n; i += nw) {
-      const int bt = P.bus_type[i];
+      const int bt = __ldg(bus_type + i);
       if (bt == 3) continue;
       const double ei = ve[at(i)], fi = vf[at(i)];
       double Ir = 0.0, Ii = 0.0;
-      for (int d = P.rowptr[i]; d < P.rowptr[i + 1]; ++d) {
-        const int k = P.colidx[d];
-        const double G = P.yre[d], Bv = P.yim[d];
+      const int d1 = __ldg(rowptr + i + 1);
+      for (int d = __ldg(rowptr + i); d < d1; ++d) {
+        const int k = __ldg(colidx + d);
+        const double G = __ldg(yre + d), Bv = __ldg(yim + d);
         const double ek = ve[at(k)], fk = vf[at(k)];
         const double yr = G * ek - Bv * fk, yi = G * fk + Bv * ek;
         Ir += yr;
         Ii += yi;
         if (k != i) {
-          const int4 jm = reinterpret_cast<const int4*>(P.jmap)[d];
+          const int4 jm = __ldg(jmap + d);
           if (jm.x >= 0) {
             // off-diagonal Jacobian entries in the LU precision (stored in
             // it); the mismatch stays FP64
@@ -143,39 +172,33 @@ __device__ __forceinline__ void run_item(const DevMulti& M, const Item& it, char
       const double Pc = ei * Ir + fi * Ii, Qc = fi * Ir - ei * Ii;
       const int64_t o = at(i);
       const double dP = Pc - psp[o];
-      double a = fabs(dP);
-      X[at(P.rhs_p[i])] = (T)(-dP);
+      nrm = max(nrm, magnitude(dP));
+      X[at(__ldg(rhs_p + i))] = (T)(-dP);
       if (bt == 1) {
         const double dQ = Qc - qsp[o];
-        X[at(P.rhs_q[i])] = (T)(-dQ);
-        const double q = fabs(dQ);
-        a = (q > a || q != q) ? q : a;
+        X[at(__ldg(rhs_q + i))] = (T)(-dQ);
+        nrm = max(nrm, magnitude(dQ));
       }
-      nrm = (a > nrm || a != a) ? a : nrm;
-      const int dd = P.ydiag[i];
-      const int4 jm = reinterpret_cast<const int4*>(P.jmap)[dd];
-      const double G = P.yre[dd], Bv = P.yim[dd];
+      const int dd = __ldg(ydiag + i);
+      const int4 jm = __ldg(jmap + dd);
+      const double G = __ldg(yre + dd), Bv = __ldg(yim + dd);
       const double vm2 = ei * ei + fi * fi, ivm = vinv[o], mg = vm2 * ivm;
       LU[at(jm.x)] = (T)(-Qc - Bv * vm2);
       if (jm.y >= 0) LU[at(jm.y)] = (T)(Pc * ivm + G * mg);
       if (jm.z >= 0) LU[at(jm.z)] = (T)(Pc - G * vm2);
       if (jm.w >= 0) LU[at(jm.w)] = (T)(Qc * ivm - Bv * mg);
     }
-    if (!(nrm <= DBL_MAX)) nrm = __longlong_as_double(0x7ff0000000000000ll);
     // max over the workers of each scenario: within the warp (lanes of the
     // same scenario differ in the bits above log S), then across warps
     for (int off = S; off < 32; off <<= 1) {
-      const double o2 = __shfl_xor_sync(0xffffffffu, nrm, off);
-      nrm = (o2 > nrm || o2 != o2) ? o2 : nrm;
+      nrm = max(nrm, __shfl_xor_sync(0xffffffffu, nrm, off));
     }
     if (lane < S) s_red[warp * 32 + lane] = nrm;
     __syncthreads();
     // ---- convergence test (every thread computes its scenario's outcome) ----
-    double tot = s_red[sc];
-    for (int w = 1; w < W; ++w) {
-      const double o2 = s_red[w * 32 + sc];
-      tot = (o2 > tot || o2 != o2) ? o2 : tot;
-    }
+    nrm = s_red[sc];
+    for (int w = 1; w < W; ++w) nrm = max(nrm, s_red[w * 32 + sc]);
+    const double tot = __longlong_as_double((long long)nrm);
     if (act) {
       if (s_bad[sc]) {
         my_status = NRPF_FAILED_CODE;
@@ -199,58 +222,86 @@ __device__ __forceinline__ void run_item(const DevMulti& M, const Item& it, char
     }
     if (!__syncthreads_or(act)) break;
     // ---- sparse left-looking refactor, level by level ----
-    for (int l = 0; l < P.n_lu_lvl; ++l) {
-      const int c0 = P.lu_lvl_ptr[l], c1 = P.lu_lvl_ptr[l + 1];
-      for (int ci = c0 + wk; ci < c1; ci += nw) {
-        const int j = P.lu_cols[ci];
-        for (int u = P.col_upd_ptr[j]; u < P.col_upd_ptr[j + 1]; ++u) {
-          const DevUpd up = P.upd[u];
-          const T x = LU[at(up.ukj)];
-          const int32_t* dst = P.dst + up.dst_off;
-          for (int q = 0; q < up.llen; ++q) LU[at(dst[q])] -= x * LU[at(up.lsrc + q)];
+    {
+      const int nl = P.n_lu_lvl;
+      const int32_t *__restrict__ lp = P.lu_lvl_ptr, *__restrict__ cols = P.lu_cols, *__restrict__ up0 = P.col_upd_ptr,
+                    *__restrict__ dsts = P.dst, *__restrict__ dps = P.dp;
+      static_assert(sizeof(DevUpd) == sizeof(int4), "read as one");
+      const int4* __restrict__ upds = reinterpret_cast<const int4*>(P.upd);
+      const int64_t* __restrict__ ces = P.ce;
+      int c1 = nl > 0 ? __ldg(lp) : 0;
+      for (int l = 0; l < nl; ++l) {
+        const int c0 = c1;
+        c1 = __ldg(lp + l + 1);
+        for (int ci = c0 + wk; ci < c1; ci += nw) {
+          const int j = __ldg(cols + ci);
+          const int u0 = __ldg(up0 + j), u1 = __ldg(up0 + j + 1), dpj = __ldg(dps + j);
+          const int cej = (int)__ldg(ces + j);
+          int4 nup = u0 < u1 ? __ldg(upds + u0) : make_int4(0, 0, 0, 0);
+          for (int u = u0; u < u1; ++u) {
+            const int4 up = nup;  // U(k, j), first row of L(., k), rows, destinations
+            if (u + 1 < u1) nup = __ldg(upds + u + 1);
+            const T x = LU[at(up.x)];
+            for (int q = 0; q < up.z; ++q) {
+              T* d = LU + at(__ldg(dsts + up.w + q));
+              *d -= x * LU[at(up.y + q)];
+            }
+          }
+          if (dpj >= 0) {
+            const T inv = (T)1 / LU[at(dpj)];
+            for (int p = dpj + 1; p < cej; ++p) LU[at(p)] *= inv;
+          }
         }
-        const int dpj = P.dp[j];
-        if (dpj >= 0) {
-          const T inv = (T)1 / LU[at(dpj)];
-          for (int64_t p = dpj + 1; p < P.ce[j]; ++p) LU[at(p)] *= inv;
-        }
+        __syncthreads();
       }
-      __syncthreads();
     }
     // ---- forward / backward substitution ----
-    for (int l = 0; l < P.n_fw_lvl; ++l) {
-      const int r0 = P.fw_lvl_ptr[l], r1 = P.fw_lvl_ptr[l + 1];
-      for (int ri = r0 + wk; ri < r1; ri += nw) {
-        const int i = P.fw_rows[ri];
-        T acc = X[at(i)];
-        for (int e = P.fw_ptr[ri]; e < P.fw_ptr[ri + 1]; ++e) acc -= LU[at(P.fw_pos[e])] * X[at(P.fw_col[e])];
-        X[at(i)] = acc;
+    // a worker's next row comes ahead of the barrier
+    auto substitute = [&](auto dir, int nl, const int32_t* __restrict__ lp, const int32_t* __restrict__ rows,
+                          const int32_t* __restrict__ ptr, const int32_t* __restrict__ pos,
+                          const int32_t* __restrict__ col) {
+      constexpr bool backward = decltype(dir)::value;
+      const int32_t* __restrict__ dps = P.dp;
+      const int total = nl > 0 ? __ldg(lp + nl) : 0;
+      int nt = -1, ni = 0, n0 = 0, n1 = 0, nd = 0;
+      auto fetch = [&](int t) {
+        nt = t;
+        if (t >= total) return;
+        ni = __ldg(rows + t);
+        n0 = __ldg(ptr + t);
+        n1 = __ldg(ptr + t + 1);
+        if (backward) nd = __ldg(dps + ni);
+      };
+      int r1 = nl > 0 ? __ldg(lp) : 0;
+      for (int l = 0; l < nl; ++l) {
+        const int r0 = r1;
+        r1 = __ldg(lp + l + 1);
+        for (int ri = r0 + wk; ri < r1; ri += nw) {
+          if (nt != ri) fetch(ri);
+          const int i = ni, e0 = n0, e1 = n1, dp = nd;
+          fetch(ri + nw < r1 ? ri + nw : r1 + wk);
+          T acc = X[at(i)], piv = backward ? LU[at(dp)] : (T)1;
+          for (int e = e0; e < e1; ++e) acc -= LU[at(__ldg(pos + e))] * X[at(__ldg(col + e))];
+          X[at(i)] = backward ? acc / piv : acc;
+        }
+        __syncthreads();
       }
-      __syncthreads();
-    }
-    for (int l = 0; l < P.n_bw_lvl; ++l) {
-      const int r0 = P.bw_lvl_ptr[l], r1 = P.bw_lvl_ptr[l + 1];
-      for (int ri = r0 + wk; ri < r1; ri += nw) {
-        const int i = P.bw_rows[ri];
-        T acc = X[at(i)];
-        for (int e = P.bw_ptr[ri]; e < P.bw_ptr[ri + 1]; ++e) acc -= LU[at(P.bw_pos[e])] * X[at(P.bw_col[e])];
-        X[at(i)] = acc / LU[at(P.dp[i])];
-      }
-      __syncthreads();
-    }
+    };
+    substitute(std::false_type(), P.n_fw_lvl, P.fw_lvl_ptr, P.fw_rows, P.fw_ptr, P.fw_pos, P.fw_col);
+    substitute(std::true_type(), P.n_bw_lvl, P.bw_lvl_ptr, P.bw_rows, P.bw_ptr, P.bw_pos, P.bw_col);
     // ---- voltage update (Sec. 3 step 4) ----
     if (act) {
       for (int i = wk; i < n; i += nw) {
-        const int bt = P.bus_type[i];
+        const int bt = __ldg(bus_type + i);
         if (bt == 3) continue;
         const int64_t o = at(i);
-        const double dth = (double)X[at(P.rhs_p[i])];
-        double a = va[o] + dth, g = vm[o];
-        bool ok = fabs(dth) <= DBL_MAX;
+        const T dth = X[at(__ldg(rhs_p + i))];
+        double a = va[o] + (double)dth, g = vm[o];
+        bool ok = finite(dth);
         if (bt == 1) {
-          const double dv = (double)X[at(P.rhs_q[i])];
-          ok = ok && fabs(dv) <= DBL_MAX;
-          g += dv;
+          const T dv = X[at(__ldg(rhs_q + i))];
+          ok = ok && finite(dv);
+          g += (double)dv;
         }
         if (!ok) {
           s_bad[sc] = 1;
@@ -280,13 +331,13 @@ __device__ __forceinline__ void run_item(const DevMulti& M, const Item& it, char
 }
 
 template <typename T>
-__global__ void __launch_bounds__(32 * kMaxWarps) k_multi(DevMulti M, const double2* __restrict__ sbus,
+__global__ void __launch_bounds__(32 * kMaxWarps, 2) k_multi(DevMulti M, const double2* __restrict__ sbus,
                                                           const double2* __restrict__ v0, double tol, int maxit,
                                                           double2* __restrict__ vout, int32_t* __restrict__ iters_out,
                                                           uint8_t* __restrict__ status_out) {
   extern __shared__ __align__(16) unsigned char msm[];
   __shared__ int s_item;
-  __shared__ double s_red[kMaxWarps * 32];
+  __shared__ unsigned long long s_red[kMaxWarps * 32];
   __shared__ int s_bad[32];
   const int tid = threadIdx.y * 32 + threadIdx.x;
   char* slot = M.ws + (size_t)blockIdx.x * M.slot_bytes;
@@ -381,10 +432,14 @@ int build_items(pf_multi* mp, int S, int use_smem) {
     const size_t b = state_bytes(h, S, w);
     const int sm = smem > 0 && b <= smem;
     if (!sm) slot = std::max(slot, b);
-    const double work = h.lu_fma + h.solve_fma + 16.0 * (double)h.colidx.size();
+    // Time of an iteration in thousands of cycles, eight CTAs per SM, as measured:
+    // mostly levels, and buses.  By multiply-adds, deep and narrow grids came late
+    // and the last of them ran alone (the last CTA 15 % after the average one).
+    const double work = 24.0 * (double)h.lu_lvl_ptr.size() +
+                        6.0 * (double)(h.fw_lvl_ptr.size() + h.bw_lvl_ptr.size()) + 3.0 * (double)h.n;
     for (int b0 = 0; b0 < mp->batch[f]; b0 += S) {
       Item it{f, b0, std::min(S, mp->batch[f] - b0), sm};
-      items.push_back({work * it.nb, it});
+      items.push_back({work, it});
       in_smem += sm;
     }
   }

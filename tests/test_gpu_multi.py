@@ -138,3 +138,31 @@ def test_multi_rejects_bad_groups():
     p32 = pf.Plan.from_branches(g.n, g.f, g.t, g.r, g.x, g.b, g.bus_type, dense_frac=1.0, lu_precision="fp32")
     with pytest.raises(pf.NrpfError):
         pf.MultiPlan([p64, p32], [4, 4])
+
+
+@pytest.mark.parametrize("lu", ["fp64", "fp32"])
+@pytest.mark.parametrize("per_item,warps", [(32, 1), (32, 8), (2, 4)])
+def test_multi_failing_scenarios_fail_alone(lu, per_item, warps):
+    """The largest mismatch is found among magnitudes of every kind, by every split
+    of the buses: a NaN, an infinite and a huge injection each fail their own
+    scenario, one that is solved at the start takes no iteration, and the
+    others are the oracle's."""
+    fs, scen = _feeders([(37,), (5,), (21,)])
+    plans, mp, S, V0, Sc, Vc = _group(fs, scen, lu)
+    mp.set_scenarios(per_item, False)
+    mp.set_config(warps, 2)
+    v, it, st = mp.solve(Sc, Vc, TOL, 10)
+    _check(fs, S, V0, v, it, st, lu == "fp64")
+    n = fs[0].n
+    Sc[3 * n + n - 1] = complex("nan")
+    Sc[11 * n + 1] = complex("inf")
+    Sc[20 * n + 2] = -1e300
+    Vc[5 * n:6 * n] = v[5 * n:6 * n]
+    v2, it2, st2 = mp.solve(Sc, Vc, TOL, 10)
+    assert all(st2[k] == 2 for k in (3, 11, 20)) and it2[5] == 0 and st2[5] == 0
+    keep = torch.ones_like(st, dtype=torch.bool)
+    keep[[3, 5, 11, 20]] = False
+    assert torch.equal(st2[keep], st[keep]) and torch.equal(it2[keep], it[keep])
+    off = 37 * n
+    assert torch.equal(v2[off:], v[off:]) and torch.equal(v2[:3 * n], v[:3 * n])
+    mp.close()
