@@ -1173,40 +1173,6 @@ __global__ void __launch_bounds__(32 * kFixWR * kFixWC, 3) k_dense_update_fixed(
 // level instead of the paper's atomicAdd scatter: every row writes only its
 // own entry, so the result is deterministic.
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void k_fwd_level(DevPlan P, DevState S, int r0, int r1, const int32_t* __restrict__ gate) {
-  if (gate && *gate == 0) return;
-  const int lane = threadIdx.x;
-  const int ri = r0 + blockIdx.x * blockDim.y + threadIdx.y;
-  const int tile = blockIdx.y;
-  if (ri >= r1) return;
-  if (!tile_active(S, tile, lane)) return;
-  const T* __restrict__ LU = reinterpret_cast<const T*>(S.lu) + (size_t)tile * P.NLU * kTile + lane;
-  T* __restrict__ X = reinterpret_cast<T*>(S.x) + (size_t)tile * P.mp * kTile + lane;
-  const int i = P.fw_rows[ri];
-  T acc = X[(size_t)i * kTile];
-  const int e0 = P.fw_ptr[ri], e1 = P.fw_ptr[ri + 1];
-  for (int e = e0; e < e1; ++e) acc -= LU[(size_t)P.fw_pos[e] * kTile] * X[(size_t)P.fw_col[e] * kTile];
-  X[(size_t)i * kTile] = acc;
-}
-
-template <typename T>
-__global__ void k_bwd_level(DevPlan P, DevState S, int r0, int r1, const int32_t* __restrict__ gate) {
-  if (gate && *gate == 0) return;
-  const int lane = threadIdx.x;
-  const int ri = r0 + blockIdx.x * blockDim.y + threadIdx.y;
-  const int tile = blockIdx.y;
-  if (ri >= r1) return;
-  if (!tile_active(S, tile, lane)) return;
-  const T* __restrict__ LU = reinterpret_cast<const T*>(S.lu) + (size_t)tile * P.NLU * kTile + lane;
-  T* __restrict__ X = reinterpret_cast<T*>(S.x) + (size_t)tile * P.mp * kTile + lane;
-  const int i = P.bw_rows[ri];
-  T acc = X[(size_t)i * kTile];
-  const int e0 = P.bw_ptr[ri], e1 = P.bw_ptr[ri + 1];
-  for (int e = e0; e < e1; ++e) acc -= LU[(size_t)P.bw_pos[e] * kTile] * X[(size_t)P.bw_col[e] * kTile];
-  X[(size_t)i * kTile] = acc / LU[(size_t)P.dp[i] * kTile];
-}
-
 // All levels of the forward (BWD: backward) schedule in one launch (see
 // k_sparse_factor): a warp per row, its entries in the order of the list, four
 // products' loads in flight; the warp's next row and that row's first four

@@ -17,7 +17,7 @@
 // feeders of 20 to 400 buses x 100 scenarios) and the latency of the levels' chains of
 // index, value and store, which the other CTAs of an SM cover.  So: no magnitude or
 // finiteness test in FP64, no FP64 instruction with few lanes (four entries in flight
-// per lane, predicated, took 8.7 ms), few registers (64: sixteen CTAs of four warps),
+// per lane, predicated, took 8.7 ms), few registers (64: eight CTAs of four warps),
 // the plan's pointers in registers and its arrays read as constants (a store to the
 // state made every one of them be read again), and items in the order of their time.
 // That case, FP32 / FP64 LU: 7.4 / 9.2 ms before these, 6.6 / 8.7 with the reads, 6.1 /
