@@ -40,10 +40,6 @@ MAXIT = 10
 # Peaks: HBM copy bandwidth from the pool's measurement file; FP64 / FP32 FMA
 # throughput measured live by pf_fma_peak (independent FMA chains on every SM).
 HBM_FALLBACK_GBS = 6800.0
-# DRAM bytes (read + write) of one k_dense_update launch per instance and per
-# trailing-matrix entry r^2, from the ncu capture summarised in
-# profiles/dense_update_fp64_mesh2000.md (batch 640, panel 8, r = 200).
-DENSE_UPDATE_DRAM_B_PER_R2 = 14.3
 
 
 def measured_hbm():
@@ -349,24 +345,13 @@ def combine_ranks(ms, converged, device):
 # ---------------------------------------------------------------------------
 # GPU arm
 # ---------------------------------------------------------------------------
-# ncu DRAM bytes over algorithmic bytes of the depth-64 FP32 trailing update
-# of the interleaved layout; None: the kernel changed (packed two-wide FMAs)
-# after the capture in profiles/dense_update_fp32_mesh2000.md (371.7 MB of
-# 419.4 MB), which is not repeated for it.
-DENSE_UPDATE_FP32_DRAM_PER_ALG = None
-
-# ncu DRAM bytes (read + write) of one k_im_gemm launch over its algorithmic
-# bytes (im_update_bytes), from the capture summarised in
-# profiles/im_gemm_mesh9000_b64.md (batch 64, outer panel 8: 739.5 MB
-# against 746.6 MB).
-IM_GEMM_DRAM_PER_ALG = 0.99
-
 KERNEL_TIMING = ("CUDA events around every dense_update launch on its stream, during a second pass of the "
                  "K timed steps")
 
 
 def dense_update_launches(ndp, kb):
-    """The k_dense_update launches of one dense refactor, each a list of the
+    """The k_dense_update launches of one dense refactor (FP64, and FP32 panels
+    below 16), each a list of the
     rectangles A[rows, cols] -= L U of depth d it updates, as (rows, cols, d).
     Panels of 4-16: one trailing update per panel.  Two-level panels (32, 64):
     per 16-wide inner step, the outer panel's columns below the step plus, for
@@ -390,16 +375,24 @@ def dense_update_launches(ndp, kb):
     return out
 
 
+def dense_update_launches_il(nde):
+    """The k_il_gemm launches of one refactor of an interleaved FP32 block with
+    panels of 16 and more: per outer panel of 64 the columns and rows of its
+    second to fourth step, each with the products of the steps before, then one
+    trailing update of depth 64.  nde: the block's unknowns rounded up to 16."""
+    out = []
+    for k in range(0, nde, 64):
+        for ki in range(k + 16, min(k + 64, nde), 16):
+            out.append([(nde - ki, 16, ki - k), (16, nde - ki - 16, ki - k)])
+        if nde - k - 64 > 0:
+            out.append([(nde - k - 64, nde - k - 64, 64)])
+    return out
+
+
 def dense_update_flop(ndp, kb):
     """Algorithmic flops of the updates of one dense refactor: 2 * rows * cols
     * depth per rectangle."""
     return sum(2 * r * c * d for L in dense_update_launches(ndp, kb) for r, c, d in L)
-
-
-def dense_update_bytes(ndp, kb, w):
-    """Algorithmic bytes of the same updates: each rectangle read and written
-    once, its two operand panels read once (w bytes a value)."""
-    return sum(w * (2 * r * c + d * (r + c)) for L in dense_update_launches(ndp, kb) for r, c, d in L)
 
 
 def run_feeders(args):
@@ -920,13 +913,11 @@ def measure_mesh(args, pf, name, lu, steps, warmup, dev, rank=0, world=1, with_c
     if im:
         du_flop = sum(2 * r * c * d for L in dense_update_launches_im(ndp) for r, c, d in L) * refactors
         achieved = du_flop / (du[2] / 1e3) / 1e12 if du[2] > 0 else None
-        alg = [im_update_bytes(ndp, kj) for kj in range(128, ndp, 128)]
-        roof = {"bound": "alu", "kernel": "dense_update (k_im_gemm, FP32 CTA-tiled product)", "achieved": achieved,
+        roof = {"bound": "alu", "kernel": "dense_update (k_im_gemm_tc, six BF16 tensor-core products per FP32 one, "
+                                          "far from the solution; k_im_gemm, FP32 FMA, near it)",
+                "achieved": achieved,
                 "peak": fp32_peak, "unit": "TFLOP/s", "frac": (achieved / fp32_peak) if achieved else None,
-                "traffic": (IM_GEMM_DRAM_PER_ALG * B * sum(alg) / len(alg)
-                            if alg and IM_GEMM_DRAM_PER_ALG is not None else None),
-                "traffic_kind": "ncu DRAM bytes over algorithmic bytes of one launch of a batch-64 capture, times "
-                                "the batch and the mean algorithmic bytes of the refactor's launches",
+                "traffic": None,
                 "peak_kind": "measured FP32 FMA-chain throughput (pf_fma_peak)",
                 "launches": du[0], "ms_total": du[2], "timing": timing,
                 "algorithmic_bytes": "per launch and instance: the panel's block column and row read and "
@@ -934,25 +925,22 @@ def measure_mesh(args, pf, name, lu, steps, warmup, dev, rank=0, world=1, with_c
     elif lu == "fp64":
         du_flop = dense_update_flop(ndp, kb) * refactors
         achieved = du_flop / (du[2] / 1e3) / 1e12 if du[2] > 0 else None
-        r2 = [(ndp - k - kb) ** 2 for k in range(0, ndp, kb) if ndp - k - kb > 0]
-        traffic = (DENSE_UPDATE_DRAM_B_PER_R2 * B * sum(r2) / len(r2) if r2 and kb == 8 else None)
-        roof = {"bound": "alu", "kernel": "dense_update", "achieved": achieved, "peak": fp64_peak,
-                "unit": "TFLOP/s", "frac": (achieved / fp64_peak) if achieved else None, "traffic": traffic,
-                "peak_kind": "measured FP64 FMA-chain throughput (pf_fma_peak)",
-                "traffic_kind": "ncu DRAM bytes per average active launch, scaled from a batch-640 capture",
+        roof = {"bound": "alu", "kernel": "dense_update (k_dense_update_fixed, integer multiply-adds in fixed point, "
+                                          "panel 8; k_dense_update, FP64 FMA, otherwise)",
+                "achieved": achieved, "peak": fp64_peak,
+                "unit": "TFLOP/s", "frac": (achieved / fp64_peak) if achieved else None, "traffic": None,
+                "peak_kind": "measured FP64 FMA-chain throughput (pf_fma_peak); the fixed-point form does not use it",
                 "launches": du[0], "ms_total": du[2], "timing": timing}
     else:
-        du_flop = dense_update_flop(ndp, kb) * refactors
+        launches = dense_update_launches_il((info["dense_dim"] + 15) // 16 * 16) if kb >= 16 else \
+            dense_update_launches(ndp, kb)
+        du_flop = sum(2 * r * c * d for L in launches for r, c, d in L) * refactors
+        du_bytes = sum(w * (2 * r * c + d * (r + c)) for L in launches for r, c, d in L) * refactors
         achieved = du_flop / (du[2] / 1e3) / 1e12 if du[2] > 0 else None
-        du_bytes = dense_update_bytes(ndp, kb, w) * refactors
-        active_launches = len(dense_update_launches(ndp, kb)) * int(iters.max()) * rsteps
         gbs = du_bytes / (du[2] / 1e3) / 1e9 if du[2] > 0 else None
         roof = {"bound": "hbm", "kernel": "dense_update", "achieved": gbs, "peak": hbm, "unit": "GB/s",
                 "frac": (gbs / hbm) if gbs else None,
-                "traffic": (DENSE_UPDATE_FP32_DRAM_PER_ALG * du_bytes / max(active_launches, 1)
-                            if DENSE_UPDATE_FP32_DRAM_PER_ALG is not None else None),
-                "traffic_kind": "ncu DRAM bytes / algorithmic bytes of a batch-640 depth-64 capture, times the "
-                                "algorithmic bytes per launch",
+                "traffic": None,
                 "peak_kind": f"{hbm_kind} HBM copy bandwidth", "fp32_tflops": achieved, "fp32_peak_tflops": fp32_peak,
                 "launches": du[0], "ms_total": du[2], "timing": timing}
     # whole-step HBM roofline (metric's second half): algorithmic bytes per
