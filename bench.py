@@ -918,7 +918,7 @@ def measure_mesh(args, pf, name, lu, steps, warmup, dev, rank=0, world=1, with_c
                 "achieved": achieved,
                 "peak": fp32_peak, "unit": "TFLOP/s", "frac": (achieved / fp32_peak) if achieved else None,
                 "traffic": None,
-                "peak_kind": "measured FP32 FMA-chain throughput (pf_fma_peak)",
+                "peak_kind": "measured FP32 FMA-chain throughput (pf_fma_peak); the tensor-core form does not use it",
                 "launches": du[0], "ms_total": du[2], "timing": timing,
                 "algorithmic_bytes": "per launch and instance: the panel's block column and row read and "
                                      "written once, the operands L(kj:, :kj) and U(:kj, kj:) read once"}
