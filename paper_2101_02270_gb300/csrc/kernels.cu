@@ -1115,14 +1115,18 @@ __global__ void __launch_bounds__(32 * kFixWR * kFixWC, 3) k_dense_update_fixed(
       hl[r][q] = 1ll << 27;  // rounds hl / 2^28
     }
   __syncthreads();  // the barrier is initialised
-  uint32_t ok = 0;
-  for (uint32_t spins = 0; !ok && spins < kFixSpinLimit; ++spins)
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(sb)
-        : "memory");
-  if (__syncthreads_or(!ok)) {  // a copy did not land in time: the step is discarded
+  auto wait = [&] {
+    uint32_t ok = 0;
+    for (uint32_t spins = 0; !ok && spins < kFixSpinLimit; ++spins)
+      asm volatile(
+          "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}\n"
+          : "=r"(ok)
+          : "r"(sb)
+          : "memory");
+    return ok != 0;
+  };
+  if (__syncthreads_or(!wait())) {  // a copy did not land in time: the step is discarded
+    wait();  // no copy of this CTA's may land after it
     S.bad[tile * kTile + lane] = 1;
     return;
   }
