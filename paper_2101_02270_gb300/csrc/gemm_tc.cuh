@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kGemmTmaThreads, 2) k_gemm_tma(const __grid_co
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   __shared__ __align__(8) uint64_t full[G::kStages], empty[G::kStages], done;
   __shared__ uint32_t tmem_holder;
-  __shared__ int s_fail;
+  __shared__ int s_fail, s_issued;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m0 = blockIdx.y * kGemmBM, n0 = blockIdx.x * BN;
   const int nk = K / kGemmBK;
@@ -359,7 +359,8 @@ __global__ void __launch_bounds__(kGemmTmaThreads, 2) k_gemm_tma(const __grid_co
   const uint32_t base = smem_u32(smem);
   if (warp == 0 && lane == 0) {
     // producer
-    for (int kc = 0; kc < nk; ++kc) {
+    int kc = 0;
+    for (; kc < nk; ++kc) {
       const int s = kc % G::kStages;
       if (kc >= G::kStages && !mbar_wait(&empty[s], ((kc / G::kStages) - 1) & 1)) {
         s_fail = 1;
@@ -382,6 +383,7 @@ __global__ void __launch_bounds__(kGemmTmaThreads, 2) k_gemm_tma(const __grid_co
         tma_load_2d(sb, &tmB, kc * kGemmBK, n0, &full[s]);
       }
     }
+    s_issued = kc;
   } else if (warp == 1 && lane == 0) {
     // MMA issuer
     constexpr uint32_t idesc = make_idesc_bf16(kGemmBM, BN, AT, BT);
@@ -409,7 +411,13 @@ __global__ void __launch_bounds__(kGemmTmaThreads, 2) k_gemm_tma(const __grid_co
   if (!got) s_fail = 1;
   __syncthreads();
   if (s_fail) {
-    if (tid == 0) atomicExch(err, 1);
+    if (tid == 0) {
+      atomicExch(err, 1);
+      // no load of this CTA's may land, and no product end, after it has left
+      for (int kc = max(0, s_issued - G::kStages); kc < s_issued; ++kc)
+        mbar_wait(&full[kc % G::kStages], (kc / G::kStages) & 1);
+      mbar_wait(&done, 0);
+    }
   } else {
     float* tr = reinterpret_cast<float*>(smem) + warp * (32 * 33);
     const int rg = warp & 3, row0 = m0 + rg * 32;

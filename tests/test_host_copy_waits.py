@@ -38,6 +38,7 @@ def _source(name):
     ("dense_il.cu", "k_il_gemm(", r"if \(__syncthreads_or\(!"),
     ("dense_im.cu", " update_fma(", r"if \(fail >= 0"),
     ("dense_im.cu", " update_tc(", r"if \(__syncthreads_or\(!ok \|\|"),
+    ("gemm_tc.cuh", " k_gemm_tma(", r"if \(s_fail\)"),
 ])
 def test_a_failed_wait_waits_for_what_is_in_flight(name, kernel, failed):
     body = _block(_source(name), _source(name).index(kernel))
