@@ -67,17 +67,20 @@ int upload(pf_plan* p, const std::vector<T>& v, const T** out) {
   return NRPF_OK;
 }
 
-// Fold the launches made by loop graphs (one body's launches x bodies run)
-// into the counters and zero the device count.  Synchronises the device.
+// Fold the launches made by loop graphs (each graph's launches per body x
+// bodies run) into the counters and zero the device counts.  Synchronises the
+// device.
 void fold_graph_launches(pf_plan* p) {
   if (!p->st.ctl) return;
   cudaDeviceSynchronize();
-  long long gi = 0;
+  long long gi[nrpf::kLoopSlots];
   char* f = reinterpret_cast<char*>(p->st.ctl) + offsetof(nrpf::SolveCtl, graph_iters);
-  if (cudaMemcpy(&gi, f, sizeof(gi), cudaMemcpyDeviceToHost) != cudaSuccess) return;
-  for (int c = 0; c < nrpf::K_NCLASS; ++c) p->rec.launches[c] += p->body_launches[c] * gi;
-  const long long zero = 0;
-  cudaMemcpy(f, &zero, sizeof(zero), cudaMemcpyHostToDevice);
+  if (cudaMemcpy(gi, f, sizeof(gi), cudaMemcpyDeviceToHost) != cudaSuccess) return;
+  for (const auto& kv : p->loops)
+    for (int c = 0; c < nrpf::K_NCLASS; ++c)
+      p->rec.launches[c] += kv.second.body_launches[c] * gi[kv.second.slot];
+  std::fill(gi, gi + nrpf::kLoopSlots, 0);
+  cudaMemcpy(f, gi, sizeof(gi), cudaMemcpyHostToDevice);
 }
 
 void destroy_loop_graphs(pf_plan* p) {
@@ -228,7 +231,13 @@ int ensure_loop_graph(pf_plan* p, const DevState& S, cudaGraphExec_t* out) {
     *out = it->second.exec;
     return NRPF_OK;
   }
+  if (p->loops.size() == (size_t)nrpf::kLoopSlots) {
+    // every slot is taken: count what the graphs ran and start over
+    fold_graph_launches(p);
+    destroy_loop_graphs(p);
+  }
   if (!p->capture_stream) CK(cudaStreamCreateWithFlags(&p->capture_stream, cudaStreamNonBlocking));
+  const int slot = (int)p->loops.size();
   cudaGraph_t g = nullptr;
   CK(cudaGraphCreate(&g, 0));
   auto fail = [&](cudaError_t e) {
@@ -250,7 +259,7 @@ int ensure_loop_graph(pf_plan* p, const DevState& S, cudaGraphExec_t* out) {
   e = cudaStreamBeginCaptureToGraph(p->capture_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
   if (e != cudaSuccess) return fail(e);
   nrpf::Recorder count;  // launches of one body, by class
-  enqueue_body<T>(p, S, p->capture_stream, &count, cond, 1);
+  enqueue_body<T>(p, S, p->capture_stream, &count, cond, slot + 1);
   cudaGraph_t captured = nullptr;
   const cudaError_t el = cudaGetLastError();
   e = cudaStreamEndCapture(p->capture_stream, &captured);
@@ -258,8 +267,11 @@ int ensure_loop_graph(pf_plan* p, const DevState& S, cudaGraphExec_t* out) {
   if (e != cudaSuccess) return fail(e);
   cudaGraphExec_t exec = nullptr;
   if ((e = cudaGraphInstantiate(&exec, g, 0)) != cudaSuccess) return fail(e);
-  p->loops[key] = pf_plan::LoopGraph{g, exec};
-  for (int c = 0; c < nrpf::K_NCLASS; ++c) p->body_launches[c] = count.launches[c];
+  pf_plan::LoopGraph& lg = p->loops[key];
+  lg.graph = g;
+  lg.exec = exec;
+  lg.slot = slot;
+  std::copy(count.launches, count.launches + nrpf::K_NCLASS, lg.body_launches);
   *out = exec;
   return NRPF_OK;
 }

@@ -87,6 +87,7 @@ struct DevPlan {
 // Device-resident control of the Newton loop, so that one iteration can run
 // unchanged from a graph: every kernel of an iteration reads its gate and the
 // iteration number here.
+constexpr int kLoopSlots = 64;  // loop graphs kept per workspace, one per padded batch size and kind of admittances
 struct SolveCtl {
   int32_t prev;     // instances active after the previous check: gate of the
                     // LU preparation and mismatch (nonzero before the first)
@@ -95,7 +96,7 @@ struct SolveCtl {
   int32_t it;       // Newton iteration of the check
   int32_t maxit;
   double tol;
-  long long graph_iters;  // loop bodies run by the graph since the last reset
+  long long graph_iters[kLoopSlots];  // loop bodies run by each loop graph since the last reset
 };
 
 struct DevState {

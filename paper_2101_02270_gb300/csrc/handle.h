@@ -29,14 +29,17 @@ struct pf_plan {
   nrpf::Recorder rec;
   // Newton loop as a graph: one iteration captured as the body of a WHILE
   // node whose condition the iteration's last kernel sets (built per
-  // workspace; launches of one body by kernel class, for the counters)
+  // workspace).  Which kernels a body launches depends on the batch, so each
+  // graph has its own launches per body, by kernel class, and its own device
+  // count of bodies run (SolveCtl::graph_iters[slot])
   struct LoopGraph {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+    int slot = 0;
+    int64_t body_launches[nrpf::K_NCLASS] = {};
   };
   std::map<int, LoopGraph> loops;  // by 2 x padded batch + per-instance Ybus flag
   cudaStream_t capture_stream = nullptr;
-  int64_t body_launches[nrpf::K_NCLASS] = {};
   int32_t* h_prev = nullptr;  // pinned: ctl->prev read back by profiled solves
   // host-resident batches: two device staging slots of stage_cap instances,
   // a copy stream and the events that order copies and solves

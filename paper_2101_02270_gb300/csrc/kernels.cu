@@ -326,7 +326,7 @@ __global__ void k_iter_tail(SolveCtl* c, cudaGraphConditionalHandle cond, int gr
   c->cur = 0;
   c->it += 1;
   if (graph) {
-    c->graph_iters += 1;
+    c->graph_iters[graph - 1] += 1;
     cudaGraphSetConditional(cond, (cur > 0 && c->it < c->maxit) ? 1u : 0u);
   }
 }

@@ -59,6 +59,7 @@ void launch_ctl_init(const DevState& S, int maxit, double tol, cudaStream_t st, 
 void launch_check(const DevState& S, cudaStream_t st, Recorder* rec = nullptr);
 // End of one iteration: prev = cur, cur = 0, it += 1; with a graph handle
 // (graph != 0), also sets the loop's condition to (cur > 0 && it < maxit).
+// graph: 0, or 1 + the loop graph's slot in SolveCtl::graph_iters
 void launch_iter_tail(const DevState& S, cudaGraphConditionalHandle cond, int graph, cudaStream_t st,
                       Recorder* rec = nullptr);
 

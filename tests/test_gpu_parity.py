@@ -540,3 +540,46 @@ def test_few_instances_of_an_interleaved_block(n, branches):
             assert np.array_equal(f[0], Vg, equal_nan=True) and np.array_equal(f[1], itg)
             x = p.stage_linear_solve(v[:36], torch.ones(36, p.info["m"], dtype=torch.float64, device="cuda"))
             assert torch.isfinite(x).all()
+
+
+def test_launch_counts_of_batches_on_different_kernels():
+    """Which kernels an iteration launches depends on the batch (a cluster per
+    instance up to two tiles, sparse columns instead of entries beyond 152, per
+    loop graph): the counts of one plan that solves several sizes are the sum
+    of the counts of plans that solve one each."""
+    import gridgen
+    g = gridgen.make_grid("mesh2000_b10k", 0, n=300, n_branch=400, n_pv=30, load_scale=1 / 16)
+    sc = gridgen.make_scenarios(g, 152 * 32 + 1, 0.6, 1.4)
+    S, V0 = _dev(sc.sbus(g)), _dev(sc.v0_flat(g))
+    total = {}
+    for B in (64, len(S)):
+        with _plan(g) as p:
+            p.profile_start([])
+            p.solve(S[:B], V0[:B], TOL, 10)
+            one = {k: c[0] for k, c in p.profile_read().items()}
+        for k, c in one.items():
+            total[k] = total.get(k, 0) + (2 * c if B == 64 else c)
+    assert total["dense_update"] > 0 and total["lu_sparse_level"] > 0
+    with _plan(g) as p:
+        p.solve(S, V0, TOL, 10)  # the workspace of the largest batch, so that no graph is made anew
+        p.profile_start([])
+        for B in (64, len(S), 64):
+            p.solve(S[:B], V0[:B], TOL, 10)
+        assert {k: c[0] for k, c in p.profile_read().items()} == total
+
+
+def test_more_batch_sizes_than_loop_graphs():
+    """A plan keeps 64 loop graphs; further batch sizes start the set over, with
+    the same results and every launch counted."""
+    g, S, V0 = case("mesh30_b64", batch=64)
+    idx = np.arange(70 * 32) % 64
+    with _plan(g) as p:
+        v, it, st = p.solve(_dev(S), _dev(V0), TOL, 10)
+        Sd, Vd, k = _dev(S[idx]), _dev(V0[idx]), torch.from_numpy(idx).cuda()
+        p.solve(Sd, Vd, TOL, 10)
+        p.profile_start([])
+        for t in range(1, 71):
+            w, it2, st2 = p.solve(Sd[:32 * t], Vd[:32 * t], TOL, 10)
+            assert torch.equal(w, v[k[:32 * t]]) and torch.equal(it2, it[k[:32 * t]])
+        counts = p.profile_read()
+    assert counts["update"][0] == 70 * (int(it.max()) + 1)
