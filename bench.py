@@ -775,6 +775,48 @@ def im_update_bytes(ndp, kj):
     return 8 * entries + 8 * kj * (ndp - kj)
 
 
+def update_roofline(lu, im, info, refactors, du, fp64_peak, fp32_peak, hbm, hbm_kind, timing):
+    """The line's roofline entry of the dense updates: du is their (launches,
+    timed launches, ms), refactors the refactorisations they belong to, im
+    whether the block was factorised instance-major."""
+    w = 8 if lu == "fp64" else 4
+    ndp, kb = info["dense_pad"], info["panel"]
+    if im:
+        du_flop = sum(2 * r * c * d for L in dense_update_launches_im(ndp) for r, c, d in L) * refactors
+        achieved = du_flop / (du[2] / 1e3) / 1e12 if du[2] > 0 else None
+        roof = {"bound": "alu", "kernel": "dense_update (k_im_gemm_tc, six BF16 tensor-core products per FP32 one, "
+                                          "far from the solution; k_im_gemm, FP32 FMA, near it)",
+                "achieved": achieved,
+                "peak": fp32_peak, "unit": "TFLOP/s", "frac": (achieved / fp32_peak) if achieved else None,
+                "traffic": None,
+                "peak_kind": "measured FP32 FMA-chain throughput (pf_fma_peak); the tensor-core form does not use it",
+                "launches": du[0], "ms_total": du[2], "timing": timing,
+                "algorithmic_bytes": "per launch and instance: the panel's block column and row read and "
+                                     "written once, the operands L(kj:, :kj) and U(:kj, kj:) read once"}
+    elif lu == "fp64":
+        du_flop = dense_update_flop(ndp, kb) * refactors
+        achieved = du_flop / (du[2] / 1e3) / 1e12 if du[2] > 0 else None
+        roof = {"bound": "alu", "kernel": "dense_update (k_dense_update_fixed, integer multiply-adds in fixed point, "
+                                          "panel 8; k_dense_update, FP64 FMA, otherwise)",
+                "achieved": achieved, "peak": fp64_peak,
+                "unit": "TFLOP/s", "frac": (achieved / fp64_peak) if achieved else None, "traffic": None,
+                "peak_kind": "measured FP64 FMA-chain throughput (pf_fma_peak); the fixed-point form does not use it",
+                "launches": du[0], "ms_total": du[2], "timing": timing}
+    else:
+        rects = dense_update_launches_il((info["dense_dim"] + 15) // 16 * 16) if kb >= 16 else \
+            dense_update_launches(ndp, kb)
+        du_flop = sum(2 * r * c * d for L in rects for r, c, d in L) * refactors
+        du_bytes = sum(w * (2 * r * c + d * (r + c)) for L in rects for r, c, d in L) * refactors
+        achieved = du_flop / (du[2] / 1e3) / 1e12 if du[2] > 0 else None
+        gbs = du_bytes / (du[2] / 1e3) / 1e9 if du[2] > 0 else None
+        roof = {"bound": "hbm", "kernel": "dense_update", "achieved": gbs, "peak": hbm, "unit": "GB/s",
+                "frac": (gbs / hbm) if gbs else None,
+                "traffic": None,
+                "peak_kind": f"{hbm_kind} HBM copy bandwidth", "fp32_tflops": achieved, "fp32_peak_tflops": fp32_peak,
+                "launches": du[0], "ms_total": du[2], "timing": timing}
+    return roof
+
+
 def measure_mesh(args, pf, name, lu, steps, warmup, dev, rank=0, world=1, with_cpu=True, batch=None,
                  roof_steps=None, e2e=True):
     """One meshed-grid workload: K timed pf_solve_batch steps (graph-ended
@@ -910,39 +952,10 @@ def measure_mesh(args, pf, name, lu, steps, warmup, dev, rank=0, world=1, with_c
     hbm, hbm_kind = measured_hbm()
     timing = (f"CUDA events around every dense_update launch on its stream, during a second pass of {rsteps} of "
               f"the {steps} timed steps")
-    if im:
-        du_flop = sum(2 * r * c * d for L in dense_update_launches_im(ndp) for r, c, d in L) * refactors
-        achieved = du_flop / (du[2] / 1e3) / 1e12 if du[2] > 0 else None
-        roof = {"bound": "alu", "kernel": "dense_update (k_im_gemm_tc, six BF16 tensor-core products per FP32 one, "
-                                          "far from the solution; k_im_gemm, FP32 FMA, near it)",
-                "achieved": achieved,
-                "peak": fp32_peak, "unit": "TFLOP/s", "frac": (achieved / fp32_peak) if achieved else None,
-                "traffic": None,
-                "peak_kind": "measured FP32 FMA-chain throughput (pf_fma_peak); the tensor-core form does not use it",
-                "launches": du[0], "ms_total": du[2], "timing": timing,
-                "algorithmic_bytes": "per launch and instance: the panel's block column and row read and "
-                                     "written once, the operands L(kj:, :kj) and U(:kj, kj:) read once"}
-    elif lu == "fp64":
-        du_flop = dense_update_flop(ndp, kb) * refactors
-        achieved = du_flop / (du[2] / 1e3) / 1e12 if du[2] > 0 else None
-        roof = {"bound": "alu", "kernel": "dense_update (k_dense_update_fixed, integer multiply-adds in fixed point, "
-                                          "panel 8; k_dense_update, FP64 FMA, otherwise)",
-                "achieved": achieved, "peak": fp64_peak,
-                "unit": "TFLOP/s", "frac": (achieved / fp64_peak) if achieved else None, "traffic": None,
-                "peak_kind": "measured FP64 FMA-chain throughput (pf_fma_peak); the fixed-point form does not use it",
-                "launches": du[0], "ms_total": du[2], "timing": timing}
-    else:
-        launches = dense_update_launches_il((info["dense_dim"] + 15) // 16 * 16) if kb >= 16 else \
-            dense_update_launches(ndp, kb)
-        du_flop = sum(2 * r * c * d for L in launches for r, c, d in L) * refactors
-        du_bytes = sum(w * (2 * r * c + d * (r + c)) for L in launches for r, c, d in L) * refactors
-        achieved = du_flop / (du[2] / 1e3) / 1e12 if du[2] > 0 else None
-        gbs = du_bytes / (du[2] / 1e3) / 1e9 if du[2] > 0 else None
-        roof = {"bound": "hbm", "kernel": "dense_update", "achieved": gbs, "peak": hbm, "unit": "GB/s",
-                "frac": (gbs / hbm) if gbs else None,
-                "traffic": None,
-                "peak_kind": f"{hbm_kind} HBM copy bandwidth", "fp32_tflops": achieved, "fp32_peak_tflops": fp32_peak,
-                "launches": du[0], "ms_total": du[2], "timing": timing}
+    # solves of 65 to 512 instances factorise an FP32 block that is interleaved
+    # for its size in the instance-major form
+    few = lu == "fp32" and args.dense_layout == "auto" and kb == 64 and 64 < B <= 512
+    roof = update_roofline(lu, im or few, info, refactors, du, fp64_peak, fp32_peak, hbm, hbm_kind, timing)
     # whole-step HBM roofline (metric's second half): algorithmic bytes per
     # instance-iteration = LU written once and read once + voltages, injections,
     # rhs and solution
