@@ -583,10 +583,10 @@ def warmstart_measure(args, steps, warmup):
     prof = plan64.profile_read()
     # library launches of the timed warm solves: the plan's (solves, including
     # any flat-start fallback) plus the network's per guess: features, v0 and,
-    # per chunk of bmax instances, input scaling + three GEMMs + output scaling
+    # per chunk of bmax instances, input scaling + three GEMMs
     # (the counters also saw the warm-up calls: scale to the timed ones)
     calls = max(warmup, 1) + steps
-    per_call = sum(v[0] for v in prof.values()) / calls + 3 + 5 * -(-S_np.shape[0] // net.bmax)
+    per_call = sum(v[0] for v in prof.values()) / calls + 3 + 4 * -(-S_np.shape[0] // net.bmax)
     launches = int(round(per_call * steps))
     ms_flat32, (vf32, itf32, stf32) = timed(lambda: plan32.solve(Sh, Vh, TOL, 20))
     ms_warm32, (vw32, itw32, stw32, fb32) = timed(lambda: ws32.solve(Sh, Vh, TOL, 20))
