@@ -46,7 +46,11 @@ constexpr double kSparseWeightFp32 = 15.0;
 //   500 (115 wide)    1.46 / 1.19  1.59 / 1.40  1.68 / 1.62  1.97 / 2.10  2.23 / 2.40
 //   1,000 (224)       2.23 / 1.84  3.02 / 2.94  3.40 / 3.38  3.93 / 4.34  4.48 / 5.02
 //   2,000 (308)       4.24 / 3.22  6.49 / 5.48  8.94 / 8.08  9.45 / 9.04  10.9 / 10.6
+// The instance-major kernels work on blocks padded to 64, so narrow ones stay as they
+// are (96 and 512 instances): 300 buses (62 wide) 0.93 / 0.84, 1.07 / 1.01; 150 (42)
+// 0.67 / 0.67, 0.72 / 0.76; 100 (32) 0.50 / 0.57, 0.53 / 0.66.
 constexpr int kFewTiles = 16;
+constexpr int kFewDense = 49;
 
 #define CK(call)                                   \
   do {                                             \
@@ -198,7 +202,7 @@ void enqueue_body(pf_plan* p, DevState S, cudaStream_t st, nrpf::Recorder* rec,
   const HostPlan& h = p->hp;
   const int32_t* prev = nrpf::ctl_prev(S);
   const int32_t* cur = nrpf::ctl_cur(S);
-  const bool small = P.n_sm_lvl > 0;  // one kernel for the whole linear solve
+  const bool small = nrpf::small_solve_instances(P, S.Bp, sizeof(T)) > 0;  // one kernel for the whole linear solve
   const bool dense = !nrpf::dense_cluster_fits(P, S, sizeof(T));
   if (!small && dense && p->few_inv && S.Bp <= kFewTiles * kTile) {
     P.dim = 1;
@@ -206,7 +210,7 @@ void enqueue_body(pf_plan* p, DevState S, cudaStream_t st, nrpf::Recorder* rec,
     S.inv = p->few_inv;
     S.im_maps = &p->im_maps;
   }
-  nrpf::launch_prepare_lu<T>(P, S, prev, st, rec, small);
+  nrpf::launch_prepare_lu<T>(P, S, prev, st, rec, small ? nrpf::LuPrep::kColumns : nrpf::LuPrep::kSparse);
   nrpf::launch_mismatch<T>(P, S, 1, prev, st, rec);
   nrpf::launch_check(S, st, rec);
   if (small) {
@@ -486,7 +490,7 @@ int pf_plan_create(int n, const int32_t* rowptr, const int32_t* colidx, const do
   // kernels to pay (a 128 x 128 tile of C per CTA)
   p->dp.dim = o.dense_layout == NRPF_DENSE_INSTANCE_MAJOR ||
               (o.dense_layout == NRPF_DENSE_AUTO && im_ok && p->hp.nd >= NRPF_DENSE_IM_MIN);
-  p->few_im = o.dense_layout == NRPF_DENSE_AUTO && im_ok && !p->dp.dim && p->hp.nd > 0;
+  p->few_im = o.dense_layout == NRPF_DENSE_AUTO && im_ok && !p->dp.dim && p->hp.nd >= kFewDense;
   if (p->host_only) {
     *out = p;
     return NRPF_OK;
@@ -496,6 +500,11 @@ int pf_plan_create(int n, const int32_t* rowptr, const int32_t* colidx, const do
   DevPlan& d = p->dp;
   d.n = h.n; d.m = h.m; d.s = h.s; d.nd = h.nd; d.ndp = h.ndp; d.kb = h.kb; d.mp = h.s + h.ndp;
   d.nde = p->lu_precision == NRPF_LU_FP32 && !d.dim && h.kb > 16 ? std::min(h.ndp, (h.nd + 15) / 16 * 16) : h.ndp;
+  if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
+    cudaGetLastError();
+    pf_plan_destroy(p);
+    return NRPF_ERR_CUDA;
+  }
   d.NS = h.NS; d.NLU = h.NLU; d.nnzY = (int)h.colidx.size();
   d.n_one = (int)h.one_pos.size();
   d.n_lu_lvl = (int)h.lu_lvl_ptr.size() - 1;
@@ -542,7 +551,7 @@ int pf_plan_create(int n, const int32_t* rowptr, const int32_t* colidx, const do
     d.fac_op = reinterpret_cast<const int2*>(ops);
     d.n_fac_lvl = std::max((int)h.fac_lvl_ptr.size() - 1, 0);
     d.n_fac_task = std::max((int)h.fac_task.size() - 1, 0);
-    // the whole-solve schedule, where eight instances' values fit in this precision
+    // the whole-solve schedule, where some batch takes it in this precision
     if (nrpf::small_solve_fits(h, p->lu_precision == NRPF_LU_FP32 ? 4 : 8)) {
       if ((rc = upload(p, h.sm_lvl_ptr, &d.sm_lvl_ptr)) || (rc = upload(p, h.sm_task, &d.sm_task)) ||
           (rc = upload(p, h.sm_op, &ops))) {

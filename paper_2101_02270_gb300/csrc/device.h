@@ -36,6 +36,7 @@ struct DevPlan {
   // rounded up to the 16 of the FP32 kernels' steps where ndp is rounded further
   // (their outer panels), ndp otherwise
   int nde;
+  int sms;  // of the plan's device
   int dim;  // 1: instance-major dense block (FP32 LU; see dense_im.h), 0: interleaved
   int64_t NS, NLU;
   int nnzY;

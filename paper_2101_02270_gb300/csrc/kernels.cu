@@ -1570,18 +1570,20 @@ void launch_iter_tail(const DevState& S, cudaGraphConditionalHandle cond, int gr
 
 template <typename T>
 void launch_prepare_lu(const DevPlan& P, const DevState& S, const int32_t* gate, cudaStream_t st,
-                       Recorder* rec, bool whole) {
+                       Recorder* rec, LuPrep prep) {
   // per tile, NLU * 32 values; the sparse segments are the first NS * 32
-  // (both multiples of 128 bytes).  The dense block is left alone unless
-  // `whole`: the Schur tasks then write every position of it.
+  // (both multiples of 128 bytes), the dense block's nd columns follow.
   const size_t stride16 = (size_t)P.NLU * kTile * sizeof(T) / 16;
-  const size_t n16 = (whole || P.nd == 0) ? stride16 : (size_t)P.NS * kTile * sizeof(T) / 16;
+  const size_t values = prep == LuPrep::kWhole ? (size_t)P.NLU
+                        : prep == LuPrep::kSparse  ? (size_t)P.NS
+                        : P.dim ? (size_t)P.NLU : (size_t)(P.NS + (int64_t)P.nd * P.ndp);
+  const size_t n16 = P.nd == 0 ? stride16 : values * kTile * sizeof(T) / 16;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   NRPF_LAUNCH(rec, K_ZERO, st,
               k_zero16<<<sms * 8, 256, 0, st>>>(reinterpret_cast<uint4*>(S.lu), n16, stride16, S.Bp / kTile, gate));
-  if (P.n_one > 0) {
+  if (P.n_one > 0 && prep != LuPrep::kColumns) {
     if (sizeof(T) == 4 && P.dim)
       launch_dense_im_set_ones(P, S, gate, st, rec);
     else if (P.nde > P.nd)
@@ -1804,7 +1806,7 @@ void launch_lu_out(const DevPlan& P, const DevState& S, int B, const int64_t* ma
   template void launch_mismatch<T>(const DevPlan&, const DevState&, int, const int32_t*, cudaStream_t,       \
                                    Recorder*);                                                               \
   template void launch_prepare_lu<T>(const DevPlan&, const DevState&, const int32_t*, cudaStream_t,          \
-                                     Recorder*, bool);                                                       \
+                                     Recorder*, LuPrep);                                                     \
   template void launch_factor<T>(const DevPlan&, const DevState&, const std::vector<int32_t>&,               \
                                  const int32_t*, cudaStream_t, Recorder*, bool);                             \
   template void launch_solve<T>(const DevPlan&, const DevState&, const std::vector<int32_t>&,                \

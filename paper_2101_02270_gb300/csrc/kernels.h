@@ -66,12 +66,15 @@ void launch_iter_tail(const DevState& S, cudaGraphConditionalHandle cond, int gr
 template <typename T>
 void launch_mismatch(const DevPlan& P, const DevState& S, int jac, const int32_t* gate, cudaStream_t st,
                      Recorder* rec = nullptr);
+// What of the LU workspace is zeroed before a refactorisation: everything, the
+// sparse segments (the Schur tasks then write every position of the dense
+// block), or what the small plans' kernel reads (the sparse segments and the
+// dense block's columns without its padding).  Except for the last the identity
+// padding of the dense block is set too.
+enum class LuPrep { kWhole, kSparse, kColumns };
 template <typename T>
-// Zero the LU workspace (whole = false: only the sparse segments; the
-// refactorisation then writes every position of the dense block) and set the
-// identity padding of the dense block.
 void launch_prepare_lu(const DevPlan& P, const DevState& S, const int32_t* gate, cudaStream_t st,
-                       Recorder* rec = nullptr, bool whole = true);
+                       Recorder* rec = nullptr, LuPrep prep = LuPrep::kWhole);
 // Bytes of S.limb, the fixed-point operands of the FP64 trailing update, for a
 // workspace of Bp instances.
 size_t dense_limb_bytes(const DevPlan& P, int Bp);

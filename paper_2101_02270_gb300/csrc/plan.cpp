@@ -391,8 +391,8 @@ int build_plan(int n, const int32_t* rowptr, const int32_t* colidx, const double
   P.lu_fma = fma;
 
   // ---- the whole linear solve by entries ----
-  // for plans whose values, of eight instances in the smaller precision, fit the
-  // shared memory of a CTA
+  // for plans whose values, of eight instances in FP64, fit the shared memory of
+  // a CTA
   const int64_t nval = P.NS + (int64_t)P.nd * P.nd + 2 * (int64_t)m;
   if (m > 0 && nval <= kSmallValues) {
     // value index of (r, c), and the structure of each column below the diagonal

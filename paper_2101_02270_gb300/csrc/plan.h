@@ -17,8 +17,8 @@ struct Upd {
 };
 
 // Values per instance up to which a plan gets the whole-solve schedule: eight
-// instances in FP32 then take 200 KB of shared memory.
-constexpr int64_t kSmallValues = 6400;
+// instances in FP64 then take 200 KB of shared memory.
+constexpr int64_t kSmallValues = 3200;
 
 struct HostPlan {
   // ---- problem ----

@@ -12,8 +12,25 @@
 // levels; an FP64 multiply-add of a warp holds its quarter of the SM for 64
 // cycles, a division for 350).
 //
-// Layout: value v of instance i of the CTA at v * S + i, S = 32, 16 or 8 instances
-// per CTA: the most that fit, fewer while there are SMs without a CTA.  A warp is
+// When: batches whose CTAs, one per SM, are one wave, and plans and precisions for
+// which this then is the faster form.  A second wave takes as long as the first, where
+// the level kernels' time grows by a quarter.  Solves by the level kernels / by this
+// kernel, us (buses, values, dense columns: instances):
+//   FP64  30, 675, 12:     64: 695 / 391   1,216: 810 / 401     2,432: 851 / 458
+//   FP64  100, 2,424, 23:  64: 811 / 760   1,216: 1,054 / 856   2,432: 1,188 / 1,567   10,000: 2,843 / 6,742
+//   FP32  40, 1,062, 20:   64: 603 / 502   2,432: 708 / 579     10,000: 1,262 / 1,889
+//   FP32  55, 1,576, 25:   64: 483 / 632   1,216: 544 / 670     10,000: 1,215 / 2,451
+// In FP32 the level kernels are the faster ones beyond 1,200 values, and where the
+// dense tail, a chain of levels per column here, has more than 20 columns (30 buses,
+// 929 values, 22: 64 instances 409 / 486).
+// The smallest plans (30 buses: 675 values in FP64, 771 in FP32) keep to this kernel in
+// every batch, so that their results do not depend on it, bit for bit: of the sizes up
+// to 10,000 all are at least as fast as with a launch per level (10,000: 1,442 us FP64,
+// 2,435 FP32), where the level kernels take 1,225 / 1,432 and 932 / 1,472.
+//
+// Layout: value v of instance i of the CTA at v * S + i, S = 8, 16 or 32 instances
+// per CTA: the fewest with which the batch's CTAs are one wave (2,432 instances, 30
+// buses: 16 of them 458 us in one wave).  A warp is
 // 32 / S workers of S lanes (lane = instance); a worker takes a task, one entry:
 // its operations come with coalesced loads of S at a time, ahead of the barrier,
 // and are handed out by shuffles; the entry stays in a register and takes its
@@ -27,6 +44,10 @@ namespace nrpf {
 namespace {
 
 constexpr size_t kSmallSmem = 200 * 1024;
+constexpr size_t kSmallValuesFp32 = 1200;
+constexpr int kSmallDenseFp32 = 20;
+// values up to which a plan keeps to the kernel beyond one wave
+constexpr size_t kSmallAlways64 = 700, kSmallAlways32 = 800;
 constexpr int kSmallThreads = 512;
 
 template <typename T, int S, bool OPS>
@@ -151,21 +172,31 @@ void launch_for(const DevPlan& P, const DevState& st, int nval, const int32_t* g
   else launch<T, S, false>(P, st, nval, values, gate, s, rec);
 }
 
+static_assert(kSmallAlways64 * 32 * 8 <= kSmallSmem && kSmallAlways32 * 32 * 4 <= kSmallSmem, "32 instances fit");
+
 }  // namespace
 
 bool small_solve_fits(const HostPlan& h, size_t width) {
-  const int64_t nval = h.NS + (int64_t)h.nd * h.nd + 2 * (int64_t)h.m;
-  return h.sm_lvl_ptr.size() > 1 && (size_t)nval * 8 * width <= kSmallSmem;
+  const size_t nval = (size_t)(h.NS + (int64_t)h.nd * h.nd + 2 * (int64_t)h.m);
+  return h.sm_lvl_ptr.size() > 1 && nval * 8 * width <= kSmallSmem &&
+         (width == 8 || (nval <= kSmallValuesFp32 && h.nd <= kSmallDenseFp32));
+}
+
+int small_solve_instances(const DevPlan& P, int Bp, size_t width) {
+  if (P.n_sm_lvl == 0) return 0;
+  const size_t nval = (size_t)(P.NS + (int64_t)P.nd * P.nd) + 2 * (size_t)P.m;
+  for (int s = 8; s <= 32 && nval * s * width <= kSmallSmem; s *= 2)
+    if (Bp / s <= P.sms) return s;
+  return nval <= (width == 8 ? kSmallAlways64 : kSmallAlways32) ? 32 : 0;
 }
 
 template <typename T>
 void launch_small_solve(const DevPlan& P, const DevState& S, const int32_t* gate, cudaStream_t st, Recorder* rec) {
   const int nval = (int)(P.NS + (int64_t)P.nd * P.nd) + 2 * P.m;
-  int s = 32;
-  while (s > 8 && ((size_t)nval * s * sizeof(T) > kSmallSmem || S.Bp / s < 152)) s /= 2;
+  const int s = small_solve_instances(P, S.Bp, sizeof(T));
   if (s == 32) launch_for<T, 32>(P, S, nval, gate, st, rec);
   else if (s == 16) launch_for<T, 16>(P, S, nval, gate, st, rec);
-  else launch_for<T, 8>(P, S, nval, gate, st, rec);
+  else if (s == 8) launch_for<T, 8>(P, S, nval, gate, st, rec);
 }
 
 template void launch_small_solve<float>(const DevPlan&, const DevState&, const int32_t*, cudaStream_t, Recorder*);

@@ -11,9 +11,12 @@
 
 namespace nrpf {
 
-// Whether the plan has the whole-solve schedule and eight instances' values of
-// `width` bytes fit a CTA's shared memory.
+// Whether the plan has the whole-solve schedule and some batch of it, in a
+// precision of `width` bytes, would take this kernel.
 bool small_solve_fits(const HostPlan& h, size_t width);
+
+// Instances per CTA for a batch padded to Bp, or 0: the level kernels serve it.
+int small_solve_instances(const DevPlan& P, int Bp, size_t width);
 
 // S.x <- J^-1 S.x for every active tile, from the Jacobian values in S.lu (the
 // whole LU array zeroed before they were filled in); S.lu is left as it is.

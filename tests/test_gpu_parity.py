@@ -583,3 +583,30 @@ def test_more_batch_sizes_than_loop_graphs():
             assert torch.equal(w, v[k[:32 * t]]) and torch.equal(it2, it[k[:32 * t]])
         counts = p.profile_read()
     assert counts["update"][0] == 70 * (int(it.max()) + 1)
+
+
+@pytest.mark.parametrize("n,branches,lu,waves", [(55, 75, "fp64", 16), (85, 116, "fp64", 8), (40, 50, "fp32", 32),
+                                                 (55, 69, "fp32", 0), (120, 164, "fp32", 0), (30, 41, "fp64", None),
+                                                 (30, 41, "fp32", None)])
+def test_small_plans_leave_their_kernel_beyond_one_wave(n, branches, lu, waves):
+    """A batch of more CTAs of the small plans' kernel, of at most `waves` instances
+    (as many as fit), than the GPU has SMs goes to the level kernels, larger FP32
+    plans always, the smallest plans never.  Voltages on either side of the line are
+    those of the same scenarios within a few units of rounding."""
+    import gridgen
+    g = gridgen.make_grid("mesh30_b64" if n < 100 else "mesh2000_b10k", 0, n=n, n_branch=branches, n_pv=n // 10,
+                          load_scale=1 / 16)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    last = 32 * (sms * (waves or 0) // 32) or 64
+    sc = gridgen.make_scenarios(g, last + 1 if waves else 33 * sms, 0.6, 1.4)
+    S, V0 = _dev(sc.sbus(g)), _dev(sc.v0_flat(g))
+    with _plan(g, lu_precision=lu) as p:
+        out = []
+        for B in (last, len(S)):
+            p.profile_start([])
+            out.append(p.solve(S[:B], V0[:B], TOL, 10))
+            levels = p.profile_read()["bwd_level"][0] > 0
+            assert levels == (waves is not None and B > sms * waves)
+    a, b = out
+    assert torch.all(a[2] == 0) and torch.all(b[2] == 0) and torch.equal(a[1], b[1][:last])
+    assert (a[0] - b[0][:last]).abs().max().item() < (1e-12 if lu == "fp64" else 1e-9)
