@@ -6,58 +6,64 @@
 
 namespace {
 
-// A thread owns one branch and walks over the instances of its block: the
-// branch's admittance (two FP64 divisions, each about ten FMAs of an FP64 pipe
-// that runs at two per SM and clock) is formed once and kept in registers, and
-// no index is divided.  Branches are fastest across the threads, so the flow
-// writes are coalesced; the two voltage reads are gathers from the instance's
-// row, which stays in L1/L2 while the block's branches read it.
+// A thread owns one branch and walks over a group of instances: the branch's
+// admittance (two FP64 divisions, each about ten FMAs of an FP64 pipe that runs
+// at two per SM and clock) is formed once and kept in registers.  The threads are
+// numbered through the branches of the first group, then of the next, so that no
+// lane is idle whatever the number of branches (an FP64 instruction takes the same
+// time with one lane as with 32), at the price of one integer division per thread.
+// Branches are fastest, so the flow writes are coalesced; the two voltage reads are
+// gathers from the instance's row, which stays in L1/L2 while its branches read it.
 // pi model: ys = 1/(r + jx), half the charging b at each end;
 // I_f = ys (V_f - V_t) + j b/2 V_f, S_f = V_f conj(I_f), and symmetrically at t.
 // Bound: 18 FP64 operations per branch and instance (0.74 ms for 2,600 branches
 // x 10,000 instances at the FP64 peak; the bytes alone take 0.17 ms): measured
-// 0.90 ms there.  With one thread per (branch, instance), which divided for
-// each, it took 1.73 ms.
+// 0.88 ms there.  With one thread per (branch, instance), which divided for
+// each, it took 1.73 ms; 1,000 buses x 10,000 0.91, now 0.48.  A block of 256
+// threads along the branches, of which only 41 exist on a 30-bus grid, took 22.6 us
+// on 5,000 instances of it and 36.3 on 10,000; a thread per branch and instance 19.9
+// and 33.5, this form 19.8 and 33.5.
 constexpr int kThreads = 256;
 
 __global__ void __launch_bounds__(kThreads) k_branch_flows(
     int n, int nbr, const int32_t* __restrict__ f, const int32_t* __restrict__ t, const double* __restrict__ r,
-    const double* __restrict__ x, const double* __restrict__ b, int B, int per, const uint8_t* __restrict__ in_service,
-    const double2* __restrict__ v, double2* __restrict__ sf, double2* __restrict__ st) {
-  const int e = blockIdx.x * kThreads + threadIdx.x;
-  if (e >= nbr) return;
+    const double* __restrict__ x, const double* __restrict__ b, int B, int per, unsigned long long total,
+    const uint8_t* __restrict__ in_service, const double2* __restrict__ v, double2* __restrict__ sf,
+    double2* __restrict__ st) {
+  const unsigned long long idx = (unsigned long long)blockIdx.x * kThreads + threadIdx.x;
+  if (idx >= total) return;  // total: branches x groups
+  const long long g = total >> 32 ? (long long)(idx / (unsigned)nbr) : (long long)((unsigned)idx / (unsigned)nbr);
+  const int e = (int)(idx - (unsigned long long)g * (unsigned)nbr);
   const int ef = f[e], et = t[e];
   const double den = r[e] * r[e] + x[e] * x[e];
   const double gs = r[e] / den, bs = -x[e] / den, bh = 0.5 * b[e];
-  for (long long i0 = (long long)blockIdx.y * per; i0 < B; i0 += (long long)gridDim.y * per) {
-    const int i1 = (int)(i0 + per < B ? i0 + per : B);
+  const int i0 = (int)(g * per), i1 = B - i0 < per ? B : i0 + per;
 #pragma unroll 4
-    for (int i = (int)i0; i < i1; ++i) {
-      const size_t q = (size_t)i * nbr + e;
-      if (in_service && !in_service[q]) {
-        sf[q] = make_double2(0.0, 0.0);
-        st[q] = make_double2(0.0, 0.0);
-        continue;
-      }
-      const double2 vf = v[(size_t)i * n + ef], vt = v[(size_t)i * n + et];
-      const double dr = vf.x - vt.x, di = vf.y - vt.y;
-      // I_f = ys (V_f - V_t) + j bh V_f
-      const double ifr = gs * dr - bs * di - bh * vf.y;
-      const double ifi = gs * di + bs * dr + bh * vf.x;
-      // I_t = -ys (V_f - V_t) + j bh V_t
-      const double itr = -(gs * dr - bs * di) - bh * vt.y;
-      const double iti = -(gs * di + bs * dr) + bh * vt.x;
-      // S = V conj(I)
-      sf[q] = make_double2(vf.x * ifr + vf.y * ifi, vf.y * ifr - vf.x * ifi);
-      st[q] = make_double2(vt.x * itr + vt.y * iti, vt.y * itr - vt.x * iti);
+  for (int i = i0; i < i1; ++i) {
+    const size_t q = (size_t)i * nbr + e;
+    if (in_service && !in_service[q]) {
+      sf[q] = make_double2(0.0, 0.0);
+      st[q] = make_double2(0.0, 0.0);
+      continue;
     }
+    const double2 vf = v[(size_t)i * n + ef], vt = v[(size_t)i * n + et];
+    const double dr = vf.x - vt.x, di = vf.y - vt.y;
+    // I_f = ys (V_f - V_t) + j bh V_f
+    const double ifr = gs * dr - bs * di - bh * vf.y;
+    const double ifi = gs * di + bs * dr + bh * vf.x;
+    // I_t = -ys (V_f - V_t) + j bh V_t
+    const double itr = -(gs * dr - bs * di) - bh * vt.y;
+    const double iti = -(gs * di + bs * dr) + bh * vt.x;
+    // S = V conj(I)
+    sf[q] = make_double2(vf.x * ifr + vf.y * ifi, vf.y * ifr - vf.x * ifi);
+    st[q] = make_double2(vt.x * itr + vt.y * iti, vt.y * itr - vt.x * iti);
   }
 }
 
-// Instances per block: up to 16, which makes the divisions a tenth of the
+// Instances per group: up to 16, which makes the divisions a tenth of the
 // arithmetic; fewer while the blocks would not fill the GPU eight times over
 // (8 x 152 CTAs of 256 threads are all that is resident).
-constexpr int kPerBlock = 16;
+constexpr int kPerGroup = 16;
 constexpr long long kFillBlocks = 8 * 152;
 
 }  // namespace
@@ -69,15 +75,13 @@ extern "C" int pf_branch_flows(int n, int nbr, const int32_t* f, const int32_t* 
   if ((long long)B * nbr == 0) return NRPF_OK;
   if (!f || !t || !r || !x || !b || !v || !sf || !st) return NRPF_ERR_ARG;
   if (((long long)B * nbr + kThreads - 1) / kThreads > 0x7fffffffLL) return NRPF_ERR_ARG;
-  const unsigned gx = (unsigned)(((long long)nbr + kThreads - 1) / kThreads);
-  const long long fit = (long long)B * gx / kFillBlocks;
-  const int per = (int)(fit < 1 ? 1 : fit > kPerBlock ? kPerBlock : fit);
-  const long long rows = ((long long)B + per - 1) / per;
-  const unsigned gy = (unsigned)(rows < 65535 ? rows : 65535);
+  const long long fit = (long long)B * nbr / (kThreads * kFillBlocks);
+  const int per = (int)(fit < 1 ? 1 : fit > kPerGroup ? kPerGroup : fit);
+  const unsigned long long total = (unsigned long long)(((long long)B + per - 1) / per) * (unsigned)nbr;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  k_branch_flows<<<dim3(gx, gy), kThreads, 0, s>>>(n, nbr, f, t, r, x, b, B, per, in_service,
-                                                   reinterpret_cast<const double2*>(v),
-                                                   reinterpret_cast<double2*>(sf), reinterpret_cast<double2*>(st));
+  k_branch_flows<<<(unsigned)((total + kThreads - 1) / kThreads), kThreads, 0, s>>>(
+      n, nbr, f, t, r, x, b, B, per, total, in_service, reinterpret_cast<const double2*>(v),
+      reinterpret_cast<double2*>(sf), reinterpret_cast<double2*>(st));
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? NRPF_OK : NRPF_ERR_CUDA;
 }

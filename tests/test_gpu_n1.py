@@ -171,3 +171,25 @@ def test_branch_flows_every_instance_block(B):
     # |V| <= 1.1, |ys| <= 20: a dozen roundings of values below 50
     assert np.max(np.abs(sa - of)) < 1e-12 and np.max(np.abs(sb - ot)) < 1e-12
     assert np.array_equal(sf, np.where(ins, sa, 0)) and np.array_equal(st, np.where(ins, sb, 0))
+
+
+@pytest.mark.parametrize("n,branches", [(5, 6), (24, 32), (24, 33), (48, 65), (90, 129), (180, 257)])
+@pytest.mark.parametrize("B", [1, 7, 1300, 19999])
+def test_branch_flows_any_number_of_branches(n, branches, B):
+    """Fewer branches than a warp to more than a block, groups of one to four
+    instances that begin anywhere in a warp, the last of them incomplete: every flow
+    against the pi model in NumPy."""
+    rng = np.random.default_rng(branches + B)
+    f, t = rng.integers(0, n, branches), rng.integers(0, n - 1, branches)
+    t = np.where(t >= f, t + 1, t)
+    r, x, b = rng.uniform(0.01, 0.05, branches), rng.uniform(0.05, 0.2, branches), rng.uniform(0, 0.05, branches)
+    types = np.ones(n, dtype=np.int8)
+    types[0] = 3
+    V = rng.uniform(0.9, 1.1, (B, n)) * np.exp(1j * rng.uniform(-0.5, 0.5, (B, n)))
+    with _pf().Plan.from_branches(n, f, t, r, x, b, types) as p:
+        sa, sb = (a.cpu().numpy() for a in p.branch_flows(_dev(V)))
+    ys, bh = 1.0 / (r + 1j * x), 0.5j * b
+    vf, vt = V[:, f], V[:, t]
+    of, ot = vf * np.conj(ys * (vf - vt) + bh * vf), vt * np.conj(-ys * (vf - vt) + bh * vt)
+    # |V| <= 1.1, |ys| <= 20: a dozen roundings of values below 50
+    assert np.max(np.abs(sa - of)) < 1e-12 and np.max(np.abs(sb - ot)) < 1e-12
