@@ -191,45 +191,61 @@ int ensure_capacity(pf_plan* p, int B) {
   return NRPF_OK;
 }
 
+// The kernels that a batch takes for its linear solves, where the rule depends on
+// the number of instances and the results' last bits on the choice.
+struct Route {
+  bool small;    // one kernel for the whole linear solve
+  bool cluster;  // the dense block by a cluster of CTAs per instance
+  bool few;      // an interleaved FP32 block factorised instance-major
+};
+
+Route route_of(const pf_plan* p, int B, size_t width) {
+  const int Bp = (B + kTile - 1) / kTile * kTile;
+  Route r{};
+  r.small = nrpf::small_solve_instances(p->dp, Bp, width) > 0;
+  r.cluster = !r.small && nrpf::dense_cluster_pays(p->dp, B, width);
+  r.few = !r.small && !r.cluster && p->few_inv && Bp <= kFewTiles * kTile;
+  return r;
+}
+
 // One Newton iteration (Alg. 1 loop body): LU preparation and mismatch +
 // Jacobian (gated by the previous check), the convergence test, then
 // refactorisation, FS/BS and update (gated by this check), and the tail that
 // advances the loop control.
 template <typename T>
-void enqueue_body(pf_plan* p, DevState S, cudaStream_t st, nrpf::Recorder* rec,
+void enqueue_body(pf_plan* p, DevState S, Route route, cudaStream_t st, nrpf::Recorder* rec,
                   cudaGraphConditionalHandle cond, int graph) {
   DevPlan P = p->dp;
   const HostPlan& h = p->hp;
   const int32_t* prev = nrpf::ctl_prev(S);
   const int32_t* cur = nrpf::ctl_cur(S);
-  const bool small = nrpf::small_solve_instances(P, S.Bp, sizeof(T)) > 0;  // one kernel for the whole linear solve
-  const bool dense = !nrpf::dense_cluster_fits(P, S, sizeof(T));
-  if (!small && dense && p->few_inv && S.Bp <= kFewTiles * kTile) {
+  if (route.few) {
     P.dim = 1;
     P.nde = P.ndp;
     S.inv = p->few_inv;
     S.im_maps = &p->im_maps;
   }
-  nrpf::launch_prepare_lu<T>(P, S, prev, st, rec, small ? nrpf::LuPrep::kColumns : nrpf::LuPrep::kSparse);
+  nrpf::launch_prepare_lu<T>(P, S, prev, st, rec, route.small ? nrpf::LuPrep::kColumns : nrpf::LuPrep::kSparse);
   nrpf::launch_mismatch<T>(P, S, 1, prev, st, rec);
   nrpf::launch_check(S, st, rec);
-  if (small) {
+  if (route.small) {
     nrpf::launch_small_solve<T>(P, S, cur, st, rec);
   } else {
-    nrpf::launch_factor<T>(P, S, h.lu_lvl_ptr, cur, st, rec, dense);
-    nrpf::launch_solve<T>(P, S, h.fw_lvl_ptr, h.bw_lvl_ptr, cur, st, rec, dense);
+    nrpf::launch_factor<T>(P, S, h.lu_lvl_ptr, cur, st, rec, !route.cluster);
+    nrpf::launch_solve<T>(P, S, h.fw_lvl_ptr, h.bw_lvl_ptr, cur, st, rec, !route.cluster);
   }
   nrpf::launch_update<T>(P, S, cur, st, rec);
   nrpf::launch_iter_tail(S, cond, graph, st, rec);
 }
 
 // The loop graph: a WHILE node whose body is one iteration, captured once per
-// workspace and padded batch size; the iteration's tail kernel sets the
+// workspace, padded batch size and route; the iteration's tail kernel sets the
 // condition, so the loop ends on the device as soon as no instance is active
 // (or at maxit).
 template <typename T>
-int ensure_loop_graph(pf_plan* p, const DevState& S, cudaGraphExec_t* out) {
-  const int key = 2 * S.Bp + (S.yv ? 1 : 0);
+int ensure_loop_graph(pf_plan* p, const DevState& S, Route route, cudaGraphExec_t* out) {
+  const int64_t key = (int64_t)S.Bp << 4 | (S.yv ? 8 : 0) | (route.small ? 4 : 0) | (route.cluster ? 2 : 0) |
+                      (route.few ? 1 : 0);
   auto it = p->loops.find(key);
   if (it != p->loops.end()) {
     *out = it->second.exec;
@@ -263,7 +279,7 @@ int ensure_loop_graph(pf_plan* p, const DevState& S, cudaGraphExec_t* out) {
   e = cudaStreamBeginCaptureToGraph(p->capture_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
   if (e != cudaSuccess) return fail(e);
   nrpf::Recorder count;  // launches of one body, by class
-  enqueue_body<T>(p, S, p->capture_stream, &count, cond, slot + 1);
+  enqueue_body<T>(p, S, route, p->capture_stream, &count, cond, slot + 1);
   cudaGraph_t captured = nullptr;
   const cudaError_t el = cudaGetLastError();
   e = cudaStreamEndCapture(p->capture_stream, &captured);
@@ -306,6 +322,7 @@ int enqueue_solve(pf_plan* p, int B, const double* ybus, const double* sbus, con
   // the first Bp of the workspace's capacity serve)
   DevState S = p->st;
   S.Bp = (B + kTile - 1) / kTile * kTile;
+  const Route route = route_of(p, B, sizeof(T));
   nrpf::Recorder* rec = &p->rec;
   if (ybus || outages) {
     int rc = ensure_yv(p);
@@ -324,18 +341,18 @@ int enqueue_solve(pf_plan* p, int B, const double* ybus, const double* sbus, con
     if (cs != cudaStreamCaptureStatusNone) {
       // the caller captures this stream: maxit iterations, instances that
       // have finished skip through the gates
-      for (int it = 0; it < maxit; ++it) enqueue_body<T>(p, S, st, rec, 0, 0);
+      for (int it = 0; it < maxit; ++it) enqueue_body<T>(p, S, route, st, rec, 0, 0);
     } else if (rec->time_mask) {
       // profiled solve (per-launch events): the host ends the loop
       for (int it = 0; it < maxit; ++it) {
-        enqueue_body<T>(p, S, st, rec, 0, 0);
+        enqueue_body<T>(p, S, route, st, rec, 0, 0);
         CK(cudaMemcpyAsync(p->h_prev, nrpf::ctl_prev(S), sizeof(int32_t), cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
         if (*p->h_prev == 0) break;
       }
     } else {
       cudaGraphExec_t exec = nullptr;
-      int rc = ensure_loop_graph<T>(p, S, &exec);
+      int rc = ensure_loop_graph<T>(p, S, route, &exec);
       if (rc) return rc;
       CK(cudaGraphLaunch(exec, st));
     }
@@ -564,6 +581,7 @@ int pf_plan_create(int n, const int32_t* rowptr, const int32_t* colidx, const do
       d.n_sm_op = (int)(h.sm_op.size() / 2);
     }
     d.n_schur = (int)(h.schur_task.size() / 4);
+    d.clusters = nrpf::dense_cluster_resident(d, p->lu_precision == NRPF_LU_FP32 ? 4 : 8);
   }
   if (o.max_batch > 0 && (rc = ensure_capacity(p, o.max_batch))) {
     pf_plan_destroy(p);

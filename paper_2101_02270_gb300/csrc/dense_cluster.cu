@@ -28,10 +28,19 @@ constexpr int kClu = 8;         // CTAs per cluster (the portable maximum)
 constexpr int kCluThreads = 512;
 constexpr int kCluNb = 8;       // columns per block
 constexpr size_t kCluSmem = 220 * 1024;
-// up to two tiles: 512 CTAs, three to four rounds of the chip.  A solve of 64 flows on
-// the 2,000-bus grid takes 11.6 ms in FP64 (12.8 by the tile-wide kernels) and 3.6
-// in FP32 (4.5), of 128 flows 18.8 (15.2) and 5.7 (5.7).
-constexpr int kCluTiles = 2;
+// When: a block of an instance takes its time in every round of resident clusters, the
+// tile-wide kernels theirs per tile, and clusters that share an SM slow each other.  So
+// FP64 up to 64 instances and two rounds (a cluster's FP64 work alone is far less than
+// a tile's), FP32 up to one round and 32 instances, or 64 of blocks up to 192 wide.
+// Solves, tile-wide kernels / clusters, ms (width of the block: instances):
+//   FP64  400:  1: 20.0 / 12.6   16: 20.0 / 17.7   32: 20.0 / 23.1   64: 23.1 / 35.6
+//         280:  1: 11.3 / 6.76   32: 11.3 / 7.64   64: 12.3 / 11.3
+//   FP32  576:  8: 4.99 / 4.58   16: 5.11 / 6.66   32: 5.27 / 8.75   64: 6.78 / 13.9
+//         448:  8: 3.68 / 3.10   16: 3.72 / 4.41   32: 3.79 / 5.74   64: 4.24 / 8.63
+//         320:  1: 2.80 / 2.32   32: 2.85 / 2.44   48: 2.98 / 3.24   64: 3.00 / 3.39
+//         176:  1: 2.03 / 1.63   32: 2.03 / 1.66   64: 2.06 / 2.04
+constexpr int kCluInstances = 64, kCluRounds64 = 2;
+constexpr int kCluInstances32Wide = 32, kCluWide32 = 192;
 
 // dynamic shared memory of a CTA: its columns, the current panel, the right-hand
 // side, the inverse pivots of its columns
@@ -209,8 +218,45 @@ __global__ void __launch_bounds__(kCluThreads) k_dense_cluster(DevPlan P, DevSta
 
 }  // namespace
 
-bool dense_cluster_fits(const DevPlan& P, const DevState& S, size_t width) {
-  return P.nde >= 2 * kCluNb && P.nde % kCluNb == 0 && S.Bp <= kCluTiles * kTile && clu_smem(P.nde, width) <= kCluSmem;
+namespace {
+
+void configure(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, unsigned instances, size_t smem, cudaStream_t st) {
+  cfg.gridDim = dim3(instances * kClu);
+  cfg.blockDim = dim3(kCluThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kClu;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+}
+
+template <typename T>
+int resident(const DevPlan& P) {
+  cudaFuncSetAttribute(k_dense_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCluSmem);
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  configure(cfg, at, 1, clu_smem(P.nde, sizeof(T)), nullptr);
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, k_dense_cluster<T>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+}  // namespace
+
+int dense_cluster_resident(const DevPlan& P, size_t width) {
+  if (P.nde < 2 * kCluNb || P.nde % kCluNb != 0 || clu_smem(P.nde, width) > kCluSmem) return 0;
+  return width == 8 ? resident<double>(P) : resident<float>(P);
+}
+
+bool dense_cluster_pays(const DevPlan& P, int B, size_t width) {
+  if (width == 8) return B <= kCluInstances && B <= kCluRounds64 * P.clusters;
+  if (P.nde <= kCluWide32) return P.clusters > 0 && B <= kCluInstances;
+  return B <= kCluInstances32Wide && B <= P.clusters;
 }
 
 template <typename T>
@@ -223,16 +269,8 @@ void launch_dense_cluster(const DevPlan& P, const DevState& S, const int32_t* ga
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(S.Bp * kClu));
-  cfg.blockDim = dim3(kCluThreads);
-  cfg.dynamicSmemBytes = clu_smem(P.nde, sizeof(T));
-  cfg.stream = st;
   cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = kClu;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  configure(cfg, at, (unsigned)S.Bp, clu_smem(P.nde, sizeof(T)), st);
   NRPF_LAUNCH(rec, K_DENSE_SOLVE, st, cudaLaunchKernelEx(&cfg, k_dense_cluster<T>, P, S, gate));
 }
 

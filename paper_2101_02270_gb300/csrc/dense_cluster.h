@@ -9,8 +9,12 @@
 
 namespace nrpf {
 
-// Whether the plan's block fits and the batch is small enough for it to pay.
-bool dense_cluster_fits(const DevPlan& P, const DevState& S, size_t width);
+// Clusters that the device can hold at once, 0 where the plan's block does not fit
+// one (width: bytes of a value).
+int dense_cluster_resident(const DevPlan& P, size_t width);
+
+// Whether a batch of B instances of the plan is small enough for the clusters to pay.
+bool dense_cluster_pays(const DevPlan& P, int B, size_t width);
 
 // S.x rows s .. s+nde-1 <- the dense block's share of the solution, between the
 // sparse forward and backward levels.  S.lu is left as the Schur tasks wrote it.

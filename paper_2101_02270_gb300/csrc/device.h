@@ -37,6 +37,7 @@ struct DevPlan {
   // (their outer panels), ndp otherwise
   int nde;
   int sms;  // of the plan's device
+  int clusters;  // of dense_cluster.cu that the device holds at once, 0: the block does not fit one
   int dim;  // 1: instance-major dense block (FP32 LU; see dense_im.h), 0: interleaved
   int64_t NS, NLU;
   int nnzY;
@@ -88,7 +89,7 @@ struct DevPlan {
 // Device-resident control of the Newton loop, so that one iteration can run
 // unchanged from a graph: every kernel of an iteration reads its gate and the
 // iteration number here.
-constexpr int kLoopSlots = 64;  // loop graphs kept per workspace, one per padded batch size and kind of admittances
+constexpr int kLoopSlots = 64;  // loop graphs kept per workspace, one per padded batch size and set of kernels
 struct SolveCtl {
   int32_t prev;     // instances active after the previous check: gate of the
                     // LU preparation and mismatch (nonzero before the first)

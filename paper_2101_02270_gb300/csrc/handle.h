@@ -38,7 +38,7 @@ struct pf_plan {
     int slot = 0;
     int64_t body_launches[nrpf::K_NCLASS] = {};
   };
-  std::map<int, LoopGraph> loops;  // by 2 x padded batch + per-instance Ybus flag
+  std::map<int64_t, LoopGraph> loops;  // by padded batch, per-instance Ybus flag and route
   cudaStream_t capture_stream = nullptr;
   int32_t* h_prev = nullptr;  // pinned: ctl->prev read back by profiled solves
   // host-resident batches: two device staging slots of stage_cap instances,

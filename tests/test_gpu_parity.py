@@ -610,3 +610,25 @@ def test_small_plans_leave_their_kernel_beyond_one_wave(n, branches, lu, waves):
     a, b = out
     assert torch.all(a[2] == 0) and torch.all(b[2] == 0) and torch.equal(a[1], b[1][:last])
     assert (a[0] - b[0][:last]).abs().max().item() < (1e-12 if lu == "fp64" else 1e-9)
+
+
+@pytest.mark.parametrize("n,branches,lu,inside,beyond", [(2000, 2900, "fp32", 8, 32), (2000, 2900, "fp64", 8, 64),
+                                                         (2000, 2600, "fp32", 32, 33), (600, 888, "fp32", 64, 65),
+                                                         (1000, 1300, "fp64", 64, 65)])
+def test_clusters_where_they_are_resident(n, branches, lu, inside, beyond):
+    """The dense block goes to a cluster per instance while the batch's clusters fit
+    the GPU (about; FP64 twice over), however many tiles that is: wide blocks
+    only for a few instances.  Instances have the same voltages on both sides."""
+    import gridgen
+    g = gridgen.make_grid("mesh2000_b10k", 0, n=n, n_branch=branches, n_pv=n // 10, load_scale=1 / 32)
+    sc = gridgen.make_scenarios(g, beyond, 0.6, 1.4)
+    S, V0 = _dev(sc.sbus(g)), _dev(sc.v0_flat(g))
+    out = {}
+    with _plan(g, lu_precision=lu) as p:
+        for B in (inside, beyond):
+            p.profile_start([])
+            out[B] = p.solve(S[:B], V0[:B], TOL, 10)
+            assert (p.profile_read()["dense_update"][0] == 0) == (B == inside)
+    a, b = out[inside], out[beyond]
+    assert torch.all(a[2] == 0) and torch.all(b[2] == 0)
+    assert (a[0] - b[0][:inside]).abs().max().item() < (1e-12 if lu == "fp64" else 1e-9)
