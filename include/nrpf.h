@@ -180,6 +180,9 @@ int pf_plan_get_pattern(const pf_plan* p, int32_t* pos_of_unknown, int64_t* colp
  * maxit iterations instead (finished instances skip through their gates);
  * with per-kernel timing on (pf_profile_start with a nonzero mask) the host
  * ends the loop after each iteration.  All three give identical results.
+ * Which kernels factorise the Jacobian depends on B (few instances, tens,
+ * hundreds and more take different ones): the same scenario in batches of other
+ * sizes agrees to rounding, not bit for bit.
  * Calls on one plan share its workspace: serialise them (one stream).
  * Errors: NRPF_ERR_ARG (B < 0, tol not finite, maxit < 0, null pointers),
  * NRPF_ERR_NOMEM, NRPF_ERR_CUDA.  B == 0 is a no-op. */
@@ -277,7 +280,9 @@ int pf_branch_flows(int n, int nbr, const int32_t* f, const int32_t* t, const do
 
 /* pf_solve_batch for a batch held in host memory (the paper's stream study,
  * Sec. 3.2 / Sec. 5: copies overlapped with computation).  The batch is cut
- * into chunks of `chunk` instances (0 = the whole batch).  Each chunk goes
+ * into chunks of `chunk` instances (0 = the whole batch); all take the kernels
+ * that a device-resident batch of B instances takes, so the results are that
+ * solve's, bit for bit.  Each chunk goes
  * through one of two device staging slots owned by the plan, used in turn
  * across chunks and across calls: its inputs are copied in on a copy-in
  * stream owned by the plan, it is solved on `stream`, and its results are

@@ -313,16 +313,18 @@ int ensure_yv(pf_plan* p) {
 // ybus: per-instance [B, nnzY] complex device values, or null for the plan's;
 // outages (device [B, k], with ybus null): per-instance admittances built on
 // the device from the plan's base values and branch stamps
+// whole: instances of the batch that these B are a part of; its route serves all
+// parts, so that their results are those of the batch in one piece, bit for bit
 template <typename T>
 int enqueue_solve(pf_plan* p, int B, const double* ybus, const double* sbus, const double* v0, double tol,
                   int maxit, double* v_out, int32_t* iters, uint8_t* status, cudaStream_t st,
-                  const int32_t* outages = nullptr, int k = 0) {
+                  const int32_t* outages = nullptr, int k = 0, int whole = 0) {
   const DevPlan& P = p->dp;
   // grids cover this batch's tiles only (tiles are contiguous per array, so
   // the first Bp of the workspace's capacity serve)
   DevState S = p->st;
   S.Bp = (B + kTile - 1) / kTile * kTile;
-  const Route route = route_of(p, B, sizeof(T));
+  const Route route = route_of(p, std::max(B, whole), sizeof(T));
   nrpf::Recorder* rec = &p->rec;
   if (ybus || outages) {
     int rc = ensure_yv(p);
@@ -848,9 +850,9 @@ int pf_solve_batch_host(pf_plan* p, int B, const double* sbus, const double* v0,
     CK(cudaStreamWaitEvent(st, p->ev_in[i], 0));
     const Slot& d = slot[i];
     if (p->lu_precision == NRPF_LU_FP32)
-      rc = enqueue_solve<float>(p, count(c), nullptr, d.s, d.v0, tol, maxit, d.v, d.it, d.st, st);
+      rc = enqueue_solve<float>(p, count(c), nullptr, d.s, d.v0, tol, maxit, d.v, d.it, d.st, st, nullptr, 0, B);
     else
-      rc = enqueue_solve<double>(p, count(c), nullptr, d.s, d.v0, tol, maxit, d.v, d.it, d.st, st);
+      rc = enqueue_solve<double>(p, count(c), nullptr, d.s, d.v0, tol, maxit, d.v, d.it, d.st, st, nullptr, 0, B);
     if (rc) return rc;
     CK(cudaEventRecord(p->ev_done[i], st));
     CK(cudaStreamWaitEvent(os, p->ev_done[i], 0));

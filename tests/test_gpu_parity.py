@@ -632,3 +632,22 @@ def test_clusters_where_they_are_resident(n, branches, lu, inside, beyond):
     a, b = out[inside], out[beyond]
     assert torch.all(a[2] == 0) and torch.all(b[2] == 0)
     assert (a[0] - b[0][:inside]).abs().max().item() < (1e-12 if lu == "fp64" else 1e-9)
+
+
+@pytest.mark.parametrize("lu,B,chunk", [("fp64", 200, 32), ("fp64", 65, 64), ("fp32", 600, 512), ("fp32", 600, 64),
+                                        ("fp32", 300, 40), ("fp64", 64, 32)])
+def test_host_chunks_take_the_kernels_of_the_batch(lu, B, chunk):
+    """On a grid whose batches of up to 64 and up to 512 instances take kernels of
+    their own: a batch from host memory in chunks of such sizes still gives the
+    device-resident solve's results, bit for bit."""
+    import gridgen
+    g = gridgen.make_grid("mesh2000_b10k", 0, n=420, n_branch=590, n_pv=42, load_scale=1 / 16)
+    sc = gridgen.make_scenarios(g, B, 0.6, 1.4)
+    S, V0 = (torch.from_numpy(np.ascontiguousarray(a)).pin_memory() for a in (sc.sbus(g), sc.v0_flat(g)))
+    with _plan(g, lu_precision=lu) as p:
+        h = p.solve_host(S, V0, TOL, 10, chunk=chunk)
+        torch.cuda.synchronize()
+        d = p.solve(S.cuda(), V0.cuda(), TOL, 10)
+    assert torch.all(d[2] == 0)
+    for x, y in zip(h, d):
+        assert torch.equal(x, y.cpu())
