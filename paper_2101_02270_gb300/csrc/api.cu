@@ -108,6 +108,9 @@ void free_ws(pf_plan* p) {
   p->st = DevState{};
 }
 
+// staging slot of a host batch: sbus, v0, v_out [chunk, n] complex; iters [chunk]; status [chunk]
+size_t slot_bytes_per_instance(int n) { return 3 * (size_t)n * 16 + 4 + 1; }
+
 int ensure_capacity(pf_plan* p, int B) {
   const int Bp = (B + kTile - 1) / kTile * kTile;
   if (Bp <= p->capacity) return NRPF_OK;
@@ -143,20 +146,6 @@ int ensure_capacity(pf_plan* p, int B) {
   // inverse pivots of the current diagonal block (interleaved dense block),
   // or U11^-1 and L11^-1 of the current 64 x 64 block (instance-major)
   AL(p->dp.dim ? (size_t)2 * 64 * 64 * Bp * sizeof(float) : (size_t)std::max(h.kb, 1) * Bp * w, inv, void*);
-  if (p->dp.n_fac_lvl > 0) {
-    AL((size_t)h.s * Bp * w, dinv, void*);
-  }
-  // Operands of the FP64 trailing update in fixed point (7 % of the workspace):
-  // where they would be the memory that is missing, the update stays in FP64
-  if (p->lu_precision == NRPF_LU_FP64 && h.kb == 8 && h.ndp > 16) {
-    void* d = nullptr;
-    if (cudaMalloc(&d, nrpf::dense_limb_bytes(p->dp, Bp)) == cudaSuccess) {
-      p->ws_allocs.push_back(d);
-      s.limb = d;
-    } else {
-      cudaGetLastError();
-    }
-  }
   AL((size_t)Bp * sizeof(unsigned long long), norm, unsigned long long*);
   AL((size_t)Bp * 4, iters, int32_t*);
   AL((size_t)Bp * 4, status, int32_t*);
@@ -165,17 +154,33 @@ int ensure_capacity(pf_plan* p, int B) {
   AL(sizeof(nrpf::SolveCtl), ctl, nrpf::SolveCtl*);
 #undef AL
   CK(cudaMemset(s.ctl, 0, sizeof(nrpf::SolveCtl)));
-  // Solves of up to kFewTiles factorise an interleaved FP32 block instance-major;
-  // without the memory for the inverses they keep to the layout
-  if (p->few_im) {
+  // Scratch that only makes solves faster, last and only out of memory to spare: as
+  // much has to stay free as the plan itself may ask for later (per-instance
+  // admittances, two staging slots of a host batch) and as a caller's inputs and
+  // outputs take.  Without it the columns, the FP64 multiply-adds and the
+  // interleaved FP32 kernels serve, with a launch per level or more passes over the block.
+  const size_t reserve = (size_t)Bp * (16 * (size_t)p->dp.nnzY + 3 * slot_bytes_per_instance(h.n)) + ((size_t)64 << 20);
+  auto spare = [&](size_t bytes) -> void* {
+    size_t free_now = 0, all = 0;
     void* d = nullptr;
-    const size_t n = (size_t)std::min(Bp, kFewTiles * kTile);
-    if (cudaMalloc(&d, n * 2 * 64 * 64 * sizeof(float)) != cudaSuccess) {
-      cudaGetLastError();
-    } else {
+    if (cudaMemGetInfo(&free_now, &all) == cudaSuccess && free_now >= bytes + reserve &&
+        cudaMalloc(&d, std::max<size_t>(bytes, 256)) == cudaSuccess) {
       p->ws_allocs.push_back(d);
-      if (nrpf::make_dense_im_maps(p->dp, s.lu, Bp, &p->im_maps)) p->few_inv = d;
+      return d;
     }
+    cudaGetLastError();
+    return nullptr;
+  };
+  // inverse pivots of the refactorisation by entries, of the batches that take it
+  if (p->dp.n_fac_lvl > 0)
+    s.dinv = spare((size_t)h.s * (w == 4 ? Bp : std::min(Bp, nrpf::kEntryTiles64 * kTile)) * w);
+  // operands of the FP64 trailing update in fixed point (7 % of the workspace)
+  if (p->lu_precision == NRPF_LU_FP64 && h.kb == 8 && h.ndp > 16) s.limb = spare(nrpf::dense_limb_bytes(p->dp, Bp));
+  // inverses for solves of up to kFewTiles that factorise an interleaved FP32 block
+  // instance-major
+  if (p->few_im) {
+    void* d = spare((size_t)std::min(Bp, kFewTiles * kTile) * 2 * 64 * 64 * sizeof(float));
+    if (d && nrpf::make_dense_im_maps(p->dp, s.lu, Bp, &p->im_maps)) p->few_inv = d;
   }
   if (p->dp.dim && h.ndp > 0) {
     // TMA descriptors of this workspace's dense blocks
@@ -561,27 +566,29 @@ int pf_plan_create(int n, const int32_t* rowptr, const int32_t* colidx, const do
       return rc;
     }
     d.schur_task = reinterpret_cast<const int4*>(tasks);
+    // schedules that only make solves faster: without the memory for them the
+    // columns and the level kernels serve
     const int32_t* ops = nullptr;
-    if ((rc = upload(p, h.fac_lvl_ptr, &d.fac_lvl_ptr)) || (rc = upload(p, h.fac_task, &d.fac_task)) ||
-        (rc = upload(p, h.fac_op, &ops))) {
-      pf_plan_destroy(p);
-      return rc;
+    if (!(rc = upload(p, h.fac_lvl_ptr, &d.fac_lvl_ptr)) && !(rc = upload(p, h.fac_task, &d.fac_task)) &&
+        !(rc = upload(p, h.fac_op, &ops))) {
+      d.fac_op = reinterpret_cast<const int2*>(ops);
+      d.n_fac_lvl = std::max((int)h.fac_lvl_ptr.size() - 1, 0);
+      d.n_fac_task = std::max((int)h.fac_task.size() - 1, 0);
     }
-    d.fac_op = reinterpret_cast<const int2*>(ops);
-    d.n_fac_lvl = std::max((int)h.fac_lvl_ptr.size() - 1, 0);
-    d.n_fac_task = std::max((int)h.fac_task.size() - 1, 0);
     // the whole-solve schedule, where some batch takes it in this precision
-    if (nrpf::small_solve_fits(h, p->lu_precision == NRPF_LU_FP32 ? 4 : 8)) {
-      if ((rc = upload(p, h.sm_lvl_ptr, &d.sm_lvl_ptr)) || (rc = upload(p, h.sm_task, &d.sm_task)) ||
-          (rc = upload(p, h.sm_op, &ops))) {
-        pf_plan_destroy(p);
-        return rc;
-      }
+    if (!rc && nrpf::small_solve_fits(h, p->lu_precision == NRPF_LU_FP32 ? 4 : 8) &&
+        !(rc = upload(p, h.sm_lvl_ptr, &d.sm_lvl_ptr)) && !(rc = upload(p, h.sm_task, &d.sm_task)) &&
+        !(rc = upload(p, h.sm_op, &ops))) {
       d.sm_op = reinterpret_cast<const int2*>(ops);
       d.n_sm_lvl = (int)h.sm_lvl_ptr.size() - 1;
       d.n_sm_task = (int)h.sm_task.size() - 1;
       d.n_sm_op = (int)(h.sm_op.size() / 2);
     }
+    if (rc && rc != NRPF_ERR_NOMEM) {
+      pf_plan_destroy(p);
+      return rc;
+    }
+    if (rc) cudaGetLastError();
     d.n_schur = (int)(h.schur_task.size() / 4);
     d.clusters = nrpf::dense_cluster_resident(d, p->lu_precision == NRPF_LU_FP32 ? 4 : 8);
   }
@@ -790,9 +797,8 @@ int pf_solve_batch_host(pf_plan* p, int B, const double* sbus, const double* v0,
   const int n = p->hp.n;
   int rc = ensure_capacity(p, chunk);
   if (rc) return rc;
-  // staging slot layout: sbus, v0, v_out [chunk, n] complex; iters [chunk]; status [chunk]
   const size_t cplx = (size_t)n * 16;
-  auto slot_bytes = [&](int c) { return (size_t)c * (3 * cplx + 4 + 1) + 256; };
+  auto slot_bytes = [&](int c) { return (size_t)c * slot_bytes_per_instance(n) + 256; };
   if (chunk > p->stage_cap) {
     CK(cudaDeviceSynchronize());
     for (int i = 0; i < 2; ++i) {

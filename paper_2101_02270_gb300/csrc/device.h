@@ -113,7 +113,7 @@ struct DevState {
   void* x;       // [mp] right-hand side / solution (LU precision)
   void* lu;      // [NLU] LU values (LU precision)
   void* inv;     // [kb] inverse pivots of the current dense diagonal block
-  void* dinv;    // [s] inverse pivots of the sparse columns (LU precision)
+  void* dinv;    // [s] inverse pivots of the sparse columns (LU precision), or null
   void* limb;    // operands of the FP64 trailing update in fixed point (kernels.cu), or null
   unsigned long long* norm;  // [Bp] max |F| as float64 bits
   int32_t* iters;   // [Bp]

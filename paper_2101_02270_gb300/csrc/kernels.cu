@@ -1739,7 +1739,7 @@ template <typename T>
 void launch_factor(const DevPlan& P, const DevState& S, const std::vector<int32_t>& lvl_ptr,
                    const int32_t* gate, cudaStream_t st, Recorder* rec, bool dense) {
   const int tiles = S.Bp / kTile;
-  if (P.n_fac_lvl > 0 && (sizeof(T) == 4 || tiles <= 152))
+  if (P.n_fac_lvl > 0 && S.dinv && (sizeof(T) == 4 || tiles <= kEntryTiles64))
     launch_levels(k_sparse_factor<T>, K_LU_SPARSE, P, S, P.n_fac_task, P.n_fac_lvl, gate, st, rec);
   else for (size_t l = 0; l + 1 < lvl_ptr.size(); ++l) {
     int c0 = lvl_ptr[l], c1 = lvl_ptr[l + 1];

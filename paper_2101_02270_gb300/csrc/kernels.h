@@ -75,6 +75,9 @@ enum class LuPrep { kWhole, kSparse, kColumns };
 template <typename T>
 void launch_prepare_lu(const DevPlan& P, const DevState& S, const int32_t* gate, cudaStream_t st,
                        Recorder* rec = nullptr, LuPrep prep = LuPrep::kWhole);
+// Tiles up to which an FP64 refactorisation goes by entries (FP32: any number)
+constexpr int kEntryTiles64 = 152;
+
 // Bytes of S.limb, the fixed-point operands of the FP64 trailing update, for a
 // workspace of Bp instances.
 size_t dense_limb_bytes(const DevPlan& P, int Bp);
