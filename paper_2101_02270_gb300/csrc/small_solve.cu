@@ -14,9 +14,13 @@
 //
 // When: batches whose CTAs, one per SM, are one wave, and plans and precisions for
 // which this then is the faster form.  A second wave takes as long as the first, where
-// the level kernels' time grows by a quarter.  Solves by the level kernels / by this
-// kernel, us (buses, values, dense columns: instances):
+// the level kernels' time grows by a quarter; only FP64 plans of few values and many
+// levels are the faster ones still in the second: 45 to 50 buses x 3,200, level kernels /
+// this kernel, us: 1,001 values, 19 levels 1,069 / 911; 1,092, 25: 1,242 / 1,101; but 1,049,
+// 12: 866 / 922; 940, 12: 923 / 925.  Solves by the level kernels / by this kernel, us
+// (buses, values, dense columns: instances):
 //   FP64  30, 675, 12:     64: 695 / 391   1,216: 810 / 401     2,432: 851 / 458
+//   FP64  40, 918, 12:     4,864: 1,143 / 1,066 (two waves)   8,000: 1,486 / 1,982
 //   FP64  100, 2,424, 23:  64: 811 / 760   1,216: 1,054 / 856   2,432: 1,188 / 1,567   10,000: 2,843 / 6,742
 //   FP32  40, 1,062, 20:   64: 603 / 502   2,432: 708 / 579     10,000: 1,262 / 1,889
 //   FP32  55, 1,576, 25:   64: 483 / 632   1,216: 544 / 670     10,000: 1,215 / 2,451
@@ -46,7 +50,9 @@ namespace {
 constexpr size_t kSmallSmem = 200 * 1024;
 constexpr size_t kSmallValuesFp32 = 1200;
 constexpr int kSmallDenseFp32 = 20;
-// values up to which a plan keeps to the kernel beyond one wave
+// values per level of the sparse LU up to which a plan keeps to the kernel in a second
+// wave, and values up to which it always does
+constexpr size_t kSmallPerLevel64 = 60;
 constexpr size_t kSmallAlways64 = 700, kSmallAlways32 = 800;
 constexpr int kSmallThreads = 512;
 
@@ -185,9 +191,14 @@ bool small_solve_fits(const HostPlan& h, size_t width) {
 int small_solve_instances(const DevPlan& P, int Bp, size_t width) {
   if (P.n_sm_lvl == 0) return 0;
   const size_t nval = (size_t)(P.NS + (int64_t)P.nd * P.nd) + 2 * (size_t)P.m;
-  for (int s = 8; s <= 32 && nval * s * width <= kSmallSmem; s *= 2)
+  int s = 4;
+  while (s < 32 && nval * 2 * s * width <= kSmallSmem) {
+    s *= 2;
     if (Bp / s <= P.sms) return s;
-  return nval <= (width == 8 ? kSmallAlways64 : kSmallAlways32) ? 32 : 0;
+  }
+  // s: the most that fit
+  if (width == 8 && nval <= kSmallPerLevel64 * P.n_lu_lvl && Bp / s <= 2 * P.sms) return s;
+  return nval <= (width == 8 ? kSmallAlways64 : kSmallAlways32) ? s : 0;
 }
 
 template <typename T>

@@ -587,12 +587,13 @@ def test_more_batch_sizes_than_loop_graphs():
 
 @pytest.mark.parametrize("n,branches,lu,waves", [(55, 75, "fp64", 16), (85, 116, "fp64", 8), (40, 50, "fp32", 32),
                                                  (55, 69, "fp32", 0), (120, 164, "fp32", 0), (30, 41, "fp64", None),
-                                                 (30, 41, "fp32", None)])
+                                                 (30, 41, "fp32", None), (50, 63, "fp64", 32)])
 def test_small_plans_leave_their_kernel_beyond_one_wave(n, branches, lu, waves):
-    """A batch of more CTAs of the small plans' kernel, of at most `waves` instances
-    (as many as fit), than the GPU has SMs goes to the level kernels, larger FP32
-    plans always, the smallest plans never.  Voltages on either side of the line are
-    those of the same scenarios within a few units of rounding."""
+    """A batch of more than `waves` instances per SM (as many as fit a CTA, or two CTAs'
+    where a plan has few values and many levels) goes from the small plans' kernel to
+    the level kernels, larger FP32 plans always, the smallest plans never.  Voltages on
+    either side of the line are those of the same scenarios within a few units of
+    rounding."""
     import gridgen
     g = gridgen.make_grid("mesh30_b64" if n < 100 else "mesh2000_b10k", 0, n=n, n_branch=branches, n_pv=n // 10,
                           load_scale=1 / 16)
