@@ -60,11 +60,27 @@ __global__ void __launch_bounds__(kThreads) k_branch_flows(
   }
 }
 
-// Instances per group: up to 16, which makes the divisions a tenth of the
-// arithmetic; fewer while the blocks would not fill the GPU eight times over
-// (8 x 152 CTAs of 256 threads are all that is resident).
+// Instances per group, up to 16.  A thread's FP64 work is that of two divisions, 37
+// operations, and 18 per instance, and the SM with the most blocks ends last: the
+// group that makes this least, with at least three blocks per SM, which covers the
+// latency of the gathers, or single instances.
 constexpr int kPerGroup = 16;
-constexpr long long kFillBlocks = 8 * 152;
+constexpr long long kSms = 152;
+
+int instances_per_group(int B, int nbr) {
+  int best = 1;
+  long long least = 0;
+  for (int per = 1; per <= kPerGroup; ++per) {
+    const long long blocks = (((long long)B + per - 1) / per * nbr + kThreads - 1) / kThreads;
+    if (per > 1 && blocks < 3 * kSms) break;
+    const long long cost = (blocks + kSms - 1) / kSms * (37 + 18 * per);
+    if (per == 1 || cost < least) {
+      best = per;
+      least = cost;
+    }
+  }
+  return best;
+}
 
 }  // namespace
 
@@ -75,8 +91,7 @@ extern "C" int pf_branch_flows(int n, int nbr, const int32_t* f, const int32_t* 
   if ((long long)B * nbr == 0) return NRPF_OK;
   if (!f || !t || !r || !x || !b || !v || !sf || !st) return NRPF_ERR_ARG;
   if (((long long)B * nbr + kThreads - 1) / kThreads > 0x7fffffffLL) return NRPF_ERR_ARG;
-  const long long fit = (long long)B * nbr / (kThreads * kFillBlocks);
-  const int per = (int)(fit < 1 ? 1 : fit > kPerGroup ? kPerGroup : fit);
+  const int per = instances_per_group(B, nbr);
   const unsigned long long total = (unsigned long long)(((long long)B + per - 1) / per) * (unsigned)nbr;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   k_branch_flows<<<(unsigned)((total + kThreads - 1) / kThreads), kThreads, 0, s>>>(
