@@ -787,8 +787,9 @@ def update_roofline(lu, im, info, refactors, du, fp64_peak, fp32_peak, hbm, hbm_
         roof = {"bound": "alu", "kernel": "dense_update (k_im_gemm_tc, six BF16 tensor-core products per FP32 one, "
                                           "far from the solution; k_im_gemm, FP32 FMA, near it)",
                 "achieved": achieved,
-                "peak": fp32_peak, "unit": "TFLOP/s", "frac": (achieved / fp32_peak) if achieved else None,
-                "traffic": None,
+                "peak": fp32_peak, "unit": "TFLOP/s",
+                # no fraction: the far updates run on another pipe than the peak's
+                "frac": None, "over_fma_peak": (achieved / fp32_peak) if achieved else None, "traffic": None,
                 "peak_kind": "measured FP32 FMA-chain throughput (pf_fma_peak); the tensor-core form does not use it",
                 "launches": du[0], "ms_total": du[2], "timing": timing,
                 "algorithmic_bytes": "per launch and instance: the panel's block column and row read and "
@@ -796,10 +797,12 @@ def update_roofline(lu, im, info, refactors, du, fp64_peak, fp32_peak, hbm, hbm_
     elif lu == "fp64":
         du_flop = dense_update_flop(ndp, kb) * refactors
         achieved = du_flop / (du[2] / 1e3) / 1e12 if du[2] > 0 else None
+        ratio = (achieved / fp64_peak) if achieved else None
         roof = {"bound": "alu", "kernel": "dense_update (k_dense_update_fixed, integer multiply-adds in fixed point, "
                                           "panel 8; k_dense_update, FP64 FMA, otherwise)",
                 "achieved": achieved, "peak": fp64_peak,
-                "unit": "TFLOP/s", "frac": (achieved / fp64_peak) if achieved else None, "traffic": None,
+                # no fraction in fixed point: most of its work is on another pipe than the peak's
+                "unit": "TFLOP/s", "frac": None if kb == 8 else ratio, "over_fma_peak": ratio, "traffic": None,
                 "peak_kind": "measured FP64 FMA-chain throughput (pf_fma_peak); the fixed-point form does not use it",
                 "launches": du[0], "ms_total": du[2], "timing": timing}
     else:
