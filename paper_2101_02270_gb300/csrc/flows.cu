@@ -22,7 +22,7 @@ namespace {
 // each, it took 1.73 ms; 1,000 buses x 10,000 0.91, now 0.48.  A block of 256
 // threads along the branches, of which only 41 exist on a 30-bus grid, took 22.6 us
 // on 5,000 instances of it and 36.3 on 10,000; a thread per branch and instance 19.9
-// and 33.5, this form 19.8 and 33.5.
+// and 33.5, this form 19.8 and 24.8.
 constexpr int kThreads = 256;
 
 __global__ void __launch_bounds__(kThreads) k_branch_flows(
